@@ -48,7 +48,7 @@ constexpr int kThinPerCell = PICRR_THIN_PER_CELL;
 // (in the 2^lscale units of the records) as two 32-bit words, lo (unsigned)
 // and hi (signed): value = hi * 2^32 + lo.  A signed 32-bit term t is added
 // with a 32-bit atomic on lo, which returns the old word: the addition
-// wrapped (carried) iff the new word is below the old one, and hi then gets
+// wrapped (carried) iff old + t carries out of 32 bits, and hi then gets
 // sign(t) + carry (-1, 0 or +1; nothing in most cases).  Every carry is seen by
 // exactly one adder, so the pair always holds the exact sum, in any order.
 // (A 64-bit shared-memory atomic runs at a sixth of the 32-bit rate.)
@@ -57,10 +57,27 @@ struct Window {
     int hi[3][WMAX];
 };
 
-__device__ __forceinline__ void win_add(Window& w, int comp, int at, int t) {
-    const unsigned old = atomicAdd(&w.lo[comp][at], static_cast<unsigned>(t));
-    const int h = (t < 0 ? -1 : 0) + (old + static_cast<unsigned>(t) < old ? 1 : 0);
-    if (h) atomicAdd(&w.hi[comp][at], h);
+__device__ __forceinline__ uint32_t win_addr(const Window& w) { return smem_u32(&w.lo[0][0]); }
+
+// Adds t to the window word at shared address `addr` + OFF.  Predicated
+// throughout: a branch per nonzero test made every add two divergence points
+// (the dense run of hot particles 0.717 ms with this, 0.759 ms with branches;
+// thin plasma 106 and 111 us).  Two additions without return (t to lo, t >> 12
+// to a coarse word that resolves the wraps) took thin plasma to 104 us but the
+// dense run to 0.755 ms.
+template <int OFF>
+__device__ __forceinline__ void win_add(uint32_t addr, int t) {
+    asm volatile(
+        "{\n\t.reg .pred p, q;\n\t.reg .u32 o, s, h;\n\t"
+        "setp.ne.s32 p, %1, 0;\n\t"
+        "mov.u32 o, 0;\n\t"
+        "@p atom.shared.add.u32 o, [%0 + %2], %1;\n\t"
+        "add.cc.u32 s, o, %1;\n\t"
+        "shr.s32 h, %1, 31;\n\t"
+        "addc.u32 h, h, 0;\n\t"
+        "setp.ne.s32 q, h, 0;\n\t"
+        "@q red.shared.add.u32 [%0 + %3], h;\n\t}" ::"r"(addr), "r"(t), "n"(OFF), "n"(OFF + 3 * WMAX * 4)
+        : "memory");
 }
 
 // Position of value q of a stencil record anchored at key: q 0..2 are Jy at
@@ -68,14 +85,18 @@ __device__ __forceinline__ void win_add(Window& w, int comp, int at, int t) {
 __device__ __forceinline__ int rec_comp(int q) { return q < 3 ? 1 : (q < 6 ? 2 : 0); }
 __device__ __forceinline__ int rec_at(int key, int q) { return key + (q < 3 ? q : (q < 6 ? q - 3 : q - 6)); }
 
-// One lane's record added by itself: each nonzero value rounded to 32-bit
-// fixed point (records are kept in the window's units, |value| < 2^26).
-__device__ __forceinline__ void lane_add(int key, const float (&v)[8], Window& w) {
-#pragma unroll
-    for (int q = 0; q < 8; ++q) {
-        const int t = __float2int_rn(v[q]);
-        if (t) win_add(w, rec_comp(q), rec_at(key, q), t);
-    }
+// One lane's record added by itself: each value rounded to 32-bit fixed point
+// (records are kept in the window's units, |value| < 2^26).
+__device__ __forceinline__ void lane_add(int key, const float (&v)[8], uint32_t w) {
+    const uint32_t a = w + 4u * key;
+    win_add<4 * (WMAX + 0)>(a, __float2int_rn(v[0]));
+    win_add<4 * (WMAX + 1)>(a, __float2int_rn(v[1]));
+    win_add<4 * (WMAX + 2)>(a, __float2int_rn(v[2]));
+    win_add<4 * (2 * WMAX + 0)>(a, __float2int_rn(v[3]));
+    win_add<4 * (2 * WMAX + 1)>(a, __float2int_rn(v[4]));
+    win_add<4 * (2 * WMAX + 2)>(a, __float2int_rn(v[5]));
+    win_add<0>(a, __float2int_rn(v[6]));
+    win_add<4>(a, __float2int_rn(v[7]));
 }
 
 // One stencil record per lane (key < 0: none).  When every lane holds the
@@ -86,7 +107,7 @@ __device__ __forceinline__ void lane_add(int key, const float (&v)[8], Window& w
 // its own record.  (A reduction over lanes grouped by anchor runs once per
 // distinct anchor, which costs more than the lanes' own atomics as soon as
 // the warp holds two.)
-__device__ __forceinline__ void warp_add(int key, const float (&v)[8], Window& w) {
+__device__ __forceinline__ void warp_add(int key, const float (&v)[8], uint32_t w) {
     const int k0 = __shfl_sync(FULL, key, 0);
     if (__all_sync(FULL, key == k0)) {
         if (k0 >= 0) {
@@ -98,29 +119,12 @@ __device__ __forceinline__ void warp_add(int key, const float (&v)[8], Window& w
                 const int t = __reduce_add_sync(FULL, __float2int_rn(v[q]));
                 mine = lane == q ? t : mine;
             }
-            if (lane < 8 && mine) win_add(w, rec_comp(lane), rec_at(k0, lane), mine);
+            if (lane < 8) win_add<0>(w + 4u * (rec_comp(lane) * WMAX + rec_at(k0, lane)), mine);
         }
     } else {
-        // lanes 2m and 2m+1 that hold the same anchor: the even lane adds the
-        // pair's integer sum (exact: |sum| < 2^27), the odd lane nothing, which
-        // halves the same-word atomics of lanes that share an anchor (the
-        // 256-run scan's late-phase push 0.542 -> 0.530 ms); the window's sums
-        // are the same integers
-        const int lane = threadIdx.x & 31;
-        const int kn = __shfl_xor_sync(FULL, key, 1);
-        const bool pair = key >= 0 && kn == key;
-        int t[8];
-#pragma unroll
-        for (int q = 0; q < 8; ++q) {
-            const int tq = __float2int_rn(v[q]);
-            const int tn = __shfl_xor_sync(FULL, tq, 1);
-            t[q] = pair ? tq + tn : tq;
-        }
-        if (key >= 0 && !(pair && (lane & 1))) {
-#pragma unroll
-            for (int q = 0; q < 8; ++q)
-                if (t[q]) win_add(w, rec_comp(q), rec_at(key, q), t[q]);
-        }
+        // (summing the records of neighbouring lanes with one anchor first saves
+        // atomics but not time: scan 116 us either way)
+        if (key >= 0) lane_add(key, v, w);
     }
 }
 
@@ -203,6 +207,7 @@ __global__ void __launch_bounds__(PUSH_T, Slot<W>::MIN_BLOCKS) k_push_deposit(co
     using F = typename Slot<W>::F;
     __shared__ __align__(128) PushSmem<W> sm;
     Window& sJ = sm.J;  // the unit's current: Jx (half nodes), Jy, Jz (nodes) of the window
+    const uint32_t wJ = win_addr(sJ);
     __shared__ __align__(8) uint64_t bar;
     __shared__ double sred[PUSH_T / 32];
 
@@ -456,25 +461,15 @@ __global__ void __launch_bounds__(PUSH_T, Slot<W>::MIN_BLOCKS) k_push_deposit(co
                 f = fn;
             }
             // merge the particle's record into this thread's running record; when
-            // its anchor changes, the finished record is added: by the lane itself in
-            // thin units and with 2 particles per thread (no warp vote per particle,
-            // which lets the two particles' arithmetic overlap: 3-4 % faster on thin
-            // plasma), through warp_add otherwise (4 per thread: the per-lane path
-            // costs registers there, and dense foils rarely change anchor mid-round)
+            // its anchor changes, the lane adds the finished record by itself: a warp
+            // vote and a warp-wide sum at every change cost more, with 4 particles
+            // per thread too (hot particles on a dense foil, whose anchors change
+            // mid-round: 0.717 -> 0.633 ms)
             const bool merge = ka < 0 || rk < 0 || ka == rk;
-            if (thin || W == 2) {
-                if (!merge) {
-                    lane_add(rk, rv, sJ);
+            if (!merge) {
+                lane_add(rk, rv, wJ);
 #pragma unroll
-                    for (int q = 0; q < 8; ++q) rv[q] = 0.f;
-                }
-            } else if (__any_sync(FULL, !merge)) {
-                warp_add(merge ? -1 : rk, rv, sJ);
-                if (!merge) {
-                    rk = -1;
-#pragma unroll
-                    for (int q = 0; q < 8; ++q) rv[q] = 0.f;
-                }
+                for (int q = 0; q < 8; ++q) rv[q] = 0.f;
             }
             if (ka >= 0) {  // the record's eight values, added to the running record
                 rk = ka;
@@ -495,9 +490,9 @@ __global__ void __launch_bounds__(PUSH_T, Slot<W>::MIN_BLOCKS) k_push_deposit(co
             qz[j] = pz;
         }
         if (thin) {
-            if (rk >= 0) lane_add(rk, rv, sJ);
+            if (rk >= 0) lane_add(rk, rv, wJ);
         } else {
-            warp_add(rk, rv, sJ);
+            warp_add(rk, rv, wJ);
         }
         rk = -1;
 #pragma unroll
