@@ -34,26 +34,6 @@ __global__ void k_noalloc_clear(unsigned long long* bins, int n) {
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) bins[i] = 0ull;
 }
 
-__global__ void __launch_bounds__(256) k_noalloc_count(const float* px, const float* py, const float* pz,
-                                                       int64_t n, double mass_mev, int nbins, double e_min,
-                                                       double e_max, unsigned long long* bins) {
-    for (int64_t i = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x; i < n;
-         i += static_cast<int64_t>(gridDim.x) * blockDim.x) {
-        const double x = px[i], y = py[i], z = pz[i];
-        const double p2 = x * x + y * y + z * z;
-        const double e = mass_mev * p2 / (sqrt(1.0 + p2) + 1.0);
-        int k;
-        if (e < e_min) {
-            k = nbins;
-        } else {
-            const double kf = floor((e - e_min) / (e_max - e_min) * static_cast<double>(nbins));
-            // written so that a NaN energy (never produced by a checked state) lands in the overflow
-            k = kf < static_cast<double>(nbins) ? static_cast<int>(kf) : nbins + 1;
-        }
-        atomicAdd(&bins[k], 1ull);
-    }
-}
-
 __global__ void k_noalloc_finish(const unsigned long long* bins, int nbins, double scale, double* counts) {
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < nbins; i += gridDim.x * blockDim.x)
         counts[i] = static_cast<double>(bins[i]) * scale;
@@ -110,10 +90,7 @@ extern "C" pic_status pic_spectrum_noalloc(const float* px, const float* py, con
     const int nb2 = nbins + 2;
     k_noalloc_clear<<<(nb2 + 255) / 256, 256, 0, st>>>(bins, nb2);
     if (n > 0) {
-        int64_t g = (n + 255) / 256;
-        if (g > 1216) g = 1216;
-        k_noalloc_count<<<static_cast<int>(g), 256, 0, st>>>(px, py, pz, n, mass_me * 0.51099895000, nbins,
-                                                             e_min_MeV, e_max_MeV, bins);
+        launch_spectrum(px, py, pz, n, mass_me * 0.51099895000, nbins, e_min_MeV, e_max_MeV, bins, st);
     }
     const double width = (e_max_MeV - e_min_MeV) / nbins;
     k_noalloc_finish<<<(nbins + 255) / 256, 256, 0, st>>>(bins, nbins, weight_dx / width, counts);

@@ -1394,8 +1394,8 @@ pic_status run_spectra(Batch* b, int id, int species, int nbins, double e_min, d
             b->bins_cap = nbins + 2;
         }
         PIC_CK(b, cudaMemsetAsync(b->bins, 0, sizeof(unsigned long long) * (nbins + 2), b->stream));
-        launch_spectrum(r.dev.sp[species][run_pbuf(b, r)], h.n, h.m * kMec2MeV, nbins, e_min, e_max, b->bins,
-                        b->stream);
+        const DevSpecies& sp = r.dev.sp[species][run_pbuf(b, r)];
+        launch_spectrum(sp.px, sp.py, sp.pz, h.n, h.m * kMec2MeV, nbins, e_min, e_max, b->bins, b->stream);
         b->launches++;
         PIC_CK(b, cudaMemcpyAsync(hb.data(), b->bins, sizeof(unsigned long long) * (nbins + 2),
                                   cudaMemcpyDeviceToHost, b->stream));

@@ -236,8 +236,9 @@ struct DiagParams {
 int launch_field_energy(const DiagParams& D, double* partials, int max_blocks, cudaStream_t st);
 int launch_kinetic(DevSpecies sp, int64_t n, double* partials, int max_blocks, cudaStream_t st);
 void launch_reduce_partials(const double* partials, int n, double scale, double* out, cudaStream_t st);
-void launch_spectrum(DevSpecies sp, int64_t n, double mass_mev, int nbins, double e_min, double e_max,
-                     unsigned long long* bins, cudaStream_t st);
+// bins[0..nbins) counts, bins[nbins] underflow, bins[nbins+1] overflow, added to what is there.
+void launch_spectrum(const float* px, const float* py, const float* pz, int64_t n, double mass_mev, int nbins,
+                     double e_min, double e_max, unsigned long long* bins, cudaStream_t st);
 
 // Friction coefficient d (Eq. damping) and quantum parameter chi per particle
 // from the stored momentum and the fields at the particle.  d_out / chi_out
