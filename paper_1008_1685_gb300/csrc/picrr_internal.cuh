@@ -251,8 +251,6 @@ struct SnapParams {
 void launch_wait_selftest(int* status, cudaStream_t st);
 void launch_validate(const int32_t* cell, const float* off, const float* px, const float* py, const float* pz,
                      int64_t n, int Nx, unsigned long long* out, cudaStream_t st);
-void launch_electron_scan(const pic_electron_case* cases, int64_t n, int integrator, int flags, double dt,
-                          int64_t nsteps, int every, double eps, double* out, int64_t nsamples, cudaStream_t st);
 
 void launch_snapshot(DevSpecies sp, int64_t n, const SnapParams& S, float* d_out, float* chi_out,
                      unsigned long long* out, cudaStream_t st);
