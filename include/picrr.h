@@ -188,7 +188,7 @@ typedef struct {
     int64_t sort_count;       /* cell sorts performed */
     int64_t active_particles; /* particles of the runs still stepping, both species (frozen ones included) */
     double push_ms;           /* summed device time of the push kernel (timing on) */
-    double field_ms;          /* summed device time of the Yee kernel (timing on) */
+    double field_ms;          /* summed device time of the Yee kernel's own launches (timing on) */
     double sort_ms;           /* summed device time of the sort kernels (timing on) */
     int64_t timed_push_launches; /* push launches covered by push_ms */
     int64_t device_bytes;     /* device memory held by the handle */
@@ -228,7 +228,10 @@ pic_status pic_tune_shapes(pic_sim* sim, int64_t steps_per_candidate, int* unit_
                            int* particles_per_thread, double* ms_per_step);
 
 /* Counters and, when timing is on, CUDA-event times of each kernel class,
- * recorded on the launching stream.  Every whole sort interval of steps that
+ * recorded on the launching stream.  While few particles are stepped with 2 per
+ * thread, the push launch of a step also does the Yee update of the step before
+ * (it counts and is timed as a push); the last step of a call or interval has
+ * a Yee launch of its own.  Every whole sort interval of steps that
  * no run ends inside is launched as one captured CUDA graph (its pushes, Yee
  * updates and the sort); with timing on, that graph also holds an event-record
  * node before and after each push, Yee update and sort, and the other steps

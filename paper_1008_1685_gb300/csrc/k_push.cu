@@ -28,7 +28,7 @@
 // to global memory with integer atomics.  Integer addition is exact and
 // associative, so the result does not depend on the order in which lanes,
 // warps or CTAs arrive.
-#include "picrr_internal.cuh"
+#include "yee.cuh"
 
 namespace picrr {
 
@@ -107,9 +107,9 @@ __device__ __forceinline__ void lane_add(int key, const float (&v)[8], uint32_t 
 // its own record.  (A reduction over lanes grouped by anchor runs once per
 // distinct anchor, which costs more than the lanes' own atomics as soon as
 // the warp holds two.)
-__device__ __forceinline__ void warp_add(int key, const float (&v)[8], uint32_t w) {
+__device__ __forceinline__ void warp_add(int key, const float (&v)[8], uint32_t w, bool vote) {
     const int k0 = __shfl_sync(FULL, key, 0);
-    if (__all_sync(FULL, key == k0)) {
+    if (vote && __all_sync(FULL, key == k0)) {
         if (k0 >= 0) {
             // lane q (q < 8) adds the warp sum of value q: eight distinct words
             const int lane = threadIdx.x & 31;
@@ -197,27 +197,88 @@ struct PushSmem<4> {
 };
 template <>
 struct PushSmem<2> {
-    float F[5][WMAX];
+    float F[5][WMAX + 8];  // element 4 is the window's first: room for the halo of the fused update
     Window J;
 };
 
-template <int W>
-__global__ void __launch_bounds__(PUSH_T, Slot<W>::MIN_BLOCKS) k_push_deposit(const PushParams P) {
+// The Yee update of the fields in F (old, from the element `p0` - 4 of the padded grid on) to the step after,
+// for the window's L elements, by all threads of the block; the same arithmetic as field_block.
+__device__ __forceinline__ void window_yee(const FieldParams& Q, const RunDev& R, int run, unsigned phase, int p0, int L,
+                                           float (&F)[5][WMAX + 8], float (&mur)[8]) {
+    const int tid = threadIdx.x, Nx = R.Nx, is = R.is;
+    const unsigned long long* const* J = R.J[current_set(R, phase, Q.nsets)];
+    const float* inc = Q.inc + 6 * run;
+    const float c = Q.c, hc = Q.hc, fdt = Q.fdt, fpi = R.fp_inv, fph = R.fp_inv * 4294967296.0f;
+    const int n0 = p0 - PADF;  // node / half node of the window's element 0 (F[.][4])
+    const bool left = n0 <= 0, right = n0 + L >= Nx;  // block-uniform: a wall's node is among elements 0..L
+    if (tid < 2 && left) {  // old E of the walls and their neighbours, before they are overwritten
+        mur[tid] = F[1 + tid][4 - n0];
+        mur[2 + tid] = F[1 + tid][5 - n0];
+    }
+    if (tid < 2 && right) {
+        mur[4 + tid] = F[1 + tid][4 + Nx - n0];
+        mur[6 + tid] = F[1 + tid][3 + Nx - n0];
+    }
+    for (int i = tid + 3; i < L + 5; i += PUSH_T)  // B^{n+1/2} on elements -1..L
+        yee_b(F[3][i], F[4][i], F[1][i], F[1][i + 1], F[2][i], F[2][i + 1], hc, n0 + i - 4 == is - 1, inc[0], inc[1]);
+    __syncthreads();
+    for (int i = tid + 4; i < L + 5; i += PUSH_T) {  // E^{n+1} on elements 0..L
+        const int node = n0 + i - 4, p = p0 + i - 4;
+        float ey = F[1][i], ez = F[2][i];
+        yee_e(ey, ez, F[3][i - 1], F[3][i], F[4][i - 1], F[4][i], fix_to_float(__ldg(J[1] + p), fpi, fph),
+              fix_to_float(__ldg(J[2] + p), fpi, fph), c, fdt, node == is, inc[2], inc[3]);
+        const bool inner = node >= 1 && node <= Nx - 1;
+        F[1][i] = inner ? ey : 0.f;
+        F[2][i] = inner ? ez : 0.f;
+    }
+    __syncthreads();
+    if (left || right) {  // block-uniform
+        const float km = (c - 1.f) / (c + 1.f);
+        if (tid < 2) {
+            float* E = F[1 + tid];
+            if (left) E[4 - n0] = yee_mur(mur[2 + tid], E[5 - n0], mur[tid], km);
+            if (right) E[4 + Nx - n0] = yee_mur(mur[6 + tid], E[3 + Nx - n0], mur[4 + tid], km);
+        }
+        __syncthreads();
+    }
+    for (int i = tid + 4; i < L + 4; i += PUSH_T) {  // B^{n+1} and Ex^{n+1} on elements 0..L-1
+        const int node = n0 + i - 4;
+        float by = F[3][i], bz = F[4][i];
+        yee_b(by, bz, F[1][i], F[1][i + 1], F[2][i], F[2][i + 1], hc, node == is - 1, inc[4], inc[5]);
+        const bool in = node >= 0 && node < Nx;
+        F[3][i] = in ? by : 0.f;
+        F[4][i] = in ? bz : 0.f;
+        F[0][i] = in ? fmaf(-fdt, fix_to_float(__ldg(J[0] + p0 + i - 4), fpi, fph), F[0][i]) : 0.f;
+    }
+}
+
+template <int W, bool FUSED>
+__global__ void __launch_bounds__(PUSH_T, Slot<W>::MIN_BLOCKS) k_push_deposit(const PushParams P, const FieldParams Q) {
     using I = typename Slot<W>::I;
     using F = typename Slot<W>::F;
     __shared__ __align__(128) PushSmem<W> sm;
+    const unsigned phase = *P.phase + P.k;
+    [[maybe_unused]] const unsigned before = phase + 5u;  // of the step before
+    if constexpr (FUSED) {
+        static_assert(W == 2 && sizeof(FieldSmem) <= sizeof(PushSmem<2>), "");
+        if (static_cast<int>(blockIdx.x) < Q.nblk) {
+            field_block<PUSH_T>(Q, before, blockIdx.x, reinterpret_cast<FieldSmem&>(sm));
+            return;
+        }
+    }
     Window& sJ = sm.J;  // the unit's current: Jx (half nodes), Jy, Jz (nodes) of the window
     const uint32_t wJ = win_addr(sJ);
     __shared__ __align__(8) uint64_t bar;
     __shared__ double sred[PUSH_T / 32];
 
-    const int u = blockIdx.x;
+    const int u = FUSED ? blockIdx.x - Q.nblk : blockIdx.x;
     if (u >= P.units.count[0]) return;  // block-uniform
-    const RunDev& R = P.runs[P.units.run[u]];
+    const int run = P.units.run[u];
+    const RunDev& R = P.runs[run];
     if (!R.active) return;
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int tid = threadIdx.x, lane = tid & 31;
     const int s = P.units.species[u];
-    const int par = static_cast<int>((P.gstep + R.fpar) & 1);
+    const int par = field_buf(R, FUSED ? before : phase);  // fused: the fields of the step before
     const int start = P.units.start[u], end = P.units.end[u];
     const int lo = P.units.lo[u], hi = P.units.hi[u];
     const int k = P.k;
@@ -233,6 +294,12 @@ __global__ void __launch_bounds__(PUSH_T, Slot<W>::MIN_BLOCKS) k_push_deposit(co
         return;
     }
 
+    // the unit's particles are read in slots of W, from the aligned slot before
+    // `start` to the aligned slot after `end`; the at most W - 1 particles of
+    // each neighbouring unit in those slots are never written here
+    const int base = start & ~(W - 1);
+    const int nslots = (((end + W - 1) & ~(W - 1)) - base) / W;
+
     for (int i = tid; i < 3 * WMAX; i += PUSH_T) {
         (&sJ.lo[0][0])[i] = 0u;
         (&sJ.hi[0][0])[i] = 0;
@@ -244,17 +311,14 @@ __global__ void __launch_bounds__(PUSH_T, Slot<W>::MIN_BLOCKS) k_push_deposit(co
     }
     __syncthreads();
     const DevSpecies sp = R.sp[s][P.cur];
-    // the unit's particles are read in slots of W, from the aligned slot before
-    // `start` to the aligned slot after `end`; the at most W - 1 particles of
-    // each neighbouring unit in those slots are never written here
-    const int base = start & ~(W - 1);
-    const int npw = ((end + W - 1) & ~(W - 1)) - base;
     if constexpr (W == 2) {
         if (tid == 0) {
-            mbar_arrive_expect_tx(&bar, 5u * static_cast<uint32_t>(L) * 4u);
+            // fused: with a halo of 4 elements (16 bytes) on each side, which lies inside the padded array
+            constexpr int H = FUSED ? 4 : 0;
+            const uint32_t bytes = static_cast<uint32_t>(L + 2 * H) * 4u;
+            mbar_arrive_expect_tx(&bar, 5u * bytes);
 #pragma unroll
-            for (int c = 0; c < 5; ++c)
-                tma_load_1d(&sm.F[c][0], R.F[par][c] + p0, static_cast<uint32_t>(L) * 4u, &bar);
+            for (int c = 0; c < 5; ++c) tma_load_1d(&sm.F[c][4 - H], R.F[par][c] + p0 - H, bytes, &bar);
         }
     } else {
         const float* const* Fg = R.F[par];
@@ -279,7 +343,6 @@ __global__ void __launch_bounds__(PUSH_T, Slot<W>::MIN_BLOCKS) k_push_deposit(co
     // are summed in its units (an exact scaling: the same bits as scaling each sum)
     const float jxf = qw / cfl * lscale;  // q w dx / dt
     const float hqw = 0.5f * qw * lscale;
-    const int nslots = npw / W;
     const int rounds = (nslots + PUSH_T - 1) / PUSH_T;
 
     if constexpr (W == 2) {
@@ -291,12 +354,17 @@ __global__ void __launch_bounds__(PUSH_T, Slot<W>::MIN_BLOCKS) k_push_deposit(co
             }
             return;
         }
+        if constexpr (FUSED) {
+            __shared__ float mur[8];
+            window_yee(Q, R, run, before, p0, L, sm.F, mur);
+            __syncthreads();
+        }
     } else {
         __syncthreads();
     }
 
     const bool thin = end - start < kThinPerCell * (hi - lo + 1);  // block-uniform
-    float rad = 0.f;
+    float rad_h = 0.f, rad_l = 0.f;  // energy radiated by this thread's particles
     int rk = -1;  // running stencil record of this thread (anchor rk)
     float rv[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
 
@@ -363,12 +431,13 @@ __global__ void __launch_bounds__(PUSH_T, Slot<W>::MIN_BLOCKS) k_push_deposit(co
                     b_y = fmaf(g, hf.w, hf.z);
                     b_z = fmaf(g, hz.y, hz.x);
                 } else {
-                    const float(*sF)[WMAX] = sm.F;
-                    e_y = (1.f - f) * sF[1][lb] + f * sF[1][lb + 1];
-                    e_z = (1.f - f) * sF[2][lb] + f * sF[2][lb + 1];
-                    e_x = (1.f - g) * sF[0][jb] + g * sF[0][jb + 1];
-                    b_y = (1.f - g) * sF[3][jb] + g * sF[3][jb + 1];
-                    b_z = (1.f - g) * sF[4][jb] + g * sF[4][jb + 1];
+                    const float *sn = &sm.F[0][4] + lb, *sh = &sm.F[0][4] + jb;
+                    constexpr int C = WMAX + 8;
+                    e_y = (1.f - f) * sn[C] + f * sn[C + 1];
+                    e_z = (1.f - f) * sn[2 * C] + f * sn[2 * C + 1];
+                    e_x = (1.f - g) * sh[0] + g * sh[1];
+                    b_y = (1.f - g) * sh[3 * C] + g * sh[3 * C + 1];
+                    b_z = (1.f - g) * sh[4 * C] + g * sh[4 * C + 1];
                 }
                 // --- Boris step for the Lorentz force (Bx = 0 in 1D)
                 const float mx = px + hq * e_x, my = py + hq * e_y, mz = pz + hq * e_z;
@@ -409,7 +478,12 @@ __global__ void __launch_bounds__(PUSH_T, Slot<W>::MIN_BLOCKS) k_push_deposit(co
                     const float qN = 1.f + px * px + py * py + pz * pz;
                     ign = rsqrt_ge1(qN);
                     const float gL = qL * rsqrt_ge1(qL), gN = qN * ign;
-                    rad -= div_ge1(kx * (lx + px) + ky * (ly + py) + kz * (lz + pz), gL + gN);
+                    // rad_h + rad_l -= de without the rounding (Knuth): the tally must not depend on the
+                    // units' size.  (One addition in double per round: thin plasma +3 %, the scan +4 %.)
+                    const float de = div_ge1(kx * (lx + px) + ky * (ly + py) + kz * (lz + pz), gL + gN);
+                    const float t = __fsub_rn(rad_h, de), z = __fsub_rn(t, rad_h);
+                    rad_l = __fadd_rn(rad_l, __fsub_rn(__fsub_rn(rad_h, __fsub_rn(t, z)), __fadd_rn(de, z)));
+                    rad_h = t;
                 } else {
                     px = lx;
                     py = ly;
@@ -489,11 +563,7 @@ __global__ void __launch_bounds__(PUSH_T, Slot<W>::MIN_BLOCKS) k_push_deposit(co
             qy[j] = py;
             qz[j] = pz;
         }
-        if (thin) {
-            if (rk >= 0) lane_add(rk, rv, wJ);
-        } else {
-            warp_add(rk, rv, wJ);
-        }
+        warp_add(rk, rv, wJ, !thin);
         rk = -1;
 #pragma unroll
         for (int q = 0; q < 8; ++q) rv[q] = 0.f;
@@ -530,37 +600,41 @@ __global__ void __launch_bounds__(PUSH_T, Slot<W>::MIN_BLOCKS) k_push_deposit(co
         }
     }
 
-
-
-    // radiated energy of the unit: fixed-order warp reduction, warps summed in double
+    // radiated energy: fixed-order sum over the CTA
+    if (rr) {
+        double v = static_cast<double>(rad_h) + static_cast<double>(rad_l);
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) rad += __shfl_xor_sync(FULL, rad, o);
-    if (lane == 0) sred[warp] = static_cast<double>(rad);
+        for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(FULL, v, o);
+        if (lane == 0) sred[tid >> 5] = v;
+    }
     __syncthreads();  // also orders every shared-memory current update before the flush
-    if (tid == 0) {
+    if (rr && tid == 0) {
         double t = 0.0;
         for (int w = 0; w < PUSH_T / 32; ++w) t += sred[w];
         P.rad_part[u] += t * static_cast<double>(R.rad_w[s]);  // summed into the tally at the next flush
     }
+    const int cset = current_set(R, phase, P.nsets);
     // flush the window: each exact sum shifted from record units to the
     // accumulators' 2^fp units (the run's fixed-point scale keeps it in range)
     for (int i = tid; i < L; i += PUSH_T) {
 #pragma unroll
         for (int c = 0; c < 3; ++c) {
             const long long v = static_cast<long long>((static_cast<unsigned long long>(static_cast<unsigned>(sJ.hi[c][i])) << 32) | sJ.lo[c][i]);
-            if (v) atomicAdd(R.J[par][c] + p0 + i, static_cast<unsigned long long>(v) << shift);
+            if (v) atomicAdd(R.J[cset][c] + p0 + i, static_cast<unsigned long long>(v) << shift);
         }
     }
 }
 
 }  // namespace
 
-void launch_push(const PushParams& P, int grid, int slot_w, cudaStream_t st) {
+void launch_push(const PushParams& P, const FieldParams& Q, bool fused, int grid, int slot_w, cudaStream_t st) {
     if (grid <= 0) return;
-    if (slot_w == 2)
-        k_push_deposit<2><<<grid, PUSH_T, 0, st>>>(P);
+    if (slot_w == 2 && fused)
+        k_push_deposit<2, true><<<Q.nblk + grid, PUSH_T, 0, st>>>(P, Q);
+    else if (slot_w == 2)
+        k_push_deposit<2, false><<<grid, PUSH_T, 0, st>>>(P, Q);
     else
-        k_push_deposit<4><<<grid, PUSH_T, 0, st>>>(P);
+        k_push_deposit<4, false><<<grid, PUSH_T, 0, st>>>(P, Q);
 }
 
 }  // namespace picrr

@@ -20,7 +20,9 @@
 //      split into chunks of at most unit_p particles, except that an aligned
 //      group of GROUP consecutive tiles holding at most unit_p particles
 //      together forms one unit, or else an aligned half group that does
-//      (sparse regions would otherwise give many nearly empty units).
+//      (sparse regions would otherwise give many nearly empty units); when the
+//      units are too few to fill the GPU, each is cut into parts of part_p
+//      particles, which are the table's entries.
 // Every particle is read once and written once; the cell array is read once
 // more for the counts.
 #include <algorithm>
@@ -356,13 +358,13 @@ __global__ void __launch_bounds__(SCAN_T) k_tile_units(const SortParams S) {
         const int hn = ks[min(h0 + SPAN / 2, R.Nx)] - ks[h0];
         int n;
         if (gn <= S.unit_p) {
-            n = (t % GROUP == 0 && gn > 0) ? 1 : 0;
+            n = t % GROUP == 0 ? gn : 0;
         } else if (hn <= S.unit_p) {
-            n = (t % (GROUP / 2) == 0 && hn > 0) ? 1 : 0;
+            n = t % (GROUP / 2) == 0 ? hn : 0;
         } else {
-            const int ts = ks[t * TILE], te = ks[min((t + 1) * TILE, R.Nx)];
-            n = (te - ts + S.unit_p - 1) / S.unit_p;
+            n = ks[min((t + 1) * TILE, R.Nx)] - ks[t * TILE];
         }
+        n = (n + S.part_p - 1) / S.part_p;  // (unit_p is a multiple of part_p)
         R.tile_n[s][t] = n;
     }
     __syncthreads();
@@ -378,7 +380,10 @@ __global__ void __launch_bounds__(SCAN_T) k_unit_bases(const SortParams S) {
     __shared__ int sh[SCAN_T / 32];
     const int np = 2 * S.nruns;
     const int total = block_scan_ranges(S.rs_units, S.rs_units + np, np, sh);
-    if (threadIdx.x == 0) S.units.count[0] = min(total, S.max_units);
+    if (threadIdx.x == 0) {
+        S.units.count[0] = min(total, S.max_units);
+        *S.phase = (*S.phase + S.k) % 6u;
+    }
 }
 
 // 4c. one thread per unit; the sorted particles are in buffer `ubuf`
@@ -409,18 +414,23 @@ __global__ void k_fill_units(const SortParams S, int ubuf) {
     const int gs = ks[g0], ge = ks[min(g0 + SPAN, R.Nx)];
     const int h0 = (t / (GROUP / 2)) * (SPAN / 2);
     const int hs = ks[h0], he = ks[min(h0 + SPAN / 2, R.Nx)];
-    int a, b;
+    int a = ks[t * TILE], b = ks[min((t + 1) * TILE, R.Nx)];
     if (ge - gs <= S.unit_p) {  // the whole group (t is its first tile)
         a = gs;
         b = ge;
     } else if (he - hs <= S.unit_p) {  // the half group (t is its first tile)
         a = hs;
         b = he;
-    } else {
-        const int ts = ks[t * TILE], te = ks[min((t + 1) * TILE, R.Nx)];
-        a = ts + (v - tf[t]) * S.unit_p;
-        b = min(a + S.unit_p, te);
     }
+    // part i of [a, b); where parts of one unit meet, at a multiple of 4 particles, so
+    // that the push's slots, and with them its results, are those of the whole unit
+    const int i = v - tf[t], e = b;
+    auto cut = [&](int j) {
+        const int p = a + j * S.part_p;
+        return (j * S.part_p) % S.unit_p ? p & ~3 : p;
+    };
+    b = (i + 1) * S.part_p < e - a ? cut(i + 1) : e;
+    a = cut(i);
     const int32_t* cell = R.sp[s][ubuf].cell;
     S.units.run[u] = run;
     S.units.species[u] = s;
@@ -524,7 +534,7 @@ void launch_sort(const SortParams& S, cudaStream_t st, int* launches) {
     *launches += 8;
 }
 
-void launch_build_units(const SortParams& S, cudaStream_t st, int* launches) {
+void launch_build_units(const SortParams& S, cudaStream_t st, int* launches) {  // S.k == 0
     const dim3 kg(S.kb_max, S.nruns, 2);
     k_zero_keycount<<<dim3(64, S.nruns, 2), 256, 0, st>>>(S);
     k_hist<<<dim3(256, S.nruns, 2), 256, 0, st>>>(S);

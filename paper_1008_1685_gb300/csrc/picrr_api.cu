@@ -107,7 +107,7 @@ struct RunHost {
     int64_t t_offset = 0;      // steps the run had made before it was restored from a checkpoint
     int64_t steps_target = 0;  // 0: unlimited
     int64_t steps_done = 0;
-    int pbuf = 0, fbuf = 0;    // particle / field buffer of a finished run
+    int pbuf = 0, fbuf = 0, jset = 2;  // particle / field buffer and last current set of a finished run
     int fp_bits = 40;
     size_t glen = 0;
     std::vector<std::pair<void*, size_t>> mem;  // device allocations of this run
@@ -118,6 +118,7 @@ struct Batch {
     pic_config cfg{};
     int device = 0, sort_interval = 8, max_runs = 1;
     int unit_p = UNIT_P;  // particles per work unit at most (a run-time shape)
+    int part_p = UNIT_P;  // particles per part of a unit (part_size, chosen whenever the unit table is rebuilt for other runs)
     int slot_w = 2;       // particles per thread and round of the push kernel (2 or 4; the tuner picks)
     double dx = 0, dt = 0, cfl = 0, eps = 0;
     cudaStream_t stream = nullptr, own_stream = nullptr;
@@ -136,12 +137,13 @@ struct Batch {
     int inc_slot = 0;
 
     // CUDA graphs of one sort interval of steps (its pushes, Yee updates and
-    // the sort that ends it), by [step parity at the chunk start][current
-    // particle buffer].  The kernels read the run table at run time, so a
-    // graph stays valid while launch shapes and table pointers do (epoch).
+    // the sort that ends it), by the current particle buffer at its start.
+    // The kernels read the run table and the step number (d_phase) at run
+    // time, so a graph stays valid while launch shapes and table pointers do
+    // (epoch).
     cudaStream_t cap_stream = nullptr;
-    cudaGraphExec_t graph[2][2] = {};
-    uint64_t graph_epoch[2][2] = {};
+    cudaGraphExec_t graph[2] = {};
+    uint64_t graph_epoch[2] = {};
     uint64_t epoch = 1;
     bool graphs_on = true;
     int64_t graph_launches = 0;
@@ -149,15 +151,16 @@ struct Batch {
     // push, Yee update and the sort: the event pairs of each graph, whether it
     // was captured with them, and whether a launch of it has not been read yet
     // (it is read before the same graph is launched again).
-    std::vector<EventPair> graph_ev[2][2];
-    bool graph_timed[2][2] = {};
-    bool graph_unread[2][2] = {};
+    std::vector<EventPair> graph_ev[2];
+    bool graph_timed[2] = {};
+    bool graph_unread[2] = {};
 
     UnitTable units{};
     int max_units = 0;
     double* rad_part = nullptr;
     int32_t *cnt = nullptr, *offs = nullptr, *rs_units = nullptr;
     int* d_status = nullptr;
+    unsigned* d_phase = nullptr;  // batch step of the last sort mod 6, advanced by the sort
     double* diag_partials = nullptr;
     double* diag_out = nullptr;
     unsigned long long* snap_out = nullptr;  // [4]: max d bits, max chi bits, flagged count
@@ -168,6 +171,7 @@ struct Batch {
     int since_sort = 0;
     int cur = 0;
     bool table_dirty = true, layout_dirty = true;
+    int nsets = 3;          // current sets in rotation: 3 when the coming steps are fused, else 2
 
     int64_t launches = 0, push_launches = 0, sorts = 0, timed_push = 0;
     bool timing = false;
@@ -315,31 +319,30 @@ void collect_timing(Batch* b) {
     b->pending.clear();
 }
 
-// Times of the last launch of chunk graph [par0][cur] (waits for its last event).
-void read_graph_timing(Batch* b, int par0, int cur) {
-    if (!b->graph_unread[par0][cur]) return;
-    b->graph_unread[par0][cur] = false;
-    const std::vector<EventPair>& ev = b->graph_ev[par0][cur];
+// Times of the last launch of chunk graph [cur] (waits for its last event).
+void read_graph_timing(Batch* b, int cur) {
+    if (!b->graph_unread[cur]) return;
+    b->graph_unread[cur] = false;
+    const std::vector<EventPair>& ev = b->graph_ev[cur];
     if (ev.empty() || cudaEventSynchronize(ev.back().b) != cudaSuccess) return;
     for (const EventPair& ep : ev) add_timing(b, ep);
 }
 
 void read_all_graph_timing(Batch* b) {
-    for (int p = 0; p < 2; ++p)
-        for (int c = 0; c < 2; ++c) read_graph_timing(b, p, c);
+    for (int c = 0; c < 2; ++c) read_graph_timing(b, c);
 }
 
-// Drop graph [par0][cur] and give its events back (after reading them).
-void drop_graph(Batch* b, int par0, int cur) {
-    read_graph_timing(b, par0, cur);
-    if (b->graph[par0][cur]) cudaGraphExecDestroy(b->graph[par0][cur]);
-    b->graph[par0][cur] = nullptr;
-    for (EventPair& ep : b->graph_ev[par0][cur]) {
+// Drop graph [cur] and give its events back (after reading them).
+void drop_graph(Batch* b, int cur) {
+    read_graph_timing(b, cur);
+    if (b->graph[cur]) cudaGraphExecDestroy(b->graph[cur]);
+    b->graph[cur] = nullptr;
+    for (EventPair& ep : b->graph_ev[cur]) {
         b->ev_free.push_back(ep.a);
         b->ev_free.push_back(ep.b);
     }
-    b->graph_ev[par0][cur].clear();
-    b->graph_timed[par0][cur] = false;
+    b->graph_ev[cur].clear();
+    b->graph_timed[cur] = false;
 }
 
 // ---------------------------------------------------------------------------
@@ -391,6 +394,7 @@ pic_status batch_create(const pic_config* cfg, int max_runs, Batch** out) {
     if ((st = dalloc_t(b, b->mem, &b->d_runs, static_cast<size_t>(max_runs))) != PIC_OK ||
         (st = dalloc_t(b, b->mem, &b->d_inc, static_cast<size_t>(max_runs) * 6 * KMAX)) != PIC_OK ||
         (st = dalloc_t(b, b->mem, &b->d_status, 4)) != PIC_OK ||
+        (st = dalloc_t(b, b->mem, &b->d_phase, 1)) != PIC_OK ||
         (st = dalloc_t(b, b->mem, &b->diag_partials, kMaxDiagBlocks)) != PIC_OK ||
         (st = dalloc_t(b, b->mem, &b->diag_out, 8)) != PIC_OK ||
         (st = dalloc_t(b, b->mem, &b->snap_out, 4)) != PIC_OK ||
@@ -437,14 +441,13 @@ void batch_destroy(Batch* b) {
         if (b->inc_ev[i]) cudaEventDestroy(b->inc_ev[i]);
     if (b->h_runs) cudaFreeHost(b->h_runs);
     if (b->h_inc) cudaFreeHost(b->h_inc);
-    for (int p = 0; p < 2; ++p)
-        for (int c = 0; c < 2; ++c) {
-            if (b->graph[p][c]) cudaGraphExecDestroy(b->graph[p][c]);
-            for (EventPair& ep : b->graph_ev[p][c]) {
-                cudaEventDestroy(ep.a);
-                cudaEventDestroy(ep.b);
-            }
+    for (int c = 0; c < 2; ++c) {
+        if (b->graph[c]) cudaGraphExecDestroy(b->graph[c]);
+        for (EventPair& ep : b->graph_ev[c]) {
+            cudaEventDestroy(ep.a);
+            cudaEventDestroy(ep.b);
         }
+    }
     if (b->cap_stream) cudaStreamDestroy(b->cap_stream);
     if (b->own_stream) cudaStreamDestroy(b->own_stream);
     delete b;
@@ -481,7 +484,7 @@ pic_status run_open(Batch* b, double length_lambda, int source_node, int rr_on, 
     pic_status st = PIC_OK;
     for (int x = 0; x < 2 && st == PIC_OK; ++x)
         for (int c = 0; c < 5 && st == PIC_OK; ++c) st = dalloc_t(b, r.mem, &d.F[x][c], r.glen);
-    for (int x = 0; x < 2 && st == PIC_OK; ++x)
+    for (int x = 0; x < 3 && st == PIC_OK; ++x)
         for (int c = 0; c < 3 && st == PIC_OK; ++c) st = dalloc_t(b, r.mem, &d.J[x][c], r.glen);
     if (st == PIC_OK) st = dalloc_t(b, r.mem, &d.tally, 4);
     const size_t nk = static_cast<size_t>(Nx) + 2, nkb = static_cast<size_t>(Nx) / KEY_T + 2,
@@ -513,7 +516,7 @@ size_t rounded(size_t bytes) { return ((bytes ? bytes : 16) + 255) & ~static_cas
 size_t run_footprint_cpl(double cells_per_lambda, double length_lambda, int64_t n) {
     const int64_t Nx = std::llround(length_lambda * cells_per_lambda);
     const size_t glen = (static_cast<size_t>(Nx) + 1 + 2 * PADF + 4 + 3) / 4 * 4;
-    size_t t = 10 * rounded(glen * 4) + 6 * rounded(glen * 8) + 3 * rounded(glen * 4) + rounded(32);
+    size_t t = 10 * rounded(glen * 4) + 9 * rounded(glen * 8) + rounded(32);
     const size_t nk = static_cast<size_t>(Nx) + 2, nkb = static_cast<size_t>(Nx) / KEY_T + 2,
                  ntl = static_cast<size_t>(Nx) / TILE + 3;
     t += 2 * (2 * rounded(nk * 4) + 2 * rounded(nkb * 4) + 2 * rounded(ntl * 4));
@@ -797,6 +800,13 @@ void finalize_run_params(Batch* b, RunHost& r) {
     d.rr = r.rr;
 }
 
+// Particles per part of a unit for `total` particles in the batch's active runs.
+int part_size(int64_t total, int unit_p) {
+    int p = PART_MIN;
+    while (p < unit_p && total > static_cast<int64_t>(p) * PARTS) p *= 2;
+    return p;
+}
+
 // Grow the batch-level unit table and sort scratch to hold `need` units.
 pic_status ensure_units(Batch* b, int need) {
     if (need <= b->max_units) return PIC_OK;
@@ -856,6 +866,8 @@ SortParams sort_params(Batch* b) {
         if (r.used) mx = std::max(mx, r.Nx);
     S.kb_max = (mx + KEY_T - 1) / KEY_T;
     S.unit_p = b->unit_p;
+    S.phase = b->d_phase;
+    S.part_p = b->part_p;
     return S;
 }
 
@@ -940,6 +952,24 @@ void do_sort(Batch* b) {
     b->since_sort = 0;
 }
 
+// Unit table entries that the runs for which `counts` holds can need with units of unit_p particles (each tile
+// adds at most one partial entry; merged groups only lower the count), and the size of a unit's parts.
+template <class Counts>
+int64_t units_needed(const Batch* b, int unit_p, Counts counts, int* part) {
+    int64_t total = 0, need = 1;
+    for (const auto& r : b->runs)
+        for (int s = 0; counts(r) && s < 2; ++s)
+            if (r.sp[s].loaded) total += r.sp[s].n;
+    *part = part_size(total, unit_p);
+    for (const auto& r : b->runs) {
+        if (!counts(r)) continue;
+        const int ntiles = (r.Nx + TILE - 1) / TILE;
+        for (int s = 0; s < 2; ++s)
+            if (r.sp[s].loaded) need += (r.sp[s].n + *part - 1) / *part + ntiles + 1;
+    }
+    return need;
+}
+
 // Start runs that have not stepped yet.  They join at a sort boundary, so
 // that every active run's particles are sorted when the unit table is rebuilt
 // (their own particles were loaded in cell order into the current buffer).
@@ -957,27 +987,25 @@ pic_status activate_pending(Batch* b) {
             if (r.used && !r.started)
                 for (int s = 0; s < 2; ++s) std::swap(r.dev.sp[s][0], r.dev.sp[s][1]);
     }
-    // units the active and the joining runs can need (each tile adds at most one partial unit)
-    int64_t need = 1;
+    // unit table entries the active and the joining runs can need (each tile adds at most one partial one)
     std::vector<int> joining;
-    for (int i = 0; i < b->max_runs; ++i) {
-        const RunHost& r = b->runs[i];
-        if (!r.used || r.finished || (r.started && !r.active)) continue;
-        if (!r.started) joining.push_back(i);
-        const int ntiles = (r.Nx + TILE - 1) / TILE;
-        for (int s = 0; s < 2; ++s)
-            if (r.sp[s].loaded) need += (r.sp[s].n + b->unit_p - 1) / b->unit_p + ntiles + 1;
-    }
+    for (int i = 0; i < b->max_runs; ++i)
+        if (b->runs[i].used && !b->runs[i].started && !b->runs[i].finished) joining.push_back(i);
+    auto counts = [](const RunHost& r) { return r.used && !r.finished && (!r.started || r.active); };
+    int part = 0;
+    const int64_t need = units_needed(b, b->unit_p, counts, &part);
     if (need > (1 << 30)) return fail(b, PIC_ERR_INVALID_ARG, "too many work units");
     st = ensure_units(b, static_cast<int>(need));
     if (st != PIC_OK) return st;  // the joining runs stay pending
+    if (part != b->part_p) b->epoch++;
+    b->part_p = part;
     for (int i : joining) {
         RunHost& r = b->runs[i];
         finalize_run_params(b, r);
         r.started = true;
         r.active = true;
         r.admit_step = b->gstep;
-        r.dev.fpar = static_cast<int>(b->gstep & 1);  // buffer 0 is current at the first step
+        r.dev.fpar = static_cast<int>((6 - b->gstep % 6) % 6);  // buffer 0 and current set 0 at the first step
     }
     b->table_dirty = b->layout_dirty = true;
     st = upload_blocks(b);
@@ -993,12 +1021,16 @@ pic_status activate_pending(Batch* b) {
     return PIC_OK;
 }
 
+// Phase of the step `ahead` steps after the next one.
+unsigned phase_of(const Batch* b, int ahead) { return static_cast<unsigned>((b->gstep + ahead) % 6); }
+
 void deactivate(Batch* b, int id) {
     RunHost& r = b->runs[id];
     r.active = false;
     r.finished = true;
     r.pbuf = b->cur;
-    r.fbuf = static_cast<int>((b->gstep + r.dev.fpar) & 1);
+    r.fbuf = field_buf(r.dev, phase_of(b, 0));
+    r.jset = current_set(r.dev, phase_of(b, 5), b->nsets);  // the set of step gstep - 1
     b->table_dirty = b->layout_dirty = true;
 }
 
@@ -1024,13 +1056,14 @@ pic_status upload_incident(Batch* b, int steps) {
     return PIC_OK;
 }
 
-PushParams push_params(const Batch* b, int64_t gstep, int k, int cur) {
+PushParams push_params(const Batch* b, int k, int cur) {
     PushParams P{};
     P.runs = b->d_runs;
     P.units = b->units;
     P.rad_part = b->rad_part;
     P.status = b->d_status;
-    P.gstep = gstep;
+    P.phase = b->d_phase;
+    P.nsets = b->nsets;
     P.k = k;
     P.cur = cur;
     P.cfl = static_cast<float>(b->cfl);
@@ -1039,13 +1072,17 @@ PushParams push_params(const Batch* b, int64_t gstep, int k, int cur) {
     return P;
 }
 
-FieldParams field_params(const Batch* b, int64_t gstep, int j) {
+// The Yee update of the step k steps after the last sort, whose source values are row j of d_inc.
+FieldParams field_params(const Batch* b, int k, int j) {
     FieldParams Q{};
     Q.runs = b->d_runs;
     Q.blk_run = b->d_blk_run;
     Q.blk_i0 = b->d_blk_i0;
     Q.inc = b->d_inc + static_cast<size_t>(j) * 6 * b->max_runs;
-    Q.gstep = gstep;
+    Q.phase = b->d_phase;
+    Q.k = k;
+    Q.nblk = b->nblk;
+    Q.nsets = b->nsets;
     Q.dt = b->dt;
     Q.c = static_cast<float>(b->cfl);
     Q.hc = static_cast<float>(0.5 * b->cfl);
@@ -1053,18 +1090,48 @@ FieldParams field_params(const Batch* b, int64_t gstep, int j) {
     return Q;
 }
 
-// The graph of one sort interval starting at step parity par0 with current
-// particle buffer cur (captured on the batch's capture stream, then reused).
-pic_status chunk_graph(Batch* b, int par0, int cur, cudaGraphExec_t* out) {
-    cudaGraphExec_t& ex = b->graph[par0][cur];
-    if (ex && b->graph_epoch[par0][cur] == b->epoch && b->graph_timed[par0][cur] == b->timing) {
+// With 2 particles per thread a push that follows another one also does the Yee update of the step before
+// (launch_push); the last push's update is a launch of its own.  That pays while the units leave the GPU
+// half empty, where a step is a chain of latencies (small run 35 -> 30 us per step); with more units each
+// block's update of its own window costs more than the launch it saves (thin plasma, 2700 units, 142 -> 158
+// us; a 48-run scan, 1600 units, 125 -> 134 us).  The 4-per-thread kernel (dense foils, for which the Yee
+// update is a hundredth of a step) leaves every update to the Yee kernel.
+bool fuses(const Batch* b) {
+    if (b->slot_w != 2) return false;
+    int64_t units = 0;  // about: full units, and tile groups
+    for (const auto& r : b->runs) {
+        if (!r.used || !r.active) continue;
+        for (int s = 0; s < 2; ++s)
+            if (r.sp[s].loaded) units += r.sp[s].n / b->unit_p;
+    }
+    return units <= FUSE_UNITS;
+}
+
+// Whether the coming steps are fused.  Fused steps rotate three current sets, others two: a change clears them all.
+bool begin_steps(Batch* b) {
+    const bool fz = fuses(b);
+    if (b->nsets != (fz ? 3 : 2)) {
+        b->nsets = fz ? 3 : 2;
+        b->epoch++;
+        launch_zero_current(field_params(b, b->since_sort, 0), b->stream);
+        b->launches++;
+    }
+    return fz;
+}
+
+// The graph of one sort interval with current particle buffer cur at its start
+// (captured on the batch's capture stream, then reused).
+pic_status chunk_graph(Batch* b, int cur, cudaGraphExec_t* out) {
+    cudaGraphExec_t& ex = b->graph[cur];
+    if (ex && b->graph_epoch[cur] == b->epoch && b->graph_timed[cur] == b->timing) {
         *out = ex;
         return PIC_OK;
     }
-    drop_graph(b, par0, cur);
+    drop_graph(b, cur);
     const int I = b->sort_interval;
+    const bool fz = fuses(b);
     cudaStream_t cs = b->cap_stream;
-    std::vector<EventPair>& ev = b->graph_ev[par0][cur];
+    std::vector<EventPair>& ev = b->graph_ev[cur];
     // timing on: an event-record node before and after each timed launch
     auto mark = [&](int kind, bool open) {
         if (!b->timing) return;
@@ -1073,11 +1140,13 @@ pic_status chunk_graph(Batch* b, int par0, int cur, cudaGraphExec_t* out) {
     };
     PIC_CK(b, cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal));
     for (int j = 0; j < I; ++j) {
+        const bool fused = fz && j > 0;
         mark(0, true);
-        launch_push(push_params(b, par0 + j, j, cur), b->max_units, b->slot_w, cs);
+        launch_push(push_params(b, j, cur), field_params(b, j - 1, fused ? j - 1 : 0), fused, b->max_units, b->slot_w, cs);
         mark(0, false);
+        if (fz && j + 1 < I) continue;
         mark(1, true);
-        launch_field(field_params(b, par0 + j, j), b->nblk, cs);
+        launch_field(field_params(b, j, j), b->nblk, cs);
         mark(1, false);
     }
     mark(2, true);
@@ -1096,8 +1165,8 @@ pic_status chunk_graph(Batch* b, int par0, int cur, cudaGraphExec_t* out) {
         ex = nullptr;
         return cuda_fail(b, e, "chunk graph");
     }
-    b->graph_epoch[par0][cur] = b->epoch;
-    b->graph_timed[par0][cur] = b->timing;
+    b->graph_epoch[cur] = b->epoch;
+    b->graph_timed[cur] = b->timing;
     *out = ex;
     return PIC_OK;
 }
@@ -1109,11 +1178,21 @@ pic_status batch_step(Batch* b, int64_t n, int64_t* done) {
     if ((st = upload_table(b)) != PIC_OK) return st;
     if ((st = upload_blocks(b)) != PIC_OK) return st;
     const int I = b->sort_interval;
+    bool fz = n > 0 && begin_steps(b);
     int64_t it = 0;
     // laser source values of the single steps below, uploaded for up to KMAX
     // steps at a time (one copy instead of one per step); a graph launch
     // uploads its own interval over them
     int inc_pos = 0, inc_len = 0;
+    // the Yee update of the last single step, not launched yet (its source values are row inc_pos - 1)
+    bool field_due = false;
+    auto finish_field = [&] {
+        if (!field_due) return;
+        field_due = false;
+        Timed t(b, 1);
+        launch_field(field_params(b, b->since_sort - 1, inc_pos - 1), b->nblk, b->stream);
+        b->launches++;
+    };
     while (it < n) {
         int nact = 0;
         bool whole_chunk = b->graphs_on && b->since_sort == 0 && n - it >= I;
@@ -1126,15 +1205,15 @@ pic_status batch_step(Batch* b, int64_t n, int64_t* done) {
         if (whole_chunk) {
             // a whole sort interval as one graph launch; no run ends before its last step
             cudaGraphExec_t ex = nullptr;
-            const int gp = static_cast<int>(b->gstep & 1), gc = b->cur;
-            if ((st = chunk_graph(b, gp, gc, &ex)) != PIC_OK) return st;
+            const int gc = b->cur;
+            if ((st = chunk_graph(b, gc, &ex)) != PIC_OK) return st;
             if ((st = upload_incident(b, I)) != PIC_OK) return st;
             inc_pos = inc_len = 0;
-            read_graph_timing(b, gp, gc);  // its previous launch (two chunks ago), before its events are reused
+            read_graph_timing(b, gc);  // its previous launch (two chunks ago), before its events are reused
             PIC_CK(b, cudaGraphLaunch(ex, b->stream));
-            b->graph_unread[gp][gc] = b->timing;
+            b->graph_unread[gc] = b->timing;
             b->graph_launches++;
-            b->launches += 2 * I + 1 + 8;
+            b->launches += (fz ? I + 1 : 2 * I) + 1 + 8;
             b->push_launches += I;
             b->gstep += I;
             b->cur ^= 1;
@@ -1153,25 +1232,26 @@ pic_status batch_step(Batch* b, int64_t n, int64_t* done) {
                 }
                 if ((st = upload_table(b)) != PIC_OK) return st;
                 if ((st = upload_blocks(b)) != PIC_OK) return st;
+                fz = begin_steps(b);
             }
             cudaError_t e = cudaGetLastError();
             if (e != cudaSuccess) return cuda_fail(b, e, "chunk launch");
             continue;
         }
-        if (inc_pos >= inc_len) {
+        const bool upload = inc_pos >= inc_len;
+        if (upload) {
+            finish_field();  // its source values are about to be overwritten
             inc_len = static_cast<int>(std::min<int64_t>(n - it, KMAX));
             inc_pos = 0;
             if ((st = upload_incident(b, inc_len)) != PIC_OK) return st;
         }
         {
             Timed t(b, 0);
-            launch_push(push_params(b, b->gstep, b->since_sort, b->cur), b->max_units, b->slot_w, b->stream);
+            launch_push(push_params(b, b->since_sort, b->cur), field_params(b, b->since_sort - 1, field_due ? inc_pos - 1 : 0),
+                        field_due, b->max_units, b->slot_w, b->stream);
         }
-        {
-            Timed t(b, 1);
-            launch_field(field_params(b, b->gstep, inc_pos++), b->nblk, b->stream);
-        }
-        b->launches += 2;
+        b->launches++;
+        inc_pos++;
         b->push_launches++;
         b->gstep++;
         b->since_sort++;
@@ -1181,6 +1261,9 @@ pic_status batch_step(Batch* b, int64_t n, int64_t* done) {
             r.steps_done++;
             if (r.steps_target > 0 && r.steps_done >= r.steps_target) ended = true;
         }
+        // the step's Yee update: left to the next push if that one directly follows
+        field_due = true;
+        if (!fz || ended || b->since_sort >= b->sort_interval) finish_field();
         // a run that ends on a sort step is sorted first, as it would be alone
         if (b->since_sort >= b->sort_interval) do_sort(b);
         if (ended) {
@@ -1191,6 +1274,7 @@ pic_status batch_step(Batch* b, int64_t n, int64_t* done) {
             }
             if ((st = upload_table(b)) != PIC_OK) return st;
             if ((st = upload_blocks(b)) != PIC_OK) return st;
+            fz = begin_steps(b);
         }
         if ((it & 255) == 255) {
             cudaError_t e = cudaGetLastError();
@@ -1198,6 +1282,7 @@ pic_status batch_step(Batch* b, int64_t n, int64_t* done) {
         }
         ++it;
     }
+    finish_field();
     if (it > 0 && b->since_sort > 0) rad_flush(b);
     cudaError_t e = cudaStreamSynchronize(b->stream);
     if (e == cudaSuccess) e = cudaGetLastError();
@@ -1210,19 +1295,6 @@ pic_status batch_step(Batch* b, int64_t n, int64_t* done) {
     if (hst & ST_TIMEOUT) return fail(b, PIC_ERR_TIMEOUT, "a bounded device wait (TMA field window) gave up");
     if (hst & ST_WINDOW) return fail(b, PIC_ERR_STATE, "a particle left its unit window");
     return PIC_OK;
-}
-
-// Units a batch can need with unit size unit_p (each tile adds at most one
-// partial unit; merged groups only lower the count).
-int64_t units_needed(const Batch* b, int unit_p) {
-    int64_t need = 1;
-    for (const auto& r : b->runs) {
-        if (!r.used || !r.active) continue;
-        const int ntiles = (r.Nx + TILE - 1) / TILE;
-        for (int s = 0; s < 2; ++s)
-            if (r.sp[s].loaded) need += (r.sp[s].n + unit_p - 1) / unit_p + ntiles + 1;
-    }
-    return need;
 }
 
 // Set the launch shapes: work-unit size (takes effect through a sort now, which
@@ -1240,10 +1312,12 @@ pic_status set_shapes(Batch* b, int unit_p, int interval, int slot_w) {
         // sort with the current table first (it also flushes the radiated
         // partials), then rebuild the table from the sorted cells with the new size
         if (any && b->since_sort > 0) do_sort(b);
-        const int64_t need = units_needed(b, unit_p);
+        int part = 0;
+        const int64_t need = units_needed(b, unit_p, [](const RunHost& r) { return r.used && r.active; }, &part);
         if (need > (1 << 30)) return fail(b, PIC_ERR_INVALID_ARG, "too many work units");
         if ((st = ensure_units(b, static_cast<int>(need))) != PIC_OK) return st;
         b->unit_p = unit_p;
+        b->part_p = part;
         if (any) {
             SortParams S = sort_params(b);
             int nl = 0;
@@ -1336,7 +1410,13 @@ int run_pbuf(const Batch* b, const RunHost& r) { return r.finished ? r.pbuf : b-
 int run_fbuf(const Batch* b, const RunHost& r) {
     if (r.finished) return r.fbuf;
     if (!r.started) return 0;
-    return static_cast<int>((b->gstep + r.dev.fpar) & 1);
+    return field_buf(r.dev, phase_of(b, 0));
+}
+// current set of a run's last step (the one before its first step: 2)
+int run_jset(const Batch* b, const RunHost& r) {
+    if (r.finished) return r.jset;
+    if (!r.started) return 2;
+    return current_set(r.dev, phase_of(b, 5), b->nsets);
 }
 
 pic_status run_energy(Batch* b, int id, double out[6]) {
@@ -1549,12 +1629,11 @@ pic_status run_snapshot(Batch* b, int id, int species, double chi_flag, int64_t 
 
 // The current of a run's last step, component c (Jx, Jy, Jz), on the whole
 // padded grid: its fixed-point accumulators (the set of the last step, kept
-// until the next step's Yee update zeroes it) times 2^-fp.  Before the first
+// until the Yee update of the next step zeroes it) times 2^-fp.  Before the first
 // step that set holds zeros, or the current a checkpoint restored into it.
 pic_status last_current(Batch* b, const RunHost& r, int c, std::vector<double>& out) {
-    const int lp = 1 - run_fbuf(b, r);
     std::vector<long long> h(r.glen);
-    PIC_CK(b, cudaMemcpyAsync(h.data(), r.dev.J[lp][c], sizeof(long long) * r.glen, cudaMemcpyDeviceToHost,
+    PIC_CK(b, cudaMemcpyAsync(h.data(), r.dev.J[run_jset(b, r)][c], sizeof(long long) * r.glen, cudaMemcpyDeviceToHost,
                               b->stream));
     PIC_CK(b, cudaStreamSynchronize(b->stream));
     out.resize(r.glen);
@@ -1714,13 +1793,13 @@ pic_status run_restore(Batch* b, int id, FILE* f, const CkHeader& h) {
     r.fields_set = true;
     r.t_offset = h.steps;
     // the saved current goes into the accumulator set a run reads back before
-    // its first step (1), in the fixed-point scale the run will step with
+    // its first step (2), in the fixed-point scale the run will step with
     finalize_run_params(b, r);
     std::vector<long long> acc(r.glen);
     for (int c = 0; c < 3; ++c) {
         for (size_t i = 0; i < r.glen; ++i)
             acc[i] = std::llround(std::ldexp(static_cast<double>(jsaved[c * r.glen + i]), r.fp_bits));
-        PIC_CK(b, cudaMemcpy(r.dev.J[1][c], acc.data(), sizeof(long long) * r.glen, cudaMemcpyHostToDevice));
+        PIC_CK(b, cudaMemcpy(r.dev.J[2][c], acc.data(), sizeof(long long) * r.glen, cudaMemcpyHostToDevice));
     }
     return PIC_OK;
 }

@@ -10,9 +10,12 @@
 //                 PADF holds node / half node 0; the guard elements are zero.
 //                 Ex, Ey, Ez, By, Bz are ping-ponged by the Yee kernel.
 //   accumulators  int64 fixed point (2^fp units) for Jx (half nodes) and
-//                 Jy, Jz (nodes), two sets alternating by step parity; the
-//                 set of the last step holds its current until the next
-//                 step's Yee update zeroes it (read-back converts it).
+//                 Jy, Jz (nodes).  A step adds into one set; its current is
+//                 read by the step's Yee update and stays readable until the
+//                 next step.  Two sets alternate, the Yee update zeroing the
+//                 other one; three rotate when the Yee update runs inside the
+//                 push of the next step, which needs the next set zero already
+//                 (the update then zeroes the third).
 //   particles     per species, structure of arrays, two buffers each
 //                 (ping-ponged by the sort): cell int32, off/px/py/pz float,
 //                 id int32.  A particle that left the box is frozen at the
@@ -47,6 +50,15 @@ constexpr int UNIT_P_MAX = 16384;
 // with which the same kernel ran 1.5 % (dense) to 2.8 % (thin) slower.
 constexpr int KMAX = 96;
 constexpr int PUSH_T = 256;       // threads of the push kernel
+// When the units (of at most unit_p particles) would not fill the GPU, they are cut into parts, each a unit
+// table entry of its own: about PARTS of them for all particles, none below PART_MIN (one round of the push).
+// One CTA per unit took 27 us for the 12 units of a small run, eight rounds one after the other; with parts
+// 12 us.
+// 1216 (8 CTAs on each of 152 SMs) against 608, 912 and 2432: the paper-scale run 27.0 us per step with 1216,
+// 27.7, 27.6 and 28.4 otherwise; the small run 15.7 with each.
+constexpr int PARTS = 1216;
+constexpr int PART_MIN = 512;
+constexpr int FUSE_UNITS = 456;  // units up to which a push also updates its fields (picrr_api.cu, fuses)
 constexpr int WMAX = SPAN + 2 * KMAX + 16;  // window length bound in the push kernel (>= SPAN + 2 KMAX + 9)
 constexpr int SSTR = SPAN + 2 * KMAX + 4;   // per-unit key-window stride of the sort scratch (>= SPAN + 2 KMAX)
 constexpr int FIELD_T = 128;      // threads of the Yee kernel
@@ -96,10 +108,10 @@ struct RunDev {
     int32_t rr;            // radiation reaction on electrons
     int32_t active;        // stepped by the batch
     int32_t Nx, is, glen;
-    int32_t fpar;          // field / current buffer at batch step g: (g + fpar) & 1
+    int32_t fpar;          // batch step g is the run's step g + fpar mod 6, its first one step 0
     float fp_inv;          // 2^-fp of the current accumulators
     float* F[2][5];        // [buffer][Ex, Ey, Ez, By, Bz], padded
-    unsigned long long* J[2][3];  // [parity][Jx, Jy, Jz], padded
+    unsigned long long* J[3][3];  // [set][Jx, Jy, Jz], padded
     double* tally;         // [4]: radiated, flux in, flux out, spare
     int32_t* keycount[2];  // sort scratch per species: [Nx + 2]
     int32_t* keystart[2];  // [Nx + 2]; keystart[Nx] = particles
@@ -109,13 +121,20 @@ struct RunDev {
     int32_t* tile_first[2];
 };
 
+// Buffers of a run at a batch step of phase g: the step, or anything equal to it mod 6 (and >= 0).
+__host__ __device__ inline int field_buf(const RunDev& R, unsigned g) { return static_cast<int>((g + R.fpar) & 1u); }
+__host__ __device__ inline int current_set(const RunDev& R, unsigned g, int nsets) {
+    return static_cast<int>(nsets == 3 ? (g + R.fpar) % 3u : (g + R.fpar) & 1u);
+}
+
 struct PushParams {
     const RunDev* runs;
     UnitTable units;
     double* rad_part;   // [max_units] radiated energy of each unit since the last flush
     int* status;
-    int64_t gstep;      // batch step
+    const unsigned* phase;  // batch step of the last sort mod 6 (kept on the device, so that a graph can be reused)
     int k;              // steps since the last sort
+    int nsets;          // current sets in rotation
     int cur;            // particle buffer
     float cfl, dt, eps;
 };
@@ -133,7 +152,10 @@ struct FieldParams {
     // t_n + dt/2 + dx/2 (half node before it) and t_{n+1}:
     // Ey_inc = Bz_inc = ay, Ez_inc = -By_inc = az
     const float* inc;        // [runs * 6]
-    int64_t gstep;
+    const unsigned* phase;   // batch step of the last sort mod 6
+    int k;                   // steps since the last sort, of the step whose fields are updated
+    int nblk;                // blocks
+    int nsets;               // current sets in rotation: 2, or 3 in sequences of fused launches
     double dt;
     float c, hc, fdt;        // cfl, cfl/2, dt
 };
@@ -194,8 +216,12 @@ __device__ __forceinline__ void tma_load_1d(void* dst_smem, const void* src_gmem
 // ---------------------------------------------------------------------------
 // Host-side launch wrappers (each defined in its own translation unit).
 // ---------------------------------------------------------------------------
-void launch_push(const PushParams& P, int grid, int slot_w, cudaStream_t st);  // slot_w: 4 or 2 particles per thread and round
+// slot_w: 4 or 2 particles per thread and round.  fused (slot_w 2 only): also the Yee update of the step
+// before, whose parameters are Q: the push's blocks update the fields of their own windows, and Q.nblk more
+// blocks in front write the new fields.
+void launch_push(const PushParams& P, const FieldParams& Q, bool fused, int grid, int slot_w, cudaStream_t st);
 void launch_field(const FieldParams& P, int grid, cudaStream_t st);
+void launch_zero_current(const FieldParams& P, cudaStream_t st);
 
 struct SortParams {
     RunDev* runs;
@@ -208,6 +234,8 @@ struct SortParams {
     int k, cur, max_units;
     int kb_max;            // key blocks of the largest run: ceil(max Nx / 256)
     int unit_p;            // particles per unit at most (UNIT_P_MIN..UNIT_P_MAX)
+    unsigned* phase;       // += k, mod 6
+    int part_p;            // particles per part of a unit (a power of two, PART_MIN..unit_p)
 };
 // Full re-sort of every active run (bounded displacement since the last sort)
 // and the new unit table; particles move from buffer cur to 1 - cur.
