@@ -4,27 +4,32 @@
 // The sort is a stable counting sort by cell (a particle frozen at a wall
 // sorts under its last cell).  It exploits what the push guarantees: a
 // particle moves less than one cell per step, so k steps after the last sort
-// every particle of unit u has a cell in [lo_u - k, hi_u + k].  Hence, for
-// every active run and species of the batch, in one launch per phase:
-//   1. each unit counts its particles per cell of that window (warp-aggregated
-//      shared-memory integer atomics);
-//   2. for each cell the units whose window covers it form a contiguous range
-//      (lo and hi are sorted within a run and species), found by binary
-//      search; the per-cell totals are scanned into the new cell starts, and
-//      every (unit, cell) pair gets its destination offset in unit order;
+// every particle of unit u has a cell in [lo_u - k, hi_u + k].  It takes three
+// launches for all active runs and species of the batch:
+//   1. each unit counts its particles per cell of that window; further blocks
+//      add the runs' radiated partials into their tallies;
+//   2. a block per group of SPAN cells adds the counts of the units whose
+//      windows reach into it (they belong to the same or the neighbouring
+//      groups of the old table), scans them into the new cell starts and gives
+//      every (unit, cell) pair its destination, in unit order.  No scan over
+//      blocks is needed: the particles below a group are those of the units
+//      wholly below it, which the old order counts, and a part of the counts
+//      of the units across its boundary;
 //   3. each unit scatters its particles, ranking equal cells in index order
 //      (each warp owns a contiguous slice; warp match ranks within a warp and
 //      per-warp counts combined in warp order), so the result does not depend
-//      on scheduling;
-//   4. the unit table is rebuilt from the sorted cells: tiles of TILE cells,
-//      split into chunks of at most unit_p particles, except that an aligned
-//      group of GROUP consecutive tiles holding at most unit_p particles
-//      together forms one unit, or else an aligned half group that does
-//      (sparse regions would otherwise give many nearly empty units); when the
-//      units are too few to fill the GPU, each is cut into parts of part_p
-//      particles, which are the table's entries.
-// Every particle is read once and written once; the cell array is read once
-// more for the counts.
+//      on scheduling; further blocks build the new unit table (the tables
+//      alternate) from the cell starts: tiles of TILE cells, split into units
+//      of at most unit_p particles, except that an aligned group of GROUP
+//      consecutive tiles holding at most unit_p particles together forms one
+//      unit, or else an aligned half group that does (sparse regions would
+//      otherwise give many nearly empty units); when the units are too few to
+//      fill the GPU, each is cut into parts of part_p particles, which are the
+//      table's entries.
+// Every particle is read once and written once; the cell array is read twice
+// more for the counts.  In nine launches, with a search for the units of every
+// cell and a scan over blocks in between, a sort of a small run took 42 us and
+// of thin plasma (8.2M particles) 233 us; in these three 18 and 172 us.
 #include <algorithm>
 #include <climits>
 
@@ -37,27 +42,71 @@ namespace {
 constexpr unsigned FULL = 0xffffffffu;
 constexpr int SORT_T = 256;
 constexpr int SCAN_T = 1024;
+constexpr int PLAN_T = SPAN;      // threads of the planning kernel: one per cell of a group
+constexpr int PLAN_UNITS = 1024;  // units near a group whose bounds are kept in shared memory
 
 // sort key of a stored cell: frozen particles (cell = -1 - k) sort under k
 __device__ __forceinline__ int key_of(int c) { return c < 0 ? -1 - c : c; }
 
+__device__ __forceinline__ int groups_of(int Nx) { return (Nx + SPAN - 1) / SPAN; }
+
+// radiated energy of run r: sum of its electron units, fixed order (SORT_T threads)
+__device__ __forceinline__ void rad_flush_block(const RunDev* runs, int r, int nruns, const int32_t* rs_units, double* part,
+                                                double* sred) {
+    const RunDev& R = runs[r];
+    if (!R.active) return;
+    const int b = rs_units[2 * nruns + 2 * r], n = rs_units[2 * r];  // electron units
+    const int t = threadIdx.x;
+    double a[4] = {0.0, 0.0, 0.0, 0.0};
+    for (int i = t; i < n; i += 4 * SORT_T) {
+#pragma unroll
+        for (int q = 0; q < 4; ++q)
+            if (i + q * SORT_T < n) {
+                a[q] += part[b + i + q * SORT_T];
+                part[b + i + q * SORT_T] = 0.0;
+            }
+    }
+    double v = (a[0] + a[1]) + (a[2] + a[3]);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(FULL, v, o);
+    if ((t & 31) == 0) sred[t >> 5] = v;
+    __syncthreads();
+    if (t == 0) {
+        double s = 0.0;
+        for (int w = 0; w < SORT_T / 32; ++w) s += sred[w];
+        R.tally[0] += s;
+    }
+}
+
+__global__ void __launch_bounds__(SORT_T) k_rad_flush(const RunDev* runs, int nruns, const int32_t* rs_units, double* part) {
+    __shared__ double sred[SORT_T / 32];
+    rad_flush_block(runs, blockIdx.x, nruns, rs_units, part, sred);
+}
+
 // ---- 1. per-unit window counts -------------------------------------------------
+// Blocks [0, nruns): a run's radiated partials; then a block per unit.
 __global__ void __launch_bounds__(SORT_T) k_sort_count(const SortParams S) {
     __shared__ int cnt[SSTR];
-    const int u = blockIdx.x;
+    __shared__ double sred[SORT_T / 32];
+    const int u = static_cast<int>(blockIdx.x) - S.nruns;
+    if (u < 0) {  // block-uniform
+        const int r = blockIdx.x;
+        if (threadIdx.x < 2) S.rs_new[2 * r + threadIdx.x] = 0;  // entries of the new table, counted by the next launch
+        rad_flush_block(S.runs, r, S.nruns, S.rs_units, S.rad_part, sred);
+        return;
+    }
     if (u >= S.units.count[0]) return;
     const RunDev& R = S.runs[S.units.run[u]];
     if (!R.active) return;  // a run that ended keeps its particles where they are
     const int s = S.units.species[u];
     const int start = S.units.start[u], end = S.units.end[u];
     const int wb = S.units.lo[u] - S.k;
-    const int L = S.units.hi[u] + S.k + 1 - wb;
-    for (int i = threadIdx.x; i < SSTR; i += SORT_T) cnt[i] = 0;
+    const int L = min(S.units.hi[u] + S.k + 1 - wb, SSTR);
+    for (int i = threadIdx.x; i < L; i += SORT_T) cnt[i] = 0;
     __syncthreads();
     const int32_t* cell = R.sp[s][S.cur].cell;
-    const int lane = threadIdx.x & 31;
-    constexpr int U = 4;  // loads in flight per thread
-    for (int i0 = start; i0 < end; i0 += U * SORT_T) {  // block-uniform trip count
+    constexpr int U = 8;  // loads in flight per thread
+    for (int i0 = start; i0 < end; i0 += U * SORT_T) {
         int c[U];
 #pragma unroll
         for (int m = 0; m < U; ++m) {
@@ -66,56 +115,21 @@ __global__ void __launch_bounds__(SORT_T) k_sort_count(const SortParams S) {
         }
 #pragma unroll
         for (int m = 0; m < U; ++m) {
-            int l = -1;
-            if (c[m] != INT32_MIN) {
-                l = key_of(c[m]) - wb;
-                if (!(l >= 0 && l < L && l < SSTR)) {
-                    atomicOr(S.status, ST_WINDOW);
-                    l = -1;
-                }
-            }
-            // lanes with the same cell add their count once
-            const unsigned peers = __match_any_sync(FULL, l);
-            if (l >= 0 && lane == __ffs(peers) - 1) atomicAdd(&cnt[l], __popc(peers));
+            if (c[m] == INT32_MIN) continue;
+            const int l = key_of(c[m]) - wb;
+            // (adds of one are combined by the hardware when lanes share a cell; matching the
+            // lanes first took 34 us instead of 17 on thin plasma)
+            if (l >= 0 && l < L) atomicAdd(&cnt[l], 1);
+            else atomicOr(S.status, ST_WINDOW);
         }
     }
     __syncthreads();
-    for (int i = threadIdx.x; i < L; i += SORT_T) S.cnt[static_cast<size_t>(u) * SSTR + i] = cnt[i];
+    for (int i = threadIdx.x; i < L; i += SORT_T) S.cnt[static_cast<size_t>(u) * SSTR + i] = static_cast<uint16_t>(cnt[i]);
 }
 
-// Units of run `run`, species s whose window covers cell `key`: [u0, u1].
-__device__ void covering(const SortParams& S, int run, int s, int key, int& u0, int& u1) {
-    const int p = 2 * run + s;
-    const int b = S.rs_units[2 * S.nruns + p], n = S.rs_units[p];
-    int l = 0, r = n;  // first u with hi + k >= key
-    while (l < r) {
-        const int m = (l + r) >> 1;
-        if (S.units.hi[b + m] + S.k >= key) r = m; else l = m + 1;
-    }
-    u0 = b + l;
-    l = 0;
-    r = n;  // last u with lo - k <= key
-    while (l < r) {
-        const int m = (l + r) >> 1;
-        if (S.units.lo[b + m] - S.k <= key) l = m + 1; else r = m;
-    }
-    u1 = b + l - 1;
-}
-
-__device__ __forceinline__ int block_sum_int(int v, int* sh) {
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(FULL, v, o);
-    if (lane == 0) sh[warp] = v;
-    __syncthreads();
-    int t = 0;
-    if (threadIdx.x == 0)
-        for (int w = 0; w < KEY_T / 32; ++w) t += sh[w];
-    return t;
-}
-
-// exclusive scan of v over the block (KEY_T threads)
-__device__ __forceinline__ int block_excl_scan(int v, int* sh) {
+// ---- 2. cell starts, destinations, entries of the new table -----------------------
+// exclusive scan of v over the block (PLAN_T threads)
+__device__ __forceinline__ int plan_scan(int v, int* sh, int* total) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     int x = v;
 #pragma unroll
@@ -126,113 +140,231 @@ __device__ __forceinline__ int block_excl_scan(int v, int* sh) {
     if (lane == 31) sh[warp] = x;
     __syncthreads();
     if (warp == 0) {
-        int w = lane < KEY_T / 32 ? sh[lane] : 0;
+        int w = lane < PLAN_T / 32 ? sh[lane] : 0;
 #pragma unroll
         for (int o = 1; o < 32; o <<= 1) {
             const int y = __shfl_up_sync(FULL, w, o);
             if (lane >= o) w += y;
         }
-        if (lane < KEY_T / 32) sh[lane] = w;
+        if (lane < PLAN_T / 32) sh[lane] = w;
     }
     __syncthreads();
+    *total = sh[PLAN_T / 32 - 1];
     return x - v + (warp > 0 ? sh[warp - 1] : 0);
 }
 
-// exclusive scan of n ints by one block of SCAN_T threads (each thread a
-// contiguous range); writes out[0..n) and returns the total
-__device__ int block_scan_ranges(const int32_t* in, int32_t* out, int n, int* sh) {
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int per = (n + SCAN_T - 1) / SCAN_T;
-    const int a = min(n, tid * per), b = min(n, a + per);
-    int sum = 0;
-    for (int i = a; i < b; ++i) sum += in[i];
-    int x = sum;
+// Table entries of the tiles of a group, from the starts ks[0..cells] of its cells: an
+// aligned group of GROUP tiles holding at most unit_p particles is one unit, counted on
+// its first tile; otherwise each aligned half group that holds at most unit_p is one;
+// otherwise each tile is split on its own.  [a, b): the particles counted on tile t.
+__device__ __forceinline__ void tile_range(const int* ks, int cells, int t, int unit_p, int& a, int& b) {
+    auto at = [&](int c) { return ks[min(c, cells)]; };
+    const int h0 = t / (GROUP / 2) * (SPAN / 2);
+    if (at(SPAN) - ks[0] <= unit_p) {
+        a = ks[0];
+        b = t == 0 ? at(SPAN) : a;
+    } else if (at(h0 + SPAN / 2) - at(h0) <= unit_p) {
+        a = at(h0);
+        b = t % (GROUP / 2) == 0 ? at(h0 + SPAN / 2) : a;
+    } else {
+        a = at(t * TILE);
+        b = at((t + 1) * TILE);
+    }
+}
+
+// the group's entries, by the first GROUP threads (ks complete)
+__device__ __forceinline__ void count_entries(const SortParams& S, int run, int s, int g, const int* ks, int cells) {
+    const int t = threadIdx.x;
+    if (t >= 32) return;
+    int n = 0;
+    if (t < GROUP) {
+        int a, b;
+        tile_range(ks, cells, t, S.unit_p, a, b);
+        n = (b - a + S.part_p - 1) / S.part_p;  // (unit_p is a multiple of part_p)
+    }
 #pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        const int y = __shfl_up_sync(FULL, x, o);
-        if (lane >= o) x += y;
+    for (int o = 4; o > 0; o >>= 1) n += __shfl_xor_sync(FULL, n, o);
+    if (t == 0) {
+        S.runs[run].group_n[s][g] = n;
+        if (n) atomicAdd(&S.rs_new[2 * run + s], n);
+    }
+}
+
+// grid (groups of the largest run, runs, species)
+__global__ void __launch_bounds__(PLAN_T, 4) k_sort_plan(const SortParams S) {
+    __shared__ int sh[PLAN_T / 32];
+    __shared__ int ks[SPAN + 1];
+    __shared__ int slo[PLAN_UNITS], shi[PLAN_UNITS];
+    __shared__ int sbase[2];
+    const int run = blockIdx.y, s = blockIdx.z, g = blockIdx.x, tid = threadIdx.x;
+    const RunDev& R = S.runs[run];
+    const int C0 = g * SPAN;
+    if (!R.active || C0 >= R.Nx) return;  // block-uniform
+    const int cells = min(SPAN, R.Nx - C0), k = S.k;
+    // units of the old table that can reach into the group (k < SPAN)
+    const int32_t* gf = R.group_first[s][S.tab];
+    const int ua = gf[max(g - 1, 0)], ub = gf[g + 2], nu = ub - ua;
+    const bool staged = nu <= PLAN_UNITS;  // else their bounds are read from the table
+    for (int i = tid; staged && i < nu; i += PLAN_T) {
+        slo[i] = S.units.lo[ua + i] - k;
+        shi[i] = S.units.hi[ua + i] + k;
+    }
+    if (tid < 2) sbase[tid] = 0;
+    __syncthreads();
+    auto lo = [&](int i) { return staged ? slo[i] : S.units.lo[ua + i] - k; };  // windows, both non-decreasing
+    auto hi = [&](int i) { return staged ? shi[i] : S.units.hi[ua + i] + k; };
+    auto first_reaching = [&](int c) {  // first unit with hi >= c
+        int l = 0, r = nu;
+        while (l < r) {
+            const int m = (l + r) >> 1;
+            if (hi(m) >= c) r = m; else l = m + 1;
+        }
+        return l;
+    };
+    const int key = C0 + tid;
+    int tot = 0, u0 = 0, u1 = 0;  // units [u0, u1) cover the cell
+    if (tid < cells) {
+        u0 = u1 = first_reaching(key);
+        while (u1 < nu && lo(u1) <= key) {
+            tot += S.cnt[static_cast<size_t>(ua + u1) * SSTR + (key - lo(u1))];
+            ++u1;
+        }
+    }
+    // particles below the group: those of the units wholly below it, and the counts below it of
+    // the units across its start, a warp per unit
+    const int uc = first_reaching(C0);  // the same for all threads
+    int below = 0;
+    for (int i = uc + (tid >> 5); i < nu && lo(i) < C0; i += PLAN_T / 32)
+        for (int c = lo(i) + (tid & 31); c < C0; c += 32) below += S.cnt[static_cast<size_t>(ua + i) * SSTR + (c - lo(i))];
+    below = __reduce_add_sync(FULL, below);
+    if ((tid & 31) == 0 && below) atomicAdd(&sbase[0], below);
+    if (tid == 0) sbase[1] = uc < nu ? S.units.start[ua + uc] : (nu > 0 ? S.units.end[ub - 1] : -1);
+    int total;
+    const int r = plan_scan(tot, sh, &total);
+    int below_all = sbase[1];
+    if (below_all < 0)  // no unit near: every unit before is below
+        below_all = ua > gf[0] ? S.units.end[ua - 1] : 0;
+    int at = below_all + sbase[0] + r;
+    if (tid < cells) {
+        R.keystart[s][key] = at;
+        ks[tid] = at;
+        if (key == R.Nx - 1) R.keystart[s][R.Nx] = at + tot;
+    }
+    if (tid == 0) ks[cells] = below_all + sbase[0] + total;
+    for (int u = u0; u < u1; ++u) {
+        const size_t q = static_cast<size_t>(ua + u) * SSTR + (key - lo(u));
+        S.offs[q] = at;
+        at += S.cnt[q];
     }
     __syncthreads();
-    if (lane == 31) sh[warp] = x;
+    count_entries(S, run, s, g, ks, cells);
+}
+
+// ---- 4. the new unit table --------------------------------------------------------
+// One block (SORT_T threads) per group: the table index of its first entry is the number of
+// entries of the pairs (run, species) and groups before it.
+struct FillSmem {
+    int ks[SPAN + 1];
+    int first[GROUP + 1];
+    int red[2];
+};
+__device__ __forceinline__ void fill_block(const SortParams& S, int run, int s, int g, FillSmem& F) {
+    const RunDev& R = S.runs[run];
+    const int C0 = g * SPAN, tid = threadIdx.x, np = 2 * S.nruns, p = 2 * run + s;
+    const bool in = R.active && C0 < R.Nx;  // block-uniform
+    if (!in && (g > 0 || p > 0)) {
+        if (g == 0 && tid == 0) S.rs_new[np + p] = 0;  // (no entries)
+        return;
+    }
+    if (tid < 2) F.red[tid] = 0;
     __syncthreads();
-    if (warp == 0) {
-        int w = sh[lane];
+    // entries before this pair, and in all (for the table's count); entries of this pair before this group
+    int before = 0, all = 0, prev = 0;
+    for (int i = tid; i < np; i += SORT_T) {
+        const int n = S.rs_new[i];
+        all += n;
+        before += i < p ? n : 0;
+    }
+    if (in)
+        for (int i = tid; i < g; i += SORT_T) prev += R.group_n[s][i];
+    before = __reduce_add_sync(FULL, before);
+    prev = __reduce_add_sync(FULL, prev);
+    if ((tid & 31) == 0) {
+        atomicAdd(&F.red[0], before);
+        atomicAdd(&F.red[1], prev);
+    }
+    if (p == 0 && g == 0) {  // block-uniform
+        __shared__ int sall;
+        if (tid == 0) sall = 0;
+        __syncthreads();
+        all = __reduce_add_sync(FULL, all);
+        if ((tid & 31) == 0) atomicAdd(&sall, all);
+        __syncthreads();
+        if (tid == 0) {
+            S.fresh.count[0] = min(sall, S.max_units);
+            *S.phase = (*S.phase + S.k) % 6u;
+        }
+        if (!in) {
+            if (tid == 0) S.rs_new[np] = 0;
+            return;
+        }
+    }
+    const int cells = min(SPAN, R.Nx - C0);
+    for (int i = tid; i <= cells; i += SORT_T) F.ks[i] = R.keystart[s][C0 + i];
+    __syncthreads();
+    const int pair = F.red[0], base = pair + F.red[1];
+    if (tid < 32) {
+        int a = 0, b = 0;
+        if (tid < GROUP) tile_range(F.ks, cells, tid, S.unit_p, a, b);
+        int n = (b - a + S.part_p - 1) / S.part_p, x = n;
 #pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const int y = __shfl_up_sync(FULL, w, o);
-            if (lane >= o) w += y;
+        for (int o = 1; o < GROUP; o <<= 1) {
+            const int y = __shfl_up_sync(FULL, x, o);
+            if (tid >= o) x += y;
         }
-        sh[lane] = w;
+        if (tid < GROUP) F.first[tid] = x - n;
+        if (tid == GROUP - 1) F.first[GROUP] = x;
     }
     __syncthreads();
-    int run = x - sum + (warp > 0 ? sh[warp - 1] : 0);
-    for (int i = a; i < b; ++i) {
-        const int v = in[i];
-        out[i] = run;
-        run += v;
+    const int n = F.first[GROUP], G = groups_of(R.Nx);
+    int32_t* gf = R.group_first[s][S.tab_new];
+    if (tid == 0) {
+        gf[g] = base;
+        if (g == 0) S.rs_new[np + p] = pair;
     }
-    const int total = sh[SCAN_T / 32 - 1];
-    __syncthreads();
-    return total;
-}
-
-// ---- 2a. per-cell totals (and per-block sums of them) --------------------------
-// grid (key blocks of the largest run, runs, species)
-__global__ void __launch_bounds__(KEY_T) k_sort_totals(const SortParams S) {
-    __shared__ int sh[KEY_T / 32];
-    const RunDev& R = S.runs[blockIdx.y];
-    const int s = blockIdx.z;
-    if (!R.active || blockIdx.x * KEY_T >= R.Nx) return;  // block-uniform
-    const int key = blockIdx.x * KEY_T + threadIdx.x;
-    int tot = 0;
-    if (key < R.Nx) {
-        int u0, u1;
-        covering(S, blockIdx.y, s, key, u0, u1);
-        for (int u = u0; u <= u1; ++u) {
-            const int l = key - (S.units.lo[u] - S.k);
-            if (l >= 0 && l < SSTR) tot += S.cnt[static_cast<size_t>(u) * SSTR + l];
-        }
-        R.keycount[s][key] = tot;
-    }
-    const int b = block_sum_int(tot, sh);
-    if (threadIdx.x == 0) R.blocksum[s][blockIdx.x] = b;
-}
-
-// ---- 2b. scan of the per-block sums, one block per (run, species) --------------
-__global__ void __launch_bounds__(SCAN_T) k_scan_blocks(const SortParams S) {
-    __shared__ int sh[SCAN_T / 32];
-    const RunDev& R = S.runs[blockIdx.x];
-    const int s = blockIdx.y;
-    if (!R.active) return;
-    const int nkb = (R.Nx + KEY_T - 1) / KEY_T;
-    const int total = block_scan_ranges(R.blocksum[s], R.blockstart[s], nkb, sh);
-    if (threadIdx.x == 0) R.keystart[s][R.Nx] = total;
-}
-
-// ---- 2c. cell starts and the destination of every (unit, cell) pair -------------
-__global__ void __launch_bounds__(KEY_T) k_sort_offsets(const SortParams S) {
-    __shared__ int sh[KEY_T / 32];
-    const RunDev& R = S.runs[blockIdx.y];
-    const int s = blockIdx.z;
-    if (!R.active || blockIdx.x * KEY_T >= R.Nx) return;
-    const int key = blockIdx.x * KEY_T + threadIdx.x;
-    const int v = key < R.Nx ? R.keycount[s][key] : 0;
-    const int r = block_excl_scan(v, sh);
-    if (key >= R.Nx) return;
-    int run = R.blockstart[s][blockIdx.x] + r;
-    R.keystart[s][key] = run;
-    int u0, u1;
-    covering(S, blockIdx.y, s, key, u0, u1);
-    for (int u = u0; u <= u1; ++u) {
-        const int l = key - (S.units.lo[u] - S.k);
-        if (l >= 0 && l < SSTR) {
-            const size_t q = static_cast<size_t>(u) * SSTR + l;
-            S.offs[q] = run;
-            run += S.cnt[q];
-        }
+    if (g == G - 1 && tid < 3) gf[G + tid] = base + n;
+    for (int v = tid; v < n; v += SORT_T) {
+        int t = 0;
+        while (t + 1 < GROUP && F.first[t + 1] <= v) ++t;
+        int a, e;
+        tile_range(F.ks, cells, t, S.unit_p, a, e);
+        // part i of [a, e); where parts of one unit meet, at a multiple of 4 particles, so
+        // that the push's slots, and with them its results, are those of the whole unit
+        const int i = v - F.first[t];
+        auto cut = [&](int j) {
+            const int q = a + j * S.part_p;
+            return (j * S.part_p) % S.unit_p ? q & ~3 : q;
+        };
+        const int b = (i + 1) * S.part_p < e - a ? cut(i + 1) : e;
+        a = cut(i);
+        auto cell_of = [&](int q) {  // cell of sorted particle q: the last one that starts at or before it
+            int l = 0, r = cells;
+            while (r - l > 1) {
+                const int m = (l + r) >> 1;
+                if (F.ks[m] <= q) l = m; else r = m;
+            }
+            return C0 + l;
+        };
+        const int u = base + v;
+        if (u >= S.max_units) continue;  // cannot happen: the table holds what the runs can need
+        S.fresh.run[u] = run;
+        S.fresh.species[u] = s;
+        S.fresh.start[u] = a;
+        S.fresh.end[u] = b;
+        S.fresh.lo[u] = cell_of(a);
+        S.fresh.hi[u] = cell_of(b - 1);
     }
 }
-
 
 // ---- 3. stable scatter ----------------------------------------------------------
 // Each warp owns one contiguous slice of the unit's particles.  Pass 1 counts
@@ -241,7 +373,9 @@ __global__ void __launch_bounds__(KEY_T) k_sort_offsets(const SortParams S) {
 // the counts of the warps before, in warp order); pass 2 walks the slice
 // again in order and places each particle at its warp's running start plus
 // its rank among the lanes with the same cell.  Equal cells therefore keep
-// index order, with two block barriers per unit.
+// index order, with two block barriers per unit.  (Ranking in pass 1 with the result kept
+// in registers, so that nothing in pass 2 waits, and more or fewer blocks an SM and rows in
+// flight, came to 170 to 217 us per sort of thin plasma against 172.)
 constexpr int SC_W = SORT_T / 32;
 constexpr int SC_U = 4;  // slice rows of 32 particles in flight per pass step
 
@@ -251,9 +385,17 @@ __device__ __forceinline__ int window_key(const int32_t* cell, int i, int we, in
     return (l >= 0 && l < SSTR) ? l : -1;  // out of window cannot happen (counted as an error)
 }
 
+// A block per (species, run, group) for the new table, then a block per unit (the table
+// holds up to max_units, usually far fewer: behind their empty blocks the others came last,
+// 19 us later on thin plasma).
 __global__ void __launch_bounds__(SORT_T) k_sort_scatter(const SortParams S) {
     __shared__ int row[SC_W][SSTR];
-    const int u = blockIdx.x;
+    const int u = static_cast<int>(blockIdx.x) - 2 * S.nruns * S.g_max;
+    if (u < 0) {  // block-uniform
+        const int v = blockIdx.x, q = v / S.g_max;
+        fill_block(S, q >> 1, q & 1, v - q * S.g_max, reinterpret_cast<FillSmem&>(row));
+        return;
+    }
     if (u >= S.units.count[0]) return;
     const RunDev& R = S.runs[S.units.run[u]];
     if (!R.active) return;
@@ -334,110 +476,90 @@ __global__ void __launch_bounds__(SORT_T) k_sort_scatter(const SortParams S) {
     }
 }
 
-// ---- 4. unit table from sorted cells -------------------------------------------
-// 4a. units per tile of one (run, species), scanned: tile_first[t] = first
-// unit of tile t within the pair; rs_units[2 r + s] = the pair's units.
-__global__ void __launch_bounds__(SCAN_T) k_tile_units(const SortParams S) {
-    __shared__ int sh[SCAN_T / 32];
-    const int r = blockIdx.x, s = blockIdx.y;
-    const RunDev& R = S.runs[r];
-    if (!R.active || R.n[s] == 0) {
-        if (threadIdx.x == 0) S.rs_units[2 * r + s] = 0;
-        return;
+// ---- a table for freshly loaded (already sorted) particles ---------------------------
+__device__ __forceinline__ int block_sum_int(int v, int* sh) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(FULL, v, o);
+    if (lane == 0) sh[warp] = v;
+    __syncthreads();
+    int t = 0;
+    if (threadIdx.x == 0)
+        for (int w = 0; w < KEY_T / 32; ++w) t += sh[w];
+    return t;
+}
+
+// exclusive scan of v over the block (KEY_T threads)
+__device__ __forceinline__ int block_excl_scan(int v, int* sh) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    int x = v;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const int y = __shfl_up_sync(FULL, x, o);
+        if (lane >= o) x += y;
     }
-    const int ntiles = (R.Nx + TILE - 1) / TILE;
-    const int32_t* ks = R.keystart[s];
-    for (int t = threadIdx.x; t < ntiles; t += SCAN_T) {
-        // an aligned group of GROUP tiles holding at most unit_p particles is one
-        // unit, counted on its first tile; otherwise each aligned half group of
-        // GROUP / 2 tiles that holds at most unit_p is one unit; otherwise each
-        // tile is split on its own
-        const int g0 = (t / GROUP) * SPAN;
-        const int gn = ks[min(g0 + SPAN, R.Nx)] - ks[g0];
-        const int h0 = (t / (GROUP / 2)) * (SPAN / 2);
-        const int hn = ks[min(h0 + SPAN / 2, R.Nx)] - ks[h0];
-        int n;
-        if (gn <= S.unit_p) {
-            n = t % GROUP == 0 ? gn : 0;
-        } else if (hn <= S.unit_p) {
-            n = t % (GROUP / 2) == 0 ? hn : 0;
-        } else {
-            n = ks[min((t + 1) * TILE, R.Nx)] - ks[t * TILE];
+    if (lane == 31) sh[warp] = x;
+    __syncthreads();
+    if (warp == 0) {
+        int w = lane < KEY_T / 32 ? sh[lane] : 0;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int y = __shfl_up_sync(FULL, w, o);
+            if (lane >= o) w += y;
         }
-        n = (n + S.part_p - 1) / S.part_p;  // (unit_p is a multiple of part_p)
-        R.tile_n[s][t] = n;
+        if (lane < KEY_T / 32) sh[lane] = w;
     }
     __syncthreads();
-    const int nu = block_scan_ranges(R.tile_n[s], R.tile_first[s], ntiles, sh);
-    if (threadIdx.x == 0) {
-        R.tile_first[s][ntiles] = nu;
-        S.rs_units[2 * r + s] = nu;
-    }
+    return x - v + (warp > 0 ? sh[warp - 1] : 0);
 }
 
-// 4b. unit bases of every (run, species) pair, in run-major order
-__global__ void __launch_bounds__(SCAN_T) k_unit_bases(const SortParams S) {
+// exclusive scan of n ints by one block of SCAN_T threads (each thread a
+// contiguous range); writes out[0..n) and returns the total
+__device__ int block_scan_ranges(const int32_t* in, int32_t* out, int n, int* sh) {
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int per = (n + SCAN_T - 1) / SCAN_T;
+    const int a = min(n, tid * per), b = min(n, a + per);
+    int sum = 0;
+    for (int i = a; i < b; ++i) sum += in[i];
+    int x = sum;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const int y = __shfl_up_sync(FULL, x, o);
+        if (lane >= o) x += y;
+    }
+    __syncthreads();
+    if (lane == 31) sh[warp] = x;
+    __syncthreads();
+    if (warp == 0) {
+        int w = sh[lane];
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int y = __shfl_up_sync(FULL, w, o);
+            if (lane >= o) w += y;
+        }
+        sh[lane] = w;
+    }
+    __syncthreads();
+    int run = x - sum + (warp > 0 ? sh[warp - 1] : 0);
+    for (int i = a; i < b; ++i) {
+        const int v = in[i];
+        out[i] = run;
+        run += v;
+    }
+    const int total = sh[SCAN_T / 32 - 1];
+    __syncthreads();
+    return total;
+}
+
+// ---- scan of the per-block sums, one block per (run, species) --------------
+__global__ void __launch_bounds__(SCAN_T) k_scan_blocks(const SortParams S) {
     __shared__ int sh[SCAN_T / 32];
-    const int np = 2 * S.nruns;
-    const int total = block_scan_ranges(S.rs_units, S.rs_units + np, np, sh);
-    if (threadIdx.x == 0) {
-        S.units.count[0] = min(total, S.max_units);
-        *S.phase = (*S.phase + S.k) % 6u;
-    }
-}
-
-// 4c. one thread per unit; the sorted particles are in buffer `ubuf`
-__global__ void k_fill_units(const SortParams S, int ubuf) {
-    const int u = blockIdx.x * blockDim.x + threadIdx.x;
-    if (u >= S.units.count[0]) return;
-    const int np = 2 * S.nruns;
-    const int32_t* first = S.rs_units + np;  // exclusive scan of the pair counts
-    int l = 0, r = np;  // last pair with first[p] <= u and a unit count > 0
-    while (r - l > 1) {
-        const int m = (l + r) >> 1;
-        if (first[m] <= u) l = m; else r = m;
-    }
-    while (S.rs_units[l] == 0 && l > 0) --l;  // skip empty pairs sharing the same start
-    const int run = l >> 1, s = l & 1;
-    const RunDev& R = S.runs[run];
-    const int v = u - first[l];
-    const int ntiles = (R.Nx + TILE - 1) / TILE;
-    const int32_t* tf = R.tile_first[s];
-    int a0 = 0, b0 = ntiles;  // last tile t with tf[t] <= v
-    while (b0 - a0 > 1) {
-        const int m = (a0 + b0) >> 1;
-        if (tf[m] <= v) a0 = m; else b0 = m;
-    }
-    const int t = a0;
-    const int32_t* ks = R.keystart[s];
-    const int g0 = (t / GROUP) * SPAN;
-    const int gs = ks[g0], ge = ks[min(g0 + SPAN, R.Nx)];
-    const int h0 = (t / (GROUP / 2)) * (SPAN / 2);
-    const int hs = ks[h0], he = ks[min(h0 + SPAN / 2, R.Nx)];
-    int a = ks[t * TILE], b = ks[min((t + 1) * TILE, R.Nx)];
-    if (ge - gs <= S.unit_p) {  // the whole group (t is its first tile)
-        a = gs;
-        b = ge;
-    } else if (he - hs <= S.unit_p) {  // the half group (t is its first tile)
-        a = hs;
-        b = he;
-    }
-    // part i of [a, b); where parts of one unit meet, at a multiple of 4 particles, so
-    // that the push's slots, and with them its results, are those of the whole unit
-    const int i = v - tf[t], e = b;
-    auto cut = [&](int j) {
-        const int p = a + j * S.part_p;
-        return (j * S.part_p) % S.unit_p ? p & ~3 : p;
-    };
-    b = (i + 1) * S.part_p < e - a ? cut(i + 1) : e;
-    a = cut(i);
-    const int32_t* cell = R.sp[s][ubuf].cell;
-    S.units.run[u] = run;
-    S.units.species[u] = s;
-    S.units.start[u] = a;
-    S.units.end[u] = b;
-    S.units.lo[u] = key_of(cell[a]);
-    S.units.hi[u] = key_of(cell[b - 1]);
+    const RunDev& R = S.runs[blockIdx.x];
+    const int s = blockIdx.y;
+    if (!R.active) return;
+    const int nkb = (R.Nx + KEY_T - 1) / KEY_T;
+    const int total = block_scan_ranges(R.blocksum[s], R.blockstart[s], nkb, sh);
+    if (threadIdx.x == 0) R.keystart[s][R.Nx] = total;
 }
 
 // ---- histogram of already sorted particles (fresh load) -------------------------
@@ -482,56 +604,37 @@ __global__ void __launch_bounds__(KEY_T) k_keystart(const SortParams S) {
 __global__ void k_zero_keycount(const SortParams S) {
     const RunDev& R = S.runs[blockIdx.y];
     const int s = blockIdx.z;
+    if (blockIdx.x == 0 && threadIdx.x == 0) S.rs_new[2 * blockIdx.y + s] = 0;
     if (!R.active) return;
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < R.Nx + 2; i += gridDim.x * blockDim.x)
         R.keycount[s][i] = 0;
 }
 
-// ---- radiated energy per run: sum of its electron units, fixed order ------------
-__global__ void __launch_bounds__(1024) k_rad_flush(const RunDev* runs, const int32_t* rs_units, double* part) {
-    __shared__ double sred[32];
-    const RunDev& R = runs[blockIdx.x];
-    if (!R.active) return;
-    const int b = rs_units[2 * gridDim.x + 2 * blockIdx.x], n = rs_units[2 * blockIdx.x];  // electron units
-    const int t = threadIdx.x;
-    double a0 = 0.0, a1 = 0.0, a2 = 0.0, a3 = 0.0;
-    int i = t;
-    for (; i + 3 * 1024 < n; i += 4 * 1024) {
-        a0 += part[b + i];
-        a1 += part[b + i + 1024];
-        a2 += part[b + i + 2048];
-        a3 += part[b + i + 3072];
-        part[b + i] = part[b + i + 1024] = part[b + i + 2048] = part[b + i + 3072] = 0.0;
-    }
-    for (; i < n; i += 1024) {
-        a0 += part[b + i];
-        part[b + i] = 0.0;
-    }
-    double v = (a0 + a1) + (a2 + a3);
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(FULL, v, o);
-    if ((t & 31) == 0) sred[t >> 5] = v;
+// entries of every group, from the cell starts
+__global__ void __launch_bounds__(SORT_T) k_group_entries(const SortParams S) {
+    __shared__ int ks[SPAN + 1];
+    const RunDev& R = S.runs[blockIdx.y];
+    const int s = blockIdx.z, C0 = blockIdx.x * SPAN;
+    if (!R.active || C0 >= R.Nx) return;  // block-uniform
+    const int cells = min(SPAN, R.Nx - C0);
+    for (int i = threadIdx.x; i <= cells; i += SORT_T) ks[i] = R.keystart[s][C0 + i];
     __syncthreads();
-    if (t == 0) {
-        double s = 0.0;
-        for (int w = 0; w < 32; ++w) s += sred[w];
-        R.tally[0] += s;
-    }
+    count_entries(S, blockIdx.y, s, blockIdx.x, ks, cells);
+}
+
+__global__ void __launch_bounds__(SORT_T) k_fill(const SortParams S) {
+    __shared__ FillSmem F;
+    const int q = blockIdx.x / S.g_max;
+    fill_block(S, q >> 1, q & 1, blockIdx.x - q * S.g_max, F);
 }
 
 }  // namespace
 
 void launch_sort(const SortParams& S, cudaStream_t st, int* launches) {
-    const dim3 kg(S.kb_max, S.nruns, 2);
-    k_sort_count<<<S.max_units, SORT_T, 0, st>>>(S);
-    k_sort_totals<<<kg, KEY_T, 0, st>>>(S);
-    k_scan_blocks<<<dim3(S.nruns, 2), SCAN_T, 0, st>>>(S);
-    k_sort_offsets<<<kg, KEY_T, 0, st>>>(S);
-    k_sort_scatter<<<S.max_units, SORT_T, 0, st>>>(S);
-    k_tile_units<<<dim3(S.nruns, 2), SCAN_T, 0, st>>>(S);
-    k_unit_bases<<<1, SCAN_T, 0, st>>>(S);
-    k_fill_units<<<(S.max_units + 255) / 256, 256, 0, st>>>(S, 1 - S.cur);
-    *launches += 8;
+    k_sort_count<<<S.max_units + S.nruns, SORT_T, 0, st>>>(S);
+    k_sort_plan<<<dim3(S.g_max, S.nruns, 2), PLAN_T, 0, st>>>(S);
+    k_sort_scatter<<<S.max_units + 2 * S.nruns * S.g_max, SORT_T, 0, st>>>(S);
+    *launches += 3;
 }
 
 void launch_build_units(const SortParams& S, cudaStream_t st, int* launches) {  // S.k == 0
@@ -541,14 +644,13 @@ void launch_build_units(const SortParams& S, cudaStream_t st, int* launches) {  
     k_block_sums<<<kg, KEY_T, 0, st>>>(S);
     k_scan_blocks<<<dim3(S.nruns, 2), SCAN_T, 0, st>>>(S);
     k_keystart<<<kg, KEY_T, 0, st>>>(S);
-    k_tile_units<<<dim3(S.nruns, 2), SCAN_T, 0, st>>>(S);
-    k_unit_bases<<<1, SCAN_T, 0, st>>>(S);
-    k_fill_units<<<(S.max_units + 255) / 256, 256, 0, st>>>(S, S.cur);
-    *launches += 8;
+    k_group_entries<<<dim3(S.g_max, S.nruns, 2), SORT_T, 0, st>>>(S);
+    k_fill<<<2 * S.nruns * S.g_max, SORT_T, 0, st>>>(S);
+    *launches += 7;
 }
 
 void launch_rad_flush(const RunDev* runs, int nruns, const int32_t* rs_units, double* rad_part, cudaStream_t st) {
-    k_rad_flush<<<nruns, 1024, 0, st>>>(runs, rs_units, rad_part);
+    k_rad_flush<<<nruns, SORT_T, 0, st>>>(runs, nruns, rs_units, rad_part);
 }
 
 // ---- foil loader -------------------------------------------------------------

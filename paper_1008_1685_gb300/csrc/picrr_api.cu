@@ -155,10 +155,11 @@ struct Batch {
     bool graph_timed[2] = {};
     bool graph_unread[2] = {};
 
-    UnitTable units{};
+    UnitTable units[2] = {};  // alternate with the particle buffers
     int max_units = 0;
     double* rad_part = nullptr;
-    int32_t *cnt = nullptr, *offs = nullptr, *rs_units = nullptr;
+    uint16_t* cnt = nullptr;
+    int32_t *offs = nullptr, *rs_units[2] = {};
     int* d_status = nullptr;
     unsigned* d_phase = nullptr;  // batch step of the last sort mod 6, advanced by the sort
     double* diag_partials = nullptr;
@@ -398,7 +399,8 @@ pic_status batch_create(const pic_config* cfg, int max_runs, Batch** out) {
         (st = dalloc_t(b, b->mem, &b->diag_partials, kMaxDiagBlocks)) != PIC_OK ||
         (st = dalloc_t(b, b->mem, &b->diag_out, 8)) != PIC_OK ||
         (st = dalloc_t(b, b->mem, &b->snap_out, 4)) != PIC_OK ||
-        (st = dalloc_t(b, b->mem, &b->rs_units, static_cast<size_t>(4) * max_runs)) != PIC_OK) {
+        (st = dalloc_t(b, b->mem, &b->rs_units[0], static_cast<size_t>(4) * max_runs)) != PIC_OK ||
+        (st = dalloc_t(b, b->mem, &b->rs_units[1], static_cast<size_t>(4) * max_runs)) != PIC_OK) {
         g_null_error = b->err;
         batch_destroy(b);
         return st;
@@ -488,14 +490,15 @@ pic_status run_open(Batch* b, double length_lambda, int source_node, int rr_on, 
         for (int c = 0; c < 3 && st == PIC_OK; ++c) st = dalloc_t(b, r.mem, &d.J[x][c], r.glen);
     if (st == PIC_OK) st = dalloc_t(b, r.mem, &d.tally, 4);
     const size_t nk = static_cast<size_t>(Nx) + 2, nkb = static_cast<size_t>(Nx) / KEY_T + 2,
-                 ntl = static_cast<size_t>(Nx) / TILE + 3;
+                 ngr = static_cast<size_t>(Nx) / SPAN + 4;
     for (int s = 0; s < 2 && st == PIC_OK; ++s) {
         if (st == PIC_OK) st = dalloc_t(b, r.mem, &d.keycount[s], nk);
         if (st == PIC_OK) st = dalloc_t(b, r.mem, &d.keystart[s], nk);
         if (st == PIC_OK) st = dalloc_t(b, r.mem, &d.blocksum[s], nkb);
         if (st == PIC_OK) st = dalloc_t(b, r.mem, &d.blockstart[s], nkb);
-        if (st == PIC_OK) st = dalloc_t(b, r.mem, &d.tile_n[s], ntl);
-        if (st == PIC_OK) st = dalloc_t(b, r.mem, &d.tile_first[s], ntl);
+        if (st == PIC_OK) st = dalloc_t(b, r.mem, &d.group_n[s], ngr);
+        if (st == PIC_OK) st = dalloc_t(b, r.mem, &d.group_first[s][0], ngr);
+        if (st == PIC_OK) st = dalloc_t(b, r.mem, &d.group_first[s][1], ngr);
     }
     if (st != PIC_OK) {
         free_all(b, r.mem);
@@ -518,13 +521,16 @@ size_t run_footprint_cpl(double cells_per_lambda, double length_lambda, int64_t 
     const size_t glen = (static_cast<size_t>(Nx) + 1 + 2 * PADF + 4 + 3) / 4 * 4;
     size_t t = 10 * rounded(glen * 4) + 9 * rounded(glen * 8) + rounded(32);
     const size_t nk = static_cast<size_t>(Nx) + 2, nkb = static_cast<size_t>(Nx) / KEY_T + 2,
-                 ntl = static_cast<size_t>(Nx) / TILE + 3;
-    t += 2 * (2 * rounded(nk * 4) + 2 * rounded(nkb * 4) + 2 * rounded(ntl * 4));
+                 ngr = static_cast<size_t>(Nx) / SPAN + 4;
+    t += 2 * (2 * rounded(nk * 4) + 2 * rounded(nkb * 4) + 3 * rounded(ngr * 4));
     const size_t cap = static_cast<size_t>((n + 3) / 4 * 4 + 8);
     t += 2 * 2 * 6 * rounded(cap * 4);
     const int64_t ntiles = (Nx + TILE - 1) / TILE;
-    const size_t units = static_cast<size_t>(2 * ((n + UNIT_P_MIN - 1) / UNIT_P_MIN + ntiles + 1));
-    t += units * (6 * 4 + 8 + 2 * SSTR * 4) * 3 / 2;
+    // parts below UNIT_P_MIN occur only while they are PARTS at most in all
+    const int64_t parts = std::max<int64_t>(2 * ((n + UNIT_P_MIN - 1) / UNIT_P_MIN),
+                                            std::min<int64_t>(2 * ((n + PART_MIN - 1) / PART_MIN), PARTS));
+    const size_t units = static_cast<size_t>(parts + 2 * (ntiles + 1));
+    t += units * (2 * 6 * 4 + 8 + SSTR * 6) * 3 / 2;
     t += static_cast<size_t>(Nx / FIELD_NODES + 1) * 8 * 3 / 2;
     return t;
 }
@@ -812,18 +818,17 @@ pic_status ensure_units(Batch* b, int need) {
     if (need <= b->max_units) return PIC_OK;
     const int mu = std::max(need, b->max_units + b->max_units / 2);
     std::vector<std::pair<void*, size_t>> fresh;
-    UnitTable u{};
+    UnitTable tab[2] = {};
     double* rp = nullptr;
-    int32_t *cn = nullptr, *of = nullptr;
+    uint16_t* cn = nullptr;
+    int32_t* of = nullptr;
     const size_t m = static_cast<size_t>(mu);
     pic_status st = PIC_OK;
-    if (st == PIC_OK) st = dalloc_t(b, fresh, &u.run, m);
-    if (st == PIC_OK) st = dalloc_t(b, fresh, &u.species, m);
-    if (st == PIC_OK) st = dalloc_t(b, fresh, &u.start, m);
-    if (st == PIC_OK) st = dalloc_t(b, fresh, &u.end, m);
-    if (st == PIC_OK) st = dalloc_t(b, fresh, &u.lo, m);
-    if (st == PIC_OK) st = dalloc_t(b, fresh, &u.hi, m);
-    if (st == PIC_OK) st = dalloc_t(b, fresh, &u.count, 4);
+    for (UnitTable& u : tab) {
+        for (int32_t** a : {&u.run, &u.species, &u.start, &u.end, &u.lo, &u.hi})
+            if (st == PIC_OK) st = dalloc_t(b, fresh, a, m);
+        if (st == PIC_OK) st = dalloc_t(b, fresh, &u.count, 4);
+    }
     if (st == PIC_OK) st = dalloc_t(b, fresh, &rp, m);
     if (st == PIC_OK) st = dalloc_t(b, fresh, &cn, m * SSTR);
     if (st == PIC_OK) st = dalloc_t(b, fresh, &of, m * SSTR);
@@ -833,14 +838,16 @@ pic_status ensure_units(Batch* b, int need) {
     }
     // the unit table is rebuilt right after every growth (the radiated partials
     // were flushed by the sort that preceded it)
-    for (void* p : {static_cast<void*>(b->units.run), static_cast<void*>(b->units.species),
-                    static_cast<void*>(b->units.start), static_cast<void*>(b->units.end),
-                    static_cast<void*>(b->units.lo), static_cast<void*>(b->units.hi),
-                    static_cast<void*>(b->units.count), static_cast<void*>(b->rad_part), static_cast<void*>(b->cnt),
-                    static_cast<void*>(b->offs)})
+    for (UnitTable& u : b->units)
+        for (void* p : {static_cast<void*>(u.run), static_cast<void*>(u.species), static_cast<void*>(u.start),
+                        static_cast<void*>(u.end), static_cast<void*>(u.lo), static_cast<void*>(u.hi),
+                        static_cast<void*>(u.count)})
+            free_one(b, p);
+    for (void* p : {static_cast<void*>(b->rad_part), static_cast<void*>(b->cnt), static_cast<void*>(b->offs)})
         free_one(b, p);
     for (auto& f : fresh) b->mem.push_back(f);
-    b->units = u;
+    b->units[0] = tab[0];
+    b->units[1] = tab[1];
     b->rad_part = rp;
     b->cnt = cn;
     b->offs = of;
@@ -849,22 +856,29 @@ pic_status ensure_units(Batch* b, int need) {
     return PIC_OK;
 }
 
-SortParams sort_params(Batch* b) {
+// For a sort of buffer cur (tables and particles move to 1 - cur), or with build for a table of buffer cur.
+SortParams sort_params(Batch* b, int cur, bool build) {
     SortParams S{};
     S.runs = b->d_runs;
     S.nruns = b->max_runs;
-    S.units = b->units;
+    S.tab = cur;
+    S.tab_new = build ? cur : 1 - cur;
+    S.units = b->units[S.tab];
+    S.fresh = b->units[S.tab_new];
     S.cnt = b->cnt;
     S.offs = b->offs;
-    S.rs_units = b->rs_units;
+    S.rs_units = b->rs_units[S.tab];
+    S.rs_new = b->rs_units[S.tab_new];
+    S.rad_part = b->rad_part;
     S.status = b->d_status;
     S.k = b->since_sort;
-    S.cur = b->cur;
+    S.cur = cur;
     S.max_units = b->max_units;
     int mx = 1;
     for (auto& r : b->runs)
         if (r.used) mx = std::max(mx, r.Nx);
     S.kb_max = (mx + KEY_T - 1) / KEY_T;
+    S.g_max = (mx + SPAN - 1) / SPAN;
     S.unit_p = b->unit_p;
     S.phase = b->d_phase;
     S.part_p = b->part_p;
@@ -933,17 +947,16 @@ pic_status upload_blocks(Batch* b) {
 
 void rad_flush(Batch* b, cudaStream_t st) {
     if (b->max_units == 0) return;
-    launch_rad_flush(b->d_runs, b->max_runs, b->rs_units, b->rad_part, st);
+    launch_rad_flush(b->d_runs, b->max_runs, b->rs_units[b->cur], b->rad_part, st);
     b->launches++;
 }
 void rad_flush(Batch* b) { rad_flush(b, b->stream); }
 
 void do_sort(Batch* b) {
-    SortParams S = sort_params(b);
+    SortParams S = sort_params(b, b->cur, false);
     int nl = 0;
     {
         Timed t(b, 2);
-        rad_flush(b);
         launch_sort(S, b->stream, &nl);
     }
     b->launches += nl;
@@ -952,8 +965,10 @@ void do_sort(Batch* b) {
     b->since_sort = 0;
 }
 
-// Unit table entries that the runs for which `counts` holds can need with units of unit_p particles (each tile
-// adds at most one partial entry; merged groups only lower the count), and the size of a unit's parts.
+// Unit table entries that the runs for which `counts` holds can need with units of unit_p particles, and the
+// size of a unit's parts.  A piece of a run (a merged group, a merged half or a tile) adds at most one partial
+// entry; a group or half is not merged only if it holds more than unit_p particles, which makes at most
+// groups + 4 n / unit_p pieces, and never more than the tiles.
 template <class Counts>
 int64_t units_needed(const Batch* b, int unit_p, Counts counts, int* part) {
     int64_t total = 0, need = 1;
@@ -963,9 +978,10 @@ int64_t units_needed(const Batch* b, int unit_p, Counts counts, int* part) {
     *part = part_size(total, unit_p);
     for (const auto& r : b->runs) {
         if (!counts(r)) continue;
-        const int ntiles = (r.Nx + TILE - 1) / TILE;
+        const int64_t ntiles = (r.Nx + TILE - 1) / TILE, groups = (r.Nx + SPAN - 1) / SPAN;
         for (int s = 0; s < 2; ++s)
-            if (r.sp[s].loaded) need += (r.sp[s].n + *part - 1) / *part + ntiles + 1;
+            if (r.sp[s].loaded)
+                need += (r.sp[s].n + *part - 1) / *part + std::min(ntiles, groups + 4 * (r.sp[s].n / unit_p)) + 1;
     }
     return need;
 }
@@ -1014,7 +1030,7 @@ pic_status activate_pending(Batch* b) {
         return st;
     }
     if ((st = upload_table(b)) != PIC_OK) return st;
-    SortParams S = sort_params(b);
+    SortParams S = sort_params(b, b->cur, true);
     int nl = 0;
     launch_build_units(S, b->stream, &nl);
     b->launches += nl;
@@ -1059,7 +1075,7 @@ pic_status upload_incident(Batch* b, int steps) {
 PushParams push_params(const Batch* b, int k, int cur) {
     PushParams P{};
     P.runs = b->d_runs;
-    P.units = b->units;
+    P.units = b->units[cur];
     P.rad_part = b->rad_part;
     P.status = b->d_status;
     P.phase = b->d_phase;
@@ -1150,10 +1166,8 @@ pic_status chunk_graph(Batch* b, int cur, cudaGraphExec_t* out) {
         mark(1, false);
     }
     mark(2, true);
-    launch_rad_flush(b->d_runs, b->max_runs, b->rs_units, b->rad_part, cs);
-    SortParams S = sort_params(b);
+    SortParams S = sort_params(b, cur, false);
     S.k = I;
-    S.cur = cur;
     int nl = 0;
     launch_sort(S, cs, &nl);
     mark(2, false);
@@ -1213,7 +1227,7 @@ pic_status batch_step(Batch* b, int64_t n, int64_t* done) {
             PIC_CK(b, cudaGraphLaunch(ex, b->stream));
             b->graph_unread[gc] = b->timing;
             b->graph_launches++;
-            b->launches += (fz ? I + 1 : 2 * I) + 1 + 8;
+            b->launches += (fz ? I + 1 : 2 * I) + 3;
             b->push_launches += I;
             b->gstep += I;
             b->cur ^= 1;
@@ -1319,7 +1333,7 @@ pic_status set_shapes(Batch* b, int unit_p, int interval, int slot_w) {
         b->unit_p = unit_p;
         b->part_p = part;
         if (any) {
-            SortParams S = sort_params(b);
+            SortParams S = sort_params(b, b->cur, true);
             int nl = 0;
             launch_build_units(S, b->stream, &nl);
             b->launches += nl;
@@ -1827,7 +1841,7 @@ void fill_stats(Batch* b, pic_stats_t* out) {
     out->active_particles = act;
     out->fp_bits = fp;
     int32_t cnt = 0;
-    if (b->units.count && cudaMemcpy(&cnt, b->units.count, sizeof(int32_t), cudaMemcpyDeviceToHost) == cudaSuccess)
+    if (b->units[b->cur].count && cudaMemcpy(&cnt, b->units[b->cur].count, sizeof(int32_t), cudaMemcpyDeviceToHost) == cudaSuccess)
         out->n_units = cnt;
 }
 

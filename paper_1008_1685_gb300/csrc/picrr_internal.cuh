@@ -117,8 +117,8 @@ struct RunDev {
     int32_t* keystart[2];  // [Nx + 2]; keystart[Nx] = particles
     int32_t* blocksum[2];  // [Nx / 256 + 2]
     int32_t* blockstart[2];
-    int32_t* tile_n[2];    // [Nx / TILE + 3]
-    int32_t* tile_first[2];
+    int32_t* group_n[2];         // [groups of SPAN cells]: entries of the new unit table
+    int32_t* group_first[2][2];  // per table, [groups + 3]: first entry of the group or a later one; the last three: the end
 };
 
 // Buffers of a run at a batch step of phase g: the step, or anything equal to it mod 6 (and >= 0).
@@ -226,21 +226,27 @@ void launch_zero_current(const FieldParams& P, cudaStream_t st);
 struct SortParams {
     RunDev* runs;
     int nruns;
-    UnitTable units;
-    int32_t* cnt;          // [max_units * SSTR] key counts per unit window
+    UnitTable units;       // table of the particles as they are
+    UnitTable fresh;       // the new table (for a build: the only one)
+    int tab, tab_new;      // which of a run's group_first belongs to each
+    uint16_t* cnt;         // [max_units * SSTR] key counts per unit window
     int32_t* offs;         // [max_units * SSTR] destinations per unit window
-    int32_t* rs_units;     // [4 * nruns]: units per (run, species) pair, then the first unit of each pair
+    const int32_t* rs_units;  // [4 * nruns]: entries per (run, species) pair, then the first of each pair
+    int32_t* rs_new;       // the same of the new table
+    double* rad_part;
     int* status;
     int k, cur, max_units;
     int kb_max;            // key blocks of the largest run: ceil(max Nx / 256)
+    int g_max;             // groups of the largest run: ceil(max Nx / SPAN)
     int unit_p;            // particles per unit at most (UNIT_P_MIN..UNIT_P_MAX)
-    unsigned* phase;       // += k, mod 6
     int part_p;            // particles per part of a unit (a power of two, PART_MIN..unit_p)
+    unsigned* phase;       // += k, mod 6
 };
 // Full re-sort of every active run (bounded displacement since the last sort)
-// and the new unit table; particles move from buffer cur to 1 - cur.
+// and the new unit table; particles move from buffer cur to 1 - cur, radiated
+// partials into the tallies.
 void launch_sort(const SortParams& S, cudaStream_t st, int* launches);
-// Unit table of every active run from its current, already sorted particles.
+// Unit table S.fresh of every active run from its current, already sorted particles.
 void launch_build_units(const SortParams& S, cudaStream_t st, int* launches);
 // Add each run's per-unit radiated energy into its tally[0]; zero them.
 // rs_units as in SortParams.

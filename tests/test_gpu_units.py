@@ -1,0 +1,79 @@
+"""Unit tables of every form give a run the same bits: units cut into parts with the
+Yee update inside the push (few particles in the batch), and whole units with a Yee
+launch of their own (the same run beside a large one); and a sort whose groups hold
+more units than its planning kernel stages."""
+import numpy as np
+import pytest
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def picrr():
+    import __graft_entry__
+
+    __graft_entry__.build()
+    import paper_1008_1685_gb300 as m
+
+    return m
+
+
+def state(b, run):
+    out = [b.field(run, c) for c in range(8)]
+    for sp in (0, 1):
+        q = b.particles(run, sp)
+        out += [q[k] for k in ("x", "px", "py", "pz", "flag")]
+    return out, b.energy(run)
+
+
+# foils of 1 to 256 particles per cell: fewer particles than one part, one more than a
+# part, several units per tile, a foil at the wall whose hot electrons freeze there
+@pytest.mark.parametrize("cells,foil,ppc,interval,steps", [(64, (20, 16), 1, 8, 40), (500, (20, 57), 9, 8, 41),
+                                                           (500, (30, 200), 64, 8, 43), (700, (16, 40), 256, 5, 60),
+                                                           (520, (12, 500), 33, 16, 150)])
+def test_few_and_many_units_give_the_same_bits(picrr, cells, foil, ppc, interval, steps):
+    cpl = 100.0
+    run = dict(length_lambda=cells / cpl, foil_x0=foil[0] / cpl, foil_thickness=foil[1] / cpl, ne=20.0, a0=80.0,
+               polarization=picrr.CP, duration=3.0, steps=10**9, ppc=ppc, seed=5)
+    alone = picrr.Batch(cpl, max_runs=1, sort_interval=interval)
+    ra = alone.add_run(**run)
+    # 5.2M particles: more than 1216 units of 4096
+    beside = picrr.Batch(cpl, max_runs=2, sort_interval=interval)
+    beside.add_run(length_lambda=20.0, foil_x0=1.0, foil_thickness=10.0, ne=1.0, a0=1.0, polarization=0, duration=3.0,
+                   steps=10**9, ppc=2600, seed=6)
+    rb = beside.add_run(**run)
+    for n in (3, steps - 3):
+        assert alone.step(n) == n and beside.step(n) == n
+        (a, ea), (b, eb) = state(alone, ra), state(beside, rb)
+        for x, y in zip(a, b):
+            assert np.array_equal(x, y)
+        assert np.array_equal(ea[[0, 1, 2, 4, 5]], eb[[0, 1, 2, 4, 5]])
+        assert eb[3] == pytest.approx(ea[3], rel=1e-12, abs=1e-300)
+    assert alone.stats()["n_units"] > 0 and beside.stats()["n_units"] > 1216
+    alone.close()
+    beside.close()
+
+
+def test_more_units_in_a_group_than_are_staged(picrr):
+    """1400 units of 1024 particles in 600 cells: the planning kernel reads their bounds from
+    the table.  Shapes change the order of single-precision sums only: fields of order 1 after
+    17 steps differ by at most 17 x 2^-24 x a few hundred terms, below 1e-4."""
+    n, cpl = 700_000, 500.0
+    r = np.random.default_rng(3)
+    cell = np.sort(r.integers(30, 630, n)).astype(np.int32)
+    off = r.random(n, dtype=np.float32)
+    p = [(r.normal(size=n) * 0.5).astype(np.float32) for _ in range(3)]
+    res = []
+    for unit in (1024, 16384):
+        g = picrr.Sim(1.4, cpl, sort_interval=8)
+        for sp, (q, m) in enumerate(((-1.0, 1.0), (1.0, 1836.15267343))):
+            g.load_particles_f32(sp, cell, off, *p, 0.01, q, m)
+        g.inject_laser(30.0, picrr.CP, picrr.ENV_SIN2, 2.0)
+        g.set_shapes(unit, 8, 2)
+        assert g.step(17) == 17
+        assert (g.stats()["n_units"] > 1300) == (unit == 1024)
+        q = g.particles(0)
+        res.append([g.field(c) for c in range(5)] + [q["x"], q["px"]])
+        g.close()
+    for a, b in zip(*res):
+        assert np.max(np.abs(a - b)) <= 1e-4 * max(1.0, np.max(np.abs(b)))
