@@ -18,6 +18,8 @@
 #include <utility>
 #include <vector>
 
+#include <unistd.h>
+
 #include "picrr.h"
 #include "picrr_internal.cuh"
 
@@ -32,6 +34,7 @@ constexpr double kMpMe = 1836.15267343;     // proton mass / electron mass
 constexpr double kMuMe = 1822.888486209;    // atomic mass unit / electron mass
 constexpr double kLambdaCUm = 3.8615926796e-7;  // reduced Compton wavelength hbar/(m_e c), um (CODATA 2018)
 constexpr int kMaxDiagBlocks = 1024;
+constexpr size_t kStage = size_t{1} << 18;  // bytes of pinned staging for read-outs
 constexpr int kIncRing = 16;                // slots of the laser-source upload ring (one chunk of steps each)
 
 thread_local std::string g_null_error;  // failures of calls without a handle
@@ -127,7 +130,9 @@ struct Batch {
 
     std::vector<RunHost> runs;
     RunDev* d_runs = nullptr;
+    char* pinned = nullptr;    // one pinned allocation for h_runs, h_inc and stage
     RunDev* h_runs = nullptr;  // pinned staging of the run table
+    char* stage = nullptr;     // pinned, kStage bytes: small read-outs (kernels and copies write it directly)
     int32_t* d_blk_run = nullptr;
     int32_t* d_blk_i0 = nullptr;
     int nblk = 0, blk_cap = 0;
@@ -163,7 +168,6 @@ struct Batch {
     int* d_status = nullptr;
     unsigned* d_phase = nullptr;  // batch step of the last sort mod 6, advanced by the sort
     double* diag_partials = nullptr;
-    double* diag_out = nullptr;
     unsigned long long* snap_out = nullptr;  // [4]: max d bits, max chi bits, flagged count
     unsigned long long* bins = nullptr;
     int bins_cap = 0;
@@ -396,8 +400,7 @@ pic_status batch_create(const pic_config* cfg, int max_runs, Batch** out) {
         (st = dalloc_t(b, b->mem, &b->d_inc, static_cast<size_t>(max_runs) * 6 * KMAX)) != PIC_OK ||
         (st = dalloc_t(b, b->mem, &b->d_status, 4)) != PIC_OK ||
         (st = dalloc_t(b, b->mem, &b->d_phase, 1)) != PIC_OK ||
-        (st = dalloc_t(b, b->mem, &b->diag_partials, kMaxDiagBlocks)) != PIC_OK ||
-        (st = dalloc_t(b, b->mem, &b->diag_out, 8)) != PIC_OK ||
+        (st = dalloc_t(b, b->mem, &b->diag_partials, 3 * kMaxDiagBlocks)) != PIC_OK ||
         (st = dalloc_t(b, b->mem, &b->snap_out, 4)) != PIC_OK ||
         (st = dalloc_t(b, b->mem, &b->rs_units[0], static_cast<size_t>(4) * max_runs)) != PIC_OK ||
         (st = dalloc_t(b, b->mem, &b->rs_units[1], static_cast<size_t>(4) * max_runs)) != PIC_OK) {
@@ -405,12 +408,15 @@ pic_status batch_create(const pic_config* cfg, int max_runs, Batch** out) {
         batch_destroy(b);
         return st;
     }
-    if (cudaMallocHost(&b->h_runs, sizeof(RunDev) * max_runs) != cudaSuccess ||
-        cudaMallocHost(&b->h_inc, sizeof(float) * 6 * max_runs * KMAX * kIncRing) != cudaSuccess) {
+    const size_t inc_bytes = sizeof(float) * 6 * static_cast<size_t>(max_runs) * KMAX * kIncRing;
+    if (cudaMallocHost(&b->pinned, kStage + inc_bytes + sizeof(RunDev) * max_runs) != cudaSuccess) {
         cudaGetLastError();
         batch_destroy(b);
         return fail(nullptr, PIC_ERR_OOM, "pinned host allocation failed");
     }
+    b->stage = b->pinned;
+    b->h_inc = reinterpret_cast<float*>(b->pinned + kStage);
+    b->h_runs = reinterpret_cast<RunDev*>(b->pinned + kStage + inc_bytes);
     std::memset(b->h_runs, 0, sizeof(RunDev) * max_runs);
     for (int i = 0; i < kIncRing; ++i) cudaEventCreateWithFlags(&b->inc_ev[i], cudaEventDisableTiming);
     if (cudaStreamCreateWithFlags(&b->cap_stream, cudaStreamNonBlocking) != cudaSuccess) {
@@ -441,8 +447,7 @@ void batch_destroy(Batch* b) {
     if (b->stream) cudaStreamSynchronize(b->stream);
     for (int i = 0; i < kIncRing; ++i)
         if (b->inc_ev[i]) cudaEventDestroy(b->inc_ev[i]);
-    if (b->h_runs) cudaFreeHost(b->h_runs);
-    if (b->h_inc) cudaFreeHost(b->h_inc);
+    if (b->pinned) cudaFreeHost(b->pinned);
     for (int c = 0; c < 2; ++c) {
         if (b->graph[c]) cudaGraphExecDestroy(b->graph[c]);
         for (EventPair& ep : b->graph_ev[c]) {
@@ -1441,29 +1446,26 @@ pic_status run_energy(Batch* b, int id, double out[6]) {
     D.Nx = r.Nx;
     D.is = r.is;
     D.hc = static_cast<float>(0.5 * b->cfl);
-    int nb = launch_field_energy(D, b->diag_partials, kMaxDiagBlocks, b->stream);
-    launch_reduce_partials(b->diag_partials, nb, b->dx, b->diag_out + 0, b->stream);
+    ReduceParams P{};
+    P.partials = b->diag_partials;
+    P.stride = kMaxDiagBlocks;
+    P.tally = r.dev.tally;
+    P.out = reinterpret_cast<double*>(b->stage);
+    P.n[0] = launch_field_energy(D, b->diag_partials, kMaxDiagBlocks, b->stream);
+    P.scale[0] = b->dx;
     b->launches += 2;
     for (int s = 0; s < 2; ++s) {
         const HostSpecies& h = r.sp[s];
-        if (!h.loaded || h.n == 0) {
-            PIC_CK(b, cudaMemsetAsync(b->diag_out + 1 + s, 0, sizeof(double), b->stream));
-            continue;
-        }
-        nb = launch_kinetic(r.dev.sp[s][run_pbuf(b, r)], h.n, b->diag_partials, kMaxDiagBlocks, b->stream);
-        launch_reduce_partials(b->diag_partials, nb, h.w * b->dx * h.m, b->diag_out + 1 + s, b->stream);
-        b->launches += 2;
+        if (!h.loaded || h.n == 0) continue;  // no partials: 0
+        P.n[1 + s] = launch_kinetic(r.dev.sp[s][run_pbuf(b, r)], h.n, b->diag_partials + (1 + s) * kMaxDiagBlocks,
+                                    kMaxDiagBlocks, b->stream);
+        P.scale[1 + s] = h.w * b->dx * h.m;
+        b->launches++;
     }
-    double d[3], t[3];
-    PIC_CK(b, cudaMemcpyAsync(d, b->diag_out, sizeof(d), cudaMemcpyDeviceToHost, b->stream));
-    PIC_CK(b, cudaMemcpyAsync(t, r.dev.tally, sizeof(t), cudaMemcpyDeviceToHost, b->stream));
+    launch_reduce(P, b->stream);
     PIC_CK(b, cudaStreamSynchronize(b->stream));
-    out[0] = d[0];
-    out[1] = d[1];
-    out[2] = d[2];
-    out[3] = t[0];
-    out[4] = t[1];
-    out[5] = t[2];
+    PIC_CK(b, cudaGetLastError());
+    std::memcpy(out, b->stage, 6 * sizeof(double));
     return PIC_OK;
 }
 
@@ -1475,8 +1477,16 @@ pic_status run_spectra(Batch* b, int id, int species, int nbins, double e_min, d
         return fail(b, PIC_ERR_INVALID_ARG, "need 1 <= nbins <= 2^24, e_max > e_min, counts != NULL");
     const RunHost& r = b->runs[id];
     const HostSpecies& h = r.sp[species];
-    std::vector<unsigned long long> hb(static_cast<size_t>(nbins) + 2, 0ull);
-    if (h.loaded && h.n > 0) {
+    // the counters come back through the pinned staging buffer where they fit
+    const size_t hb_bytes = sizeof(unsigned long long) * static_cast<size_t>(nbins);
+    std::vector<unsigned long long> big;
+    unsigned long long* hb = reinterpret_cast<unsigned long long*>(b->stage + 64);
+    if (64 + hb_bytes > kStage) {
+        big.resize(static_cast<size_t>(nbins));
+        hb = big.data();
+    }
+    const bool any = h.loaded && h.n > 0;
+    if (any) {
         if (b->bins_cap < nbins + 2) {
             std::vector<std::pair<void*, size_t>> fresh;
             unsigned long long* nbp = nullptr;
@@ -1491,21 +1501,90 @@ pic_status run_spectra(Batch* b, int id, int species, int nbins, double e_min, d
         const DevSpecies& sp = r.dev.sp[species][run_pbuf(b, r)];
         launch_spectrum(sp.px, sp.py, sp.pz, h.n, h.m * kMec2MeV, nbins, e_min, e_max, b->bins, b->stream);
         b->launches++;
-        PIC_CK(b, cudaMemcpyAsync(hb.data(), b->bins, sizeof(unsigned long long) * (nbins + 2),
-                                  cudaMemcpyDeviceToHost, b->stream));
+        PIC_CK(b, cudaMemcpyAsync(hb, b->bins, hb_bytes, cudaMemcpyDeviceToHost, b->stream));
     }
-    double tally0 = 0.0;
-    PIC_CK(b, cudaMemcpyAsync(&tally0, r.dev.tally, sizeof(double), cudaMemcpyDeviceToHost, b->stream));
+    PIC_CK(b, cudaMemcpyAsync(b->stage, r.dev.tally, sizeof(double), cudaMemcpyDeviceToHost, b->stream));
     PIC_CK(b, cudaStreamSynchronize(b->stream));
+    double tally0;
+    std::memcpy(&tally0, b->stage, sizeof(double));
     const double width = (e_max - e_min) / nbins;
     const double wdx = h.w * b->dx;
-    for (int k = 0; k < nbins; ++k) counts[k] = static_cast<double>(hb[k]) * wdx / width;
+    for (int k = 0; k < nbins; ++k) counts[k] = any ? static_cast<double>(hb[k]) * wdx / width : 0.0;
     if (radiated) {
         // energy unit per area: m_e c^2 n_c (c/omega), n_c = eps0 m_e omega^2 / e^2 (SI)
         const double me = 9.1093837015e-31, c = 299792458.0, qe = 1.602176634e-19, eps0 = 8.8541878128e-12;
         const double omega = 2.0 * kPi * c / (b->cfg.lambda_um * 1e-6);
         const double nc = eps0 * me * omega * omega / (qe * qe);
         *radiated = tally0 * me * c * c * nc * c / omega;
+    }
+    return PIC_OK;
+}
+
+// Writes to every page of a caller's array that a copy is about to fill: the copy engine reaches pages that the
+// host has not touched yet through its page faults (five fresh arrays of 3.2 MB: 12.5 ms; touched first, 1.0 ms,
+// most of it the kernel's zeroing; already resident 0.2 ms).
+void touch_pages(void* p, size_t bytes) {
+    static const size_t page = static_cast<size_t>(sysconf(_SC_PAGESIZE));
+    volatile char* c = static_cast<volatile char*>(p);
+    for (size_t i = 0; i < bytes; i += page) c[i] = 0;
+    if (bytes) c[bytes - 1] = 0;
+}
+
+// Particles with load index below m, as launch_read gives them, into the caller's host arrays dst (nullable
+// each).  Few particles go through the pinned staging buffer, one kernel and one wait for all arrays; many
+// through the species' other particle buffer (dead between sorts) in two halves, each array copied to its place.
+pic_status read_arrays(Batch* b, const RunHost& r, int species, int64_t m, const SnapParams* S, double* const dst[5],
+                       int32_t* flag, unsigned long long so[4]) {
+    const int64_t n = r.sp[species].n;
+    const int pb = run_pbuf(b, r);
+    const DevSpecies &sp = r.dev.sp[species][pb], &alt = r.dev.sp[species][1 - pb];
+    unsigned long long* hso = reinterpret_cast<unsigned long long*>(b->stage);
+    char* const st = b->stage + 64;
+    const int64_t each = (m + 1) & ~int64_t{1};  // keeps every staged array 16-byte aligned
+    const bool small = 64 + static_cast<size_t>(each) * (5 * 8 + 4) <= kStage;
+    ReadOut O{};
+    O.dx = b->dx;
+    O.Nx = r.Nx;
+    PIC_CK(b, cudaMemsetAsync(b->snap_out, 0, 4 * sizeof(unsigned long long), b->stream));
+    const int halves = m <= 0 || small ? 1 : 2;
+    const int64_t per = (m + halves - 1) / halves;
+    for (int h = 0; h < halves; ++h) {
+        O.j0 = h * per;
+        O.j1 = std::min(m, O.j0 + per);
+        void* place[6];
+        for (int q = 0; q < 5; ++q) place[q] = st + q * each * 8;
+        place[5] = st + 5 * each * 8;
+        if (!small) {
+            void* const dead[6] = {alt.cell, alt.off, alt.px, alt.py, alt.pz, alt.id};
+            for (int q = 0; q < 6; ++q) place[q] = dead[q];
+        }
+        double** const o[5] = {&O.x, &O.px, &O.a, &O.b, &O.c};
+        for (int q = 0; q < 5; ++q) *o[q] = dst[q] ? static_cast<double*>(place[q]) : nullptr;
+        O.flag = flag ? static_cast<int32_t*>(place[5]) : nullptr;
+        if (h == 1 && S) {  // the summary is the first half's
+            PIC_CK(b, cudaMemcpyAsync(hso, b->snap_out, 4 * sizeof(unsigned long long), cudaMemcpyDeviceToHost, b->stream));
+            PIC_CK(b, cudaMemsetAsync(b->snap_out, 0, 3 * sizeof(unsigned long long), b->stream));
+        }
+        launch_read(sp, n, S, O, b->snap_out, b->stream);
+        b->launches++;
+        const size_t c = static_cast<size_t>(O.j1 - O.j0);
+        for (int q = 0; h == 0 && q < 5 && !small; ++q)
+            if (dst[q]) touch_pages(dst[q], static_cast<size_t>(m) * 8);  // while the kernel runs
+        if (h == 0 && flag && !small) touch_pages(flag, static_cast<size_t>(m) * 4);
+        for (int q = 0; q < 5 && !small; ++q)
+            if (dst[q]) PIC_CK(b, cudaMemcpyAsync(dst[q] + O.j0, place[q], c * 8, cudaMemcpyDeviceToHost, b->stream));
+        if (flag && !small) PIC_CK(b, cudaMemcpyAsync(flag + O.j0, place[5], c * 4, cudaMemcpyDeviceToHost, b->stream));
+    }
+    if (halves == 1 || !S)
+        PIC_CK(b, cudaMemcpyAsync(hso, b->snap_out, 4 * sizeof(unsigned long long), cudaMemcpyDeviceToHost, b->stream));
+    PIC_CK(b, cudaStreamSynchronize(b->stream));
+    PIC_CK(b, cudaGetLastError());
+    for (int q = 0; q < 4; ++q) so[q] = hso[q];
+    if (so[3]) return fail(b, PIC_ERR_STATE, "corrupt particle id");
+    if (small && m > 0) {
+        for (int q = 0; q < 5; ++q)
+            if (dst[q]) std::memcpy(dst[q], st + q * each * 8, static_cast<size_t>(m) * 8);
+        if (flag) std::memcpy(flag, st + 5 * each * 8, static_cast<size_t>(m) * 4);
     }
     return PIC_OK;
 }
@@ -1518,37 +1597,9 @@ pic_status run_read_particles(Batch* b, int id, int species, int64_t cap, double
     const int64_t n = h.loaded ? h.n : 0;
     if (nout) *nout = n;
     if (cap <= 0 || n == 0) return PIC_OK;
-    std::vector<int32_t> c(n), idv(n);
-    std::vector<float> o(n), qx(n), qy(n), qz(n);
-    const DevSpecies& d = r.dev.sp[species][run_pbuf(b, r)];
-    const size_t by = static_cast<size_t>(n) * 4;
-    PIC_CK(b, cudaMemcpyAsync(c.data(), d.cell, by, cudaMemcpyDeviceToHost, b->stream));
-    PIC_CK(b, cudaMemcpyAsync(idv.data(), d.id, by, cudaMemcpyDeviceToHost, b->stream));
-    PIC_CK(b, cudaMemcpyAsync(o.data(), d.off, by, cudaMemcpyDeviceToHost, b->stream));
-    PIC_CK(b, cudaMemcpyAsync(qx.data(), d.px, by, cudaMemcpyDeviceToHost, b->stream));
-    PIC_CK(b, cudaMemcpyAsync(qy.data(), d.py, by, cudaMemcpyDeviceToHost, b->stream));
-    PIC_CK(b, cudaMemcpyAsync(qz.data(), d.pz, by, cudaMemcpyDeviceToHost, b->stream));
-    PIC_CK(b, cudaStreamSynchronize(b->stream));
-    for (int64_t i = 0; i < n; ++i) {
-        const int64_t j = idv[i];
-        if (j < 0 || j >= n) return fail(b, PIC_ERR_STATE, "corrupt particle id");
-        if (j >= cap) continue;
-        int fl = 0;
-        double xi;
-        if (c[i] < 0) {  // frozen at a wall, stored as -1 - (last cell)
-            const int key = -1 - c[i];
-            fl = key == 0 ? -1 : 1;
-            xi = key == 0 ? 0.0 : static_cast<double>(r.Nx);
-        } else {
-            xi = static_cast<double>(c[i]) + o[i];
-        }
-        if (x) x[j] = xi * b->dx;
-        if (px) px[j] = qx[i];
-        if (py) py[j] = qy[i];
-        if (pz) pz[j] = qz[i];
-        if (flag) flag[j] = fl;
-    }
-    return PIC_OK;
+    double* const dst[5] = {x, px, py, pz, nullptr};
+    unsigned long long so[4];
+    return read_arrays(b, r, species, std::min(cap, n), nullptr, dst, flag, so);
 }
 
 // Skin-layer snapshot: d of Eq. (damping) and chi per particle on the device,
@@ -1564,53 +1615,17 @@ pic_status run_snapshot(Batch* b, int id, int species, double chi_flag, int64_t 
     if (nout) *nout = n;
     if (summary) summary[0] = summary[1] = summary[2] = 0.0;
     if (n == 0) return PIC_OK;
-    const bool per = cap > 0 && (x || px || pperp || d || chi);
-    std::vector<std::pair<void*, size_t>> tmp;
-    float *dd = nullptr, *dc = nullptr;
-    if (per) {
-        pic_status st = dalloc_t(b, tmp, &dd, static_cast<size_t>(n));
-        if (st == PIC_OK) st = dalloc_t(b, tmp, &dc, static_cast<size_t>(n));
-        if (st != PIC_OK) {
-            free_all(b, tmp);
-            return st;
-        }
-    }
     SnapParams S{};
     const int fb = run_fbuf(b, r);
     for (int c = 0; c < 5; ++c) S.F[c] = r.dev.F[fb][c];
     S.eps = static_cast<float>(b->eps);
     S.ecr_inv = static_cast<float>(2.0 * kPi * kLambdaCUm / b->cfg.lambda_um);  // 1 / (m c^2 / hbar omega)
     S.chi_flag = static_cast<float>(chi_flag);
-    const DevSpecies& sp = r.dev.sp[species][run_pbuf(b, r)];
-    PIC_CK(b, cudaMemsetAsync(b->snap_out, 0, 4 * sizeof(unsigned long long), b->stream));
-    launch_snapshot(sp, n, S, dd, dc, b->snap_out, b->stream);
-    b->launches++;
-    unsigned long long so[3];
-    PIC_CK(b, cudaMemcpyAsync(so, b->snap_out, sizeof(so), cudaMemcpyDeviceToHost, b->stream));
-    std::vector<int32_t> c, idv;
-    std::vector<float> o, qx, qy, qz, hd, hc;
-    if (per) {
-        c.resize(n);
-        idv.resize(n);
-        o.resize(n);
-        qx.resize(n);
-        qy.resize(n);
-        qz.resize(n);
-        hd.resize(n);
-        hc.resize(n);
-        const size_t by = static_cast<size_t>(n) * 4;
-        PIC_CK(b, cudaMemcpyAsync(c.data(), sp.cell, by, cudaMemcpyDeviceToHost, b->stream));
-        PIC_CK(b, cudaMemcpyAsync(idv.data(), sp.id, by, cudaMemcpyDeviceToHost, b->stream));
-        PIC_CK(b, cudaMemcpyAsync(o.data(), sp.off, by, cudaMemcpyDeviceToHost, b->stream));
-        PIC_CK(b, cudaMemcpyAsync(qx.data(), sp.px, by, cudaMemcpyDeviceToHost, b->stream));
-        PIC_CK(b, cudaMemcpyAsync(qy.data(), sp.py, by, cudaMemcpyDeviceToHost, b->stream));
-        PIC_CK(b, cudaMemcpyAsync(qz.data(), sp.pz, by, cudaMemcpyDeviceToHost, b->stream));
-        PIC_CK(b, cudaMemcpyAsync(hd.data(), dd, by, cudaMemcpyDeviceToHost, b->stream));
-        PIC_CK(b, cudaMemcpyAsync(hc.data(), dc, by, cudaMemcpyDeviceToHost, b->stream));
-    }
-    cudaError_t e = cudaStreamSynchronize(b->stream);
-    free_all(b, tmp);
-    if (e != cudaSuccess) return cuda_fail(b, e, "snapshot");
+    double* const dst[5] = {x, px, pperp, d, chi};
+    const bool per = cap > 0 && (x || px || pperp || d || chi);
+    unsigned long long so[4];
+    const pic_status st = read_arrays(b, r, species, per ? std::min(cap, n) : 0, &S, dst, nullptr, so);
+    if (st != PIC_OK) return st;
     if (summary) {
         float f0, f1;
         const unsigned int u0 = static_cast<unsigned int>(so[0]), u1 = static_cast<unsigned int>(so[1]);
@@ -1619,24 +1634,6 @@ pic_status run_snapshot(Batch* b, int id, int species, double chi_flag, int64_t 
         summary[0] = f0;
         summary[1] = f1;
         summary[2] = static_cast<double>(so[2]);
-    }
-    if (!per) return PIC_OK;
-    for (int64_t i = 0; i < n; ++i) {
-        const int64_t j = idv[i];
-        if (j < 0 || j >= n) return fail(b, PIC_ERR_STATE, "corrupt particle id");
-        if (j >= cap) continue;
-        double xi;
-        if (c[i] < 0) {
-            const int key = -1 - c[i];
-            xi = key == 0 ? 0.0 : static_cast<double>(r.Nx);
-        } else {
-            xi = static_cast<double>(c[i]) + o[i];
-        }
-        if (x) x[j] = xi * b->dx;
-        if (px) px[j] = qx[i];
-        if (pperp) pperp[j] = std::sqrt(static_cast<double>(qy[i]) * qy[i] + static_cast<double>(qz[i]) * qz[i]);
-        if (d) d[j] = hd[i];
-        if (chi) chi[j] = hc[i];
     }
     return PIC_OK;
 }
@@ -1662,18 +1659,28 @@ pic_status run_read_fields(Batch* b, int id, int comp, int64_t cap, double* out,
     const int64_t n = node ? r.Nx + 1 : r.Nx;
     if (nout) *nout = n;
     if (!out || cap < n) return fail(b, PIC_ERR_INVALID_ARG, "output too small");
-    if (comp >= PIC_JX) {
-        std::vector<double> j;
-        pic_status st = last_current(b, r, comp - PIC_JX, j);
-        if (st != PIC_OK) return st;
-        for (int64_t i = 0; i < n; ++i) out[i] = j[static_cast<size_t>(PADF + i)];
+    const int js = run_jset(b, r);
+    const float* f = comp >= PIC_JX ? nullptr : r.dev.F[run_fbuf(b, r)][comp] + PADF;
+    const unsigned long long* fix = comp >= PIC_JX ? r.dev.J[js][comp - PIC_JX] + PADF : nullptr;
+    const double scale = std::ldexp(1.0, -r.fp_bits);
+    if (static_cast<size_t>(n) * 8 <= kStage / 2) {  // widened into the pinned staging buffer
+        launch_widen(f, fix, scale, n, reinterpret_cast<double*>(b->stage), b->stream);
+        b->launches++;
+        PIC_CK(b, cudaStreamSynchronize(b->stream));
+        PIC_CK(b, cudaGetLastError());
+        std::memcpy(out, b->stage, static_cast<size_t>(n) * 8);
         return PIC_OK;
     }
-    const float* src = r.dev.F[run_fbuf(b, r)][comp];
-    std::vector<float> h(static_cast<size_t>(n));
-    PIC_CK(b, cudaMemcpyAsync(h.data(), src + PADF, sizeof(float) * n, cudaMemcpyDeviceToHost, b->stream));
+    // widened into a current set that does not hold the last current (cleared again, as the next step wants it),
+    // then straight to the caller's array: the copy runs faster than the host could widen
+    unsigned long long* tmp = r.dev.J[(js + 1) % 3][0];
+    launch_widen(f, fix, scale, n, reinterpret_cast<double*>(tmp), b->stream);
+    b->launches++;
+    touch_pages(out, static_cast<size_t>(n) * 8);
+    PIC_CK(b, cudaMemcpyAsync(out, tmp, static_cast<size_t>(n) * 8, cudaMemcpyDeviceToHost, b->stream));
+    PIC_CK(b, cudaMemsetAsync(tmp, 0, static_cast<size_t>(n) * 8, b->stream));
     PIC_CK(b, cudaStreamSynchronize(b->stream));
-    for (int64_t i = 0; i < n; ++i) out[i] = h[static_cast<size_t>(i)];
+    PIC_CK(b, cudaGetLastError());
     return PIC_OK;
 }
 

@@ -269,15 +269,21 @@ struct DiagParams {
 // Writes double out_partials[grid]; returns grid used.
 int launch_field_energy(const DiagParams& D, double* partials, int max_blocks, cudaStream_t st);
 int launch_kinetic(DevSpecies sp, int64_t n, double* partials, int max_blocks, cudaStream_t st);
-void launch_reduce_partials(const double* partials, int n, double scale, double* out, cudaStream_t st);
+// out[0..2]: the sums of three arrays of partials (n[q] each, `stride` apart) times scale; out[3..5]: the tally.
+struct ReduceParams {
+    const double* partials;
+    int stride, n[3];
+    double scale[3];
+    const double* tally;
+    double* out;  // device or pinned host memory
+};
+void launch_reduce(const ReduceParams& P, cudaStream_t st);
 // bins[0..nbins) counts, bins[nbins] underflow, bins[nbins+1] overflow, added to what is there.
 void launch_spectrum(const float* px, const float* py, const float* pz, int64_t n, double mass_mev, int nbins,
                      double e_min, double e_max, unsigned long long* bins, cudaStream_t st);
 
 // Friction coefficient d (Eq. damping) and quantum parameter chi per particle
-// from the stored momentum and the fields at the particle.  d_out / chi_out
-// (nullable) in stored order; out[0], out[1]: float bits of max d and max chi
-// (atomicMax on the bits of non-negative floats); out[2]: count of chi >= chi_flag.
+// from the stored momentum and the fields at the particle.
 struct SnapParams {
     const float* F[5];
     float eps, ecr_inv, chi_flag;
@@ -286,7 +292,22 @@ void launch_wait_selftest(int* status, cudaStream_t st);
 void launch_validate(const int32_t* cell, const float* off, const float* px, const float* py, const float* pz,
                      int64_t n, int Nx, unsigned long long* out, cudaStream_t st);
 
-void launch_snapshot(DevSpecies sp, int64_t n, const SnapParams& S, float* d_out, float* chi_out,
-                     unsigned long long* out, cudaStream_t st);
+// Read-out of the particles whose load index lies in [j0, j1), at index - j0 of each array
+// (nullable; device memory or pinned host memory): x, p_x and, without a snapshot, a = p_y,
+// b = p_z and flag, with one a = p_perp, b = d and c = chi.
+struct ReadOut {
+    double *x, *px, *a, *b, *c;
+    int32_t* flag;
+    int64_t j0, j1;
+    double dx;
+    int Nx;
+};
+// With S also the snapshot's summary: out[0], out[1]: float bits of max d and max chi
+// (atomicMax on the bits of non-negative floats); out[2]: count of chi >= chi_flag.
+// out[3] is set if a stored id is not in [0, n).
+void launch_read(DevSpecies sp, int64_t n, const SnapParams* S, const ReadOut& O, unsigned long long* out,
+                 cudaStream_t st);
+// out[i] = f[i], or (f null) the fixed-point fix[i] * scale, in double.
+void launch_widen(const float* f, const unsigned long long* fix, double scale, int64_t n, double* out, cudaStream_t st);
 
 }  // namespace picrr
