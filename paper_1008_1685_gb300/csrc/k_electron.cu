@@ -379,6 +379,7 @@ extern "C" pic_status pic_electron_scan(const pic_electron_case* cases, int64_t 
         picrr::launch_electron_scan(dc, dorder, static_cast<int64_t>(order.size()), integrator, flags, dt, nsteps, every, eps, dout, nsamples, st);
         e = cudaGetLastError();
     }
+    if (e == cudaSuccess) picrr::touch_pages(out, out_bytes);  // while the kernel runs
     if (e == cudaSuccess && out_bytes) e = cudaMemcpyAsync(out, dout, out_bytes, cudaMemcpyDeviceToHost, st);
     if (dc) cudaFreeAsync(dc, st);
     if (dorder) cudaFreeAsync(dorder, st);

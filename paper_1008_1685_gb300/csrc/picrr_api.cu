@@ -18,8 +18,6 @@
 #include <utility>
 #include <vector>
 
-#include <unistd.h>
-
 #include "picrr.h"
 #include "picrr_internal.cuh"
 
@@ -34,7 +32,7 @@ constexpr double kMpMe = 1836.15267343;     // proton mass / electron mass
 constexpr double kMuMe = 1822.888486209;    // atomic mass unit / electron mass
 constexpr double kLambdaCUm = 3.8615926796e-7;  // reduced Compton wavelength hbar/(m_e c), um (CODATA 2018)
 constexpr int kMaxDiagBlocks = 1024;
-constexpr size_t kStage = size_t{1} << 18;  // bytes of pinned staging for read-outs
+constexpr size_t kStage = size_t{640} << 10;  // bytes of pinned staging for read-outs (1 MB cost a handle 300 us more to make and free)
 constexpr int kIncRing = 16;                // slots of the laser-source upload ring (one chunk of steps each)
 
 thread_local std::string g_null_error;  // failures of calls without a handle
@@ -239,6 +237,26 @@ pic_status dalloc_t(Batch* b, std::vector<std::pair<void*, size_t>>& owner, T** 
     return st;
 }
 
+size_t rounded(size_t bytes) { return ((bytes ? bytes : 16) + 255) & ~static_cast<size_t>(255); }
+
+// Several arrays in one allocation (each on a 256-byte boundary): an allocation and its clearing cost the host
+// 4 us, a run opened with 36 of them and each species with 12.
+struct Slab {
+    std::vector<std::pair<void**, size_t>> want;
+    size_t total = 0;
+    template <class T>
+    void add(T** p, size_t count) {
+        want.emplace_back(reinterpret_cast<void**>(p), total);
+        total += rounded(count * sizeof(T));
+    }
+};
+pic_status dalloc_slab(Batch* b, std::vector<std::pair<void*, size_t>>& owner, const Slab& S) {
+    void* base = nullptr;
+    const pic_status st = dalloc(b, owner, &base, S.total);
+    for (auto& w : S.want) *w.first = st == PIC_OK ? static_cast<char*>(base) + w.second : nullptr;
+    return st;
+}
+
 void free_all(Batch* b, std::vector<std::pair<void*, size_t>>& owner) {
     for (auto& a : owner) {
         cudaFreeAsync(a.first, b->stream);
@@ -396,14 +414,15 @@ pic_status batch_create(const pic_config* cfg, int max_runs, Batch** out) {
         return fail(nullptr, PIC_ERR_CUDA, "cudaStreamCreate failed");
     }
     b->stream = b->own_stream;
-    if ((st = dalloc_t(b, b->mem, &b->d_runs, static_cast<size_t>(max_runs))) != PIC_OK ||
-        (st = dalloc_t(b, b->mem, &b->d_inc, static_cast<size_t>(max_runs) * 6 * KMAX)) != PIC_OK ||
-        (st = dalloc_t(b, b->mem, &b->d_status, 4)) != PIC_OK ||
-        (st = dalloc_t(b, b->mem, &b->d_phase, 1)) != PIC_OK ||
-        (st = dalloc_t(b, b->mem, &b->diag_partials, 3 * kMaxDiagBlocks)) != PIC_OK ||
-        (st = dalloc_t(b, b->mem, &b->snap_out, 4)) != PIC_OK ||
-        (st = dalloc_t(b, b->mem, &b->rs_units[0], static_cast<size_t>(4) * max_runs)) != PIC_OK ||
-        (st = dalloc_t(b, b->mem, &b->rs_units[1], static_cast<size_t>(4) * max_runs)) != PIC_OK) {
+    Slab slab;
+    slab.add(&b->d_runs, static_cast<size_t>(max_runs));
+    slab.add(&b->d_inc, static_cast<size_t>(max_runs) * 6 * KMAX);
+    slab.add(&b->d_status, 4);
+    slab.add(&b->d_phase, 1);
+    slab.add(&b->diag_partials, 3 * kMaxDiagBlocks);
+    slab.add(&b->snap_out, 4);
+    for (int32_t*& t : b->rs_units) slab.add(&t, static_cast<size_t>(4) * max_runs);
+    if ((st = dalloc_slab(b, b->mem, slab)) != PIC_OK) {
         g_null_error = b->err;
         batch_destroy(b);
         return st;
@@ -488,23 +507,23 @@ pic_status run_open(Batch* b, double length_lambda, int source_node, int rr_on, 
     d.is = is;
     d.glen = static_cast<int>(r.glen);
     d.rr = r.rr;
-    pic_status st = PIC_OK;
-    for (int x = 0; x < 2 && st == PIC_OK; ++x)
-        for (int c = 0; c < 5 && st == PIC_OK; ++c) st = dalloc_t(b, r.mem, &d.F[x][c], r.glen);
-    for (int x = 0; x < 3 && st == PIC_OK; ++x)
-        for (int c = 0; c < 3 && st == PIC_OK; ++c) st = dalloc_t(b, r.mem, &d.J[x][c], r.glen);
-    if (st == PIC_OK) st = dalloc_t(b, r.mem, &d.tally, 4);
+    Slab slab;
+    for (auto& f : d.F)
+        for (float*& c : f) slab.add(&c, r.glen);
+    for (auto& j : d.J)
+        for (unsigned long long*& c : j) slab.add(&c, r.glen);
+    slab.add(&d.tally, 4);
     const size_t nk = static_cast<size_t>(Nx) + 2, nkb = static_cast<size_t>(Nx) / KEY_T + 2,
                  ngr = static_cast<size_t>(Nx) / SPAN + 4;
-    for (int s = 0; s < 2 && st == PIC_OK; ++s) {
-        if (st == PIC_OK) st = dalloc_t(b, r.mem, &d.keycount[s], nk);
-        if (st == PIC_OK) st = dalloc_t(b, r.mem, &d.keystart[s], nk);
-        if (st == PIC_OK) st = dalloc_t(b, r.mem, &d.blocksum[s], nkb);
-        if (st == PIC_OK) st = dalloc_t(b, r.mem, &d.blockstart[s], nkb);
-        if (st == PIC_OK) st = dalloc_t(b, r.mem, &d.group_n[s], ngr);
-        if (st == PIC_OK) st = dalloc_t(b, r.mem, &d.group_first[s][0], ngr);
-        if (st == PIC_OK) st = dalloc_t(b, r.mem, &d.group_first[s][1], ngr);
+    for (int s = 0; s < 2; ++s) {
+        slab.add(&d.keycount[s], nk);
+        slab.add(&d.keystart[s], nk);
+        slab.add(&d.blocksum[s], nkb);
+        slab.add(&d.blockstart[s], nkb);
+        slab.add(&d.group_n[s], ngr);
+        for (int32_t*& g : d.group_first[s]) slab.add(&g, ngr);
     }
+    const pic_status st = dalloc_slab(b, r.mem, slab);
     if (st != PIC_OK) {
         free_all(b, r.mem);
         r = RunHost();
@@ -514,8 +533,6 @@ pic_status run_open(Batch* b, double length_lambda, int source_node, int rr_on, 
     *out_id = id;
     return PIC_OK;
 }
-
-size_t rounded(size_t bytes) { return ((bytes ? bytes : 16) + 255) & ~static_cast<size_t>(255); }
 
 // Device bytes a run of length_lambda with n particles per species takes in a
 // batch: its grid, sort scratch and particle buffers as run_open and
@@ -555,16 +572,16 @@ void run_release(Batch* b, int id) {
 
 pic_status alloc_species(Batch* b, RunHost& r, int s, int64_t n) {
     const size_t cap = static_cast<size_t>((n + 3) / 4 * 4 + 8);
-    pic_status st = PIC_OK;
-    for (int x = 0; x < 2 && st == PIC_OK; ++x) {
-        DevSpecies& d = r.dev.sp[s][x];
-        if (st == PIC_OK) st = dalloc_t(b, r.mem, &d.cell, cap);
-        if (st == PIC_OK) st = dalloc_t(b, r.mem, &d.off, cap);
-        if (st == PIC_OK) st = dalloc_t(b, r.mem, &d.px, cap);
-        if (st == PIC_OK) st = dalloc_t(b, r.mem, &d.py, cap);
-        if (st == PIC_OK) st = dalloc_t(b, r.mem, &d.pz, cap);
-        if (st == PIC_OK) st = dalloc_t(b, r.mem, &d.id, cap);
+    Slab slab;
+    for (DevSpecies& d : r.dev.sp[s]) {
+        slab.add(&d.cell, cap);
+        slab.add(&d.off, cap);
+        slab.add(&d.px, cap);
+        slab.add(&d.py, cap);
+        slab.add(&d.pz, cap);
+        slab.add(&d.id, cap);
     }
+    const pic_status st = dalloc_slab(b, r.mem, slab);
     if (st == PIC_OK) {
         r.sp[s].n = n;
         r.dev.n[s] = static_cast<int32_t>(n);
@@ -828,28 +845,19 @@ pic_status ensure_units(Batch* b, int need) {
     uint16_t* cn = nullptr;
     int32_t* of = nullptr;
     const size_t m = static_cast<size_t>(mu);
-    pic_status st = PIC_OK;
+    Slab slab;
     for (UnitTable& u : tab) {
-        for (int32_t** a : {&u.run, &u.species, &u.start, &u.end, &u.lo, &u.hi})
-            if (st == PIC_OK) st = dalloc_t(b, fresh, a, m);
-        if (st == PIC_OK) st = dalloc_t(b, fresh, &u.count, 4);
+        for (int32_t** a : {&u.run, &u.species, &u.start, &u.end, &u.lo, &u.hi}) slab.add(a, m);
+        slab.add(&u.count, 4);
     }
-    if (st == PIC_OK) st = dalloc_t(b, fresh, &rp, m);
-    if (st == PIC_OK) st = dalloc_t(b, fresh, &cn, m * SSTR);
-    if (st == PIC_OK) st = dalloc_t(b, fresh, &of, m * SSTR);
-    if (st != PIC_OK) {
-        free_all(b, fresh);
-        return st;
-    }
+    slab.add(&rp, m);
+    slab.add(&cn, m * SSTR);
+    slab.add(&of, m * SSTR);
+    const pic_status st = dalloc_slab(b, fresh, slab);
+    if (st != PIC_OK) return st;
     // the unit table is rebuilt right after every growth (the radiated partials
     // were flushed by the sort that preceded it)
-    for (UnitTable& u : b->units)
-        for (void* p : {static_cast<void*>(u.run), static_cast<void*>(u.species), static_cast<void*>(u.start),
-                        static_cast<void*>(u.end), static_cast<void*>(u.lo), static_cast<void*>(u.hi),
-                        static_cast<void*>(u.count)})
-            free_one(b, p);
-    for (void* p : {static_cast<void*>(b->rad_part), static_cast<void*>(b->cnt), static_cast<void*>(b->offs)})
-        free_one(b, p);
+    free_one(b, b->units[0].run);  // the slab's first array
     for (auto& f : fresh) b->mem.push_back(f);
     b->units[0] = tab[0];
     b->units[1] = tab[1];
@@ -1303,13 +1311,14 @@ pic_status batch_step(Batch* b, int64_t n, int64_t* done) {
     }
     finish_field();
     if (it > 0 && b->since_sort > 0) rad_flush(b);
+    PIC_CK(b, cudaMemcpyAsync(b->stage, b->d_status, sizeof(int), cudaMemcpyDeviceToHost, b->stream));
     cudaError_t e = cudaStreamSynchronize(b->stream);
     if (e == cudaSuccess) e = cudaGetLastError();
     if (e != cudaSuccess) return cuda_fail(b, e, "step");
     collect_timing(b);
     read_all_graph_timing(b);
     int hst = 0;
-    PIC_CK(b, cudaMemcpy(&hst, b->d_status, sizeof(int), cudaMemcpyDeviceToHost));
+    std::memcpy(&hst, b->stage, sizeof(int));
     if (done) *done = it;
     if (hst & ST_TIMEOUT) return fail(b, PIC_ERR_TIMEOUT, "a bounded device wait (TMA field window) gave up");
     if (hst & ST_WINDOW) return fail(b, PIC_ERR_STATE, "a particle left its unit window");
@@ -1518,16 +1527,6 @@ pic_status run_spectra(Batch* b, int id, int species, int nbins, double e_min, d
         *radiated = tally0 * me * c * c * nc * c / omega;
     }
     return PIC_OK;
-}
-
-// Writes to every page of a caller's array that a copy is about to fill: the copy engine reaches pages that the
-// host has not touched yet through its page faults (five fresh arrays of 3.2 MB: 12.5 ms; touched first, 1.0 ms,
-// most of it the kernel's zeroing; already resident 0.2 ms).
-void touch_pages(void* p, size_t bytes) {
-    static const size_t page = static_cast<size_t>(sysconf(_SC_PAGESIZE));
-    volatile char* c = static_cast<volatile char*>(p);
-    for (size_t i = 0; i < bytes; i += page) c[i] = 0;
-    if (bytes) c[bytes - 1] = 0;
 }
 
 // Particles with load index below m, as launch_read gives them, into the caller's host arrays dst (nullable
