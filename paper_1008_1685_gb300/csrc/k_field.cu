@@ -8,9 +8,11 @@ namespace picrr {
 
 namespace {
 
+template <bool PDL>
 __global__ void __launch_bounds__(FIELD_T) k_field(const FieldParams P) {
     __shared__ FieldSmem S;
-    field_block<FIELD_T>(P, *P.phase + P.k, blockIdx.x, S);
+    pdl_release<PDL>();
+    field_block<FIELD_T, PDL>(P, *P.phase + P.k, blockIdx.x, S);
 }
 
 __global__ void __launch_bounds__(FIELD_T) k_zero_current(const FieldParams P) {
@@ -28,8 +30,8 @@ void launch_zero_current(const FieldParams& P, cudaStream_t st) {
     if (P.nblk > 0) k_zero_current<<<P.nblk, FIELD_T, 0, st>>>(P);
 }
 
-void launch_field(const FieldParams& P, int grid, cudaStream_t st) {
-    k_field<<<grid, FIELD_T, 0, st>>>(P);
+void launch_field(const FieldParams& P, int grid, cudaStream_t st, bool pdl) {
+    if (grid > 0) launch(pdl ? k_field<true> : k_field<false>, dim3(grid), FIELD_T, st, pdl, P);
 }
 
 }  // namespace picrr

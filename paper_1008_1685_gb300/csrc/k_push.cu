@@ -202,11 +202,11 @@ struct PushSmem<2> {
 };
 
 // The Yee update of the fields in F (old, from the element `p0` - 4 of the padded grid on) to the step after,
-// for the window's L elements, by all threads of the block; the same arithmetic as field_block.
-__device__ __forceinline__ void window_yee(const FieldParams& Q, const RunDev& R, int run, unsigned phase, int p0, int L,
-                                           float (&F)[5][WMAX + 8], float (&mur)[8]) {
+// for the window's L elements, by all threads of the block; the same arithmetic as field_block.  J: the
+// current accumulators of the step, component c's element 0..L at J + c * WMAX.
+__device__ __forceinline__ void window_yee(const FieldParams& Q, const RunDev& R, int run, int p0, int L,
+                                           float (&F)[5][WMAX + 8], const unsigned long long* J, float (&mur)[8]) {
     const int tid = threadIdx.x, Nx = R.Nx, is = R.is;
-    const unsigned long long* const* J = R.J[current_set(R, phase, Q.nsets)];
     const float* inc = Q.inc + 6 * run;
     const float c = Q.c, hc = Q.hc, fdt = Q.fdt, fpi = R.fp_inv, fph = R.fp_inv * 4294967296.0f;
     const int n0 = p0 - PADF;  // node / half node of the window's element 0 (F[.][4])
@@ -223,10 +223,10 @@ __device__ __forceinline__ void window_yee(const FieldParams& Q, const RunDev& R
         yee_b(F[3][i], F[4][i], F[1][i], F[1][i + 1], F[2][i], F[2][i + 1], hc, n0 + i - 4 == is - 1, inc[0], inc[1]);
     __syncthreads();
     for (int i = tid + 4; i < L + 5; i += PUSH_T) {  // E^{n+1} on elements 0..L
-        const int node = n0 + i - 4, p = p0 + i - 4;
+        const int node = n0 + i - 4;
         float ey = F[1][i], ez = F[2][i];
-        yee_e(ey, ez, F[3][i - 1], F[3][i], F[4][i - 1], F[4][i], fix_to_float(__ldg(J[1] + p), fpi, fph),
-              fix_to_float(__ldg(J[2] + p), fpi, fph), c, fdt, node == is, inc[2], inc[3]);
+        yee_e(ey, ez, F[3][i - 1], F[3][i], F[4][i - 1], F[4][i], fix_to_float(J[WMAX + i - 4], fpi, fph),
+              fix_to_float(J[2 * WMAX + i - 4], fpi, fph), c, fdt, node == is, inc[2], inc[3]);
         const bool inner = node >= 1 && node <= Nx - 1;
         F[1][i] = inner ? ey : 0.f;
         F[2][i] = inner ? ez : 0.f;
@@ -248,7 +248,7 @@ __device__ __forceinline__ void window_yee(const FieldParams& Q, const RunDev& R
         const bool in = node >= 0 && node < Nx;
         F[3][i] = in ? by : 0.f;
         F[4][i] = in ? bz : 0.f;
-        F[0][i] = in ? fmaf(-fdt, fix_to_float(__ldg(J[0] + p0 + i - 4), fpi, fph), F[0][i]) : 0.f;
+        F[0][i] = in ? fmaf(-fdt, fix_to_float(J[i - 4], fpi, fph), F[0][i]) : 0.f;
     }
 }
 
@@ -257,12 +257,13 @@ __global__ void __launch_bounds__(PUSH_T, Slot<W>::MIN_BLOCKS) k_push_deposit(co
     using I = typename Slot<W>::I;
     using F = typename Slot<W>::F;
     __shared__ __align__(128) PushSmem<W> sm;
+    pdl_release<FUSED>();
     const unsigned phase = *P.phase + P.k;
     [[maybe_unused]] const unsigned before = phase + 5u;  // of the step before
     if constexpr (FUSED) {
         static_assert(W == 2 && sizeof(FieldSmem) <= sizeof(PushSmem<2>), "");
         if (static_cast<int>(blockIdx.x) < Q.nblk) {
-            field_block<PUSH_T>(Q, before, blockIdx.x, reinterpret_cast<FieldSmem&>(sm));
+            field_block<PUSH_T, true>(Q, before, blockIdx.x, reinterpret_cast<FieldSmem&>(sm));
             return;
         }
     }
@@ -272,8 +273,8 @@ __global__ void __launch_bounds__(PUSH_T, Slot<W>::MIN_BLOCKS) k_push_deposit(co
     __shared__ double sred[PUSH_T / 32];
 
     const int u = FUSED ? blockIdx.x - Q.nblk : blockIdx.x;
-    if (u >= P.units.count[0]) return;  // block-uniform
     const int run = P.units.run[u];
+    if (run < 0) return;  // block-uniform: behind the last unit
     const RunDev& R = P.runs[run];
     if (!R.active) return;
     const int tid = threadIdx.x, lane = tid & 31;
@@ -289,7 +290,7 @@ __global__ void __launch_bounds__(PUSH_T, Slot<W>::MIN_BLOCKS) k_push_deposit(co
     const int p0 = (w0 + PADF) & ~3;
     const int p1 = (w1 + PADF + 3) & ~3;
     const int L = p1 - p0;
-    if (L > WMAX || p0 < 0 || p1 > R.glen) {  // cannot happen for a valid unit table; never copy out of the arrays
+    if (L + 4 > WMAX || p0 < 4 || p1 + 4 > R.glen) {  // cannot happen for a valid unit table; never copy out of the arrays
         if (tid == 0) atomicOr(P.status, ST_WINDOW);
         return;
     }
@@ -300,26 +301,40 @@ __global__ void __launch_bounds__(PUSH_T, Slot<W>::MIN_BLOCKS) k_push_deposit(co
     const int base = start & ~(W - 1);
     const int nslots = (((end + W - 1) & ~(W - 1)) - base) / W;
 
-    for (int i = tid; i < 3 * WMAX; i += PUSH_T) {
-        (&sJ.lo[0][0])[i] = 0u;
-        (&sJ.hi[0][0])[i] = 0;
-    }
-    if (W == 2 && tid == 0) {
-        mbar_init(&bar, 1);
-        fence_mbar_init();
-        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-    }
-    __syncthreads();
+    auto clear_window = [&] {
+        for (int i = tid; i < L; i += PUSH_T)
+#pragma unroll
+            for (int c = 0; c < 3; ++c) {
+                sJ.lo[c][i] = 0u;
+                sJ.hi[c][i] = 0;
+            }
+    };
+    if constexpr (!FUSED) clear_window();
     const DevSpecies sp = R.sp[s][P.cur];
     if constexpr (W == 2) {
         if (tid == 0) {
-            // fused: with a halo of 4 elements (16 bytes) on each side, which lies inside the padded array
+            mbar_init(&bar, 1);
+            fence_mbar_init();
+            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+        }
+        pdl_wait<FUSED>();
+        if (tid == 0) {
+            // fused: with a halo of 4 elements (16 bytes) on each side, which lies inside the padded array, and
+            // with the step's current (the window it goes to is not in use yet)
             constexpr int H = FUSED ? 4 : 0;
-            const uint32_t bytes = static_cast<uint32_t>(L + 2 * H) * 4u;
-            mbar_arrive_expect_tx(&bar, 5u * bytes);
+            const uint32_t bytes = static_cast<uint32_t>(L + 2 * H) * 4u, jbytes = static_cast<uint32_t>(L + 4) * 8u;
+            mbar_arrive_expect_tx(&bar, 5u * bytes + (FUSED ? 3u * jbytes : 0u));
 #pragma unroll
             for (int c = 0; c < 5; ++c) tma_load_1d(&sm.F[c][4 - H], R.F[par][c] + p0 - H, bytes, &bar);
+            if constexpr (FUSED) {
+                static_assert(sizeof(Window) >= 3 * WMAX * sizeof(unsigned long long), "");
+                unsigned long long* const* J = R.J[current_set(R, before, Q.nsets)];
+#pragma unroll
+                for (int c = 0; c < 3; ++c)
+                    tma_load_1d(reinterpret_cast<unsigned long long*>(&sJ) + c * WMAX, J[c] + p0, jbytes, &bar);
+            }
         }
+        __syncthreads();
     } else {
         const float* const* Fg = R.F[par];
         for (int i = tid; i < L; i += PUSH_T) {
@@ -356,7 +371,9 @@ __global__ void __launch_bounds__(PUSH_T, Slot<W>::MIN_BLOCKS) k_push_deposit(co
         }
         if constexpr (FUSED) {
             __shared__ float mur[8];
-            window_yee(Q, R, run, before, p0, L, sm.F, mur);
+            window_yee(Q, R, run, p0, L, sm.F, reinterpret_cast<const unsigned long long*>(&sJ), mur);
+            __syncthreads();
+            clear_window();
             __syncthreads();
         }
     } else {
@@ -627,14 +644,14 @@ __global__ void __launch_bounds__(PUSH_T, Slot<W>::MIN_BLOCKS) k_push_deposit(co
 
 }  // namespace
 
-void launch_push(const PushParams& P, const FieldParams& Q, bool fused, int grid, int slot_w, cudaStream_t st) {
+void launch_push(const PushParams& P, const FieldParams& Q, bool fused, int grid, int slot_w, cudaStream_t st, bool pdl) {
     if (grid <= 0) return;
     if (slot_w == 2 && fused)
-        k_push_deposit<2, true><<<Q.nblk + grid, PUSH_T, 0, st>>>(P, Q);
+        launch(k_push_deposit<2, true>, dim3(Q.nblk + grid), PUSH_T, st, pdl, P, Q);
     else if (slot_w == 2)
-        k_push_deposit<2, false><<<grid, PUSH_T, 0, st>>>(P, Q);
+        launch(k_push_deposit<2, false>, dim3(grid), PUSH_T, st, false, P, Q);
     else
-        k_push_deposit<4, false><<<grid, PUSH_T, 0, st>>>(P, Q);
+        launch(k_push_deposit<4, false>, dim3(grid), PUSH_T, st, false, P, Q);
 }
 
 }  // namespace picrr

@@ -85,26 +85,31 @@ __global__ void __launch_bounds__(SORT_T) k_rad_flush(const RunDev* runs, int nr
 
 // ---- 1. per-unit window counts -------------------------------------------------
 // Blocks [0, nruns): a run's radiated partials; then a block per unit.
+template <bool PDL>
 __global__ void __launch_bounds__(SORT_T) k_sort_count(const SortParams S) {
     __shared__ int cnt[SSTR];
     __shared__ double sred[SORT_T / 32];
+    pdl_release<PDL>();
     const int u = static_cast<int>(blockIdx.x) - S.nruns;
     if (u < 0) {  // block-uniform
+        pdl_wait<PDL>();
         const int r = blockIdx.x;
         if (threadIdx.x < 2) S.rs_new[2 * r + threadIdx.x] = 0;  // entries of the new table, counted by the next launch
         rad_flush_block(S.runs, r, S.nruns, S.rs_units, S.rad_part, sred);
         return;
     }
-    if (u >= S.units.count[0]) return;
-    const RunDev& R = S.runs[S.units.run[u]];
+    const int run = S.units.run[u];
+    if (run < 0) return;  // block-uniform: behind the last unit
+    const RunDev& R = S.runs[run];
     if (!R.active) return;  // a run that ended keeps its particles where they are
     const int s = S.units.species[u];
     const int start = S.units.start[u], end = S.units.end[u];
     const int wb = S.units.lo[u] - S.k;
     const int L = min(S.units.hi[u] + S.k + 1 - wb, SSTR);
     for (int i = threadIdx.x; i < L; i += SORT_T) cnt[i] = 0;
-    __syncthreads();
     const int32_t* cell = R.sp[s][S.cur].cell;
+    pdl_wait<PDL>();
+    __syncthreads();
     constexpr int U = 8;  // loads in flight per thread
     for (int i0 = start; i0 < end; i0 += U * SORT_T) {
         int c[U];
@@ -191,11 +196,13 @@ __device__ __forceinline__ void count_entries(const SortParams& S, int run, int 
 }
 
 // grid (groups of the largest run, runs, species)
+template <bool PDL>
 __global__ void __launch_bounds__(PLAN_T, 4) k_sort_plan(const SortParams S) {
     __shared__ int sh[PLAN_T / 32];
     __shared__ int ks[SPAN + 1];
     __shared__ int slo[PLAN_UNITS], shi[PLAN_UNITS];
     __shared__ int sbase[2];
+    pdl_release<PDL>();
     const int run = blockIdx.y, s = blockIdx.z, g = blockIdx.x, tid = threadIdx.x;
     const RunDev& R = S.runs[run];
     const int C0 = g * SPAN;
@@ -210,6 +217,7 @@ __global__ void __launch_bounds__(PLAN_T, 4) k_sort_plan(const SortParams S) {
         shi[i] = S.units.hi[ua + i] + k;
     }
     if (tid < 2) sbase[tid] = 0;
+    pdl_wait<PDL>();
     __syncthreads();
     auto lo = [&](int i) { return staged ? slo[i] : S.units.lo[ua + i] - k; };  // windows, both non-decreasing
     auto hi = [&](int i) { return staged ? shi[i] : S.units.hi[ua + i] + k; };
@@ -266,19 +274,15 @@ __global__ void __launch_bounds__(PLAN_T, 4) k_sort_plan(const SortParams S) {
 struct FillSmem {
     int ks[SPAN + 1];
     int first[GROUP + 1];
-    int red[2];
+    int red[3];
 };
 __device__ __forceinline__ void fill_block(const SortParams& S, int run, int s, int g, FillSmem& F) {
     const RunDev& R = S.runs[run];
     const int C0 = g * SPAN, tid = threadIdx.x, np = 2 * S.nruns, p = 2 * run + s;
     const bool in = R.active && C0 < R.Nx;  // block-uniform
-    if (!in && (g > 0 || p > 0)) {
-        if (g == 0 && tid == 0) S.rs_new[np + p] = 0;  // (no entries)
-        return;
-    }
-    if (tid < 2) F.red[tid] = 0;
+    if (tid < 3) F.red[tid] = 0;
     __syncthreads();
-    // entries before this pair, and in all (for the table's count); entries of this pair before this group
+    // entries before this pair, and in all; entries of this pair before this group
     int before = 0, all = 0, prev = 0;
     for (int i = tid; i < np; i += SORT_T) {
         const int n = S.rs_new[i];
@@ -289,25 +293,25 @@ __device__ __forceinline__ void fill_block(const SortParams& S, int run, int s, 
         for (int i = tid; i < g; i += SORT_T) prev += R.group_n[s][i];
     before = __reduce_add_sync(FULL, before);
     prev = __reduce_add_sync(FULL, prev);
+    all = __reduce_add_sync(FULL, all);
     if ((tid & 31) == 0) {
         atomicAdd(&F.red[0], before);
         atomicAdd(&F.red[1], prev);
+        atomicAdd(&F.red[2], all);
     }
-    if (p == 0 && g == 0) {  // block-uniform
-        __shared__ int sall;
-        if (tid == 0) sall = 0;
-        __syncthreads();
-        all = __reduce_add_sync(FULL, all);
-        if ((tid & 31) == 0) atomicAdd(&sall, all);
-        __syncthreads();
-        if (tid == 0) {
-            S.fresh.count[0] = min(sall, S.max_units);
-            *S.phase = (*S.phase + S.k) % 6u;
-        }
-        if (!in) {
-            if (tid == 0) S.rs_new[np] = 0;
-            return;
-        }
+    __syncthreads();
+    all = min(F.red[2], S.max_units);
+    if (p == 0 && g == 0 && tid == 0) {
+        S.fresh.count[0] = all;
+        *S.phase = (*S.phase + S.k) % 6u;
+    }
+    // behind the last entry (each block of the launch a stretch)
+    for (int64_t i = all + static_cast<int64_t>(p * S.g_max + g) * SORT_T + tid; i < S.max_units;
+         i += static_cast<int64_t>(np) * S.g_max * SORT_T)
+        S.fresh.run[i] = -1;
+    if (!in) {
+        if (g == 0 && tid == 0) S.rs_new[np + p] = 0;  // (no entries)
+        return;
     }
     const int cells = min(SPAN, R.Nx - C0);
     for (int i = tid; i <= cells; i += SORT_T) F.ks[i] = R.keystart[s][C0 + i];
@@ -388,16 +392,20 @@ __device__ __forceinline__ int window_key(const int32_t* cell, int i, int we, in
 // A block per (species, run, group) for the new table, then a block per unit (the table
 // holds up to max_units, usually far fewer: behind their empty blocks the others came last,
 // 19 us later on thin plasma).
+template <bool PDL>
 __global__ void __launch_bounds__(SORT_T) k_sort_scatter(const SortParams S) {
     __shared__ int row[SC_W][SSTR];
+    pdl_release<PDL>();
     const int u = static_cast<int>(blockIdx.x) - 2 * S.nruns * S.g_max;
     if (u < 0) {  // block-uniform
+        pdl_wait<PDL>();
         const int v = blockIdx.x, q = v / S.g_max;
         fill_block(S, q >> 1, q & 1, v - q * S.g_max, reinterpret_cast<FillSmem&>(row));
         return;
     }
-    if (u >= S.units.count[0]) return;
-    const RunDev& R = S.runs[S.units.run[u]];
+    const int of_run = S.units.run[u];
+    if (of_run < 0) return;  // block-uniform: behind the last unit
+    const RunDev& R = S.runs[of_run];
     if (!R.active) return;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int s = S.units.species[u];
@@ -408,6 +416,7 @@ __global__ void __launch_bounds__(SORT_T) k_sort_scatter(const SortParams S) {
     const int per = (end - start + SC_W - 1) / SC_W;
     const int ws = min(end, start + warp * per), we = min(end, ws + per);
     for (int i = tid; i < SC_W * SSTR; i += SORT_T) (&row[0][0])[i] = 0;
+    pdl_wait<PDL>();
     __syncthreads();
     const unsigned lt = (1u << lane) - 1u;
     // pass 1: this warp's counts per cell
@@ -630,10 +639,10 @@ __global__ void __launch_bounds__(SORT_T) k_fill(const SortParams S) {
 
 }  // namespace
 
-void launch_sort(const SortParams& S, cudaStream_t st, int* launches) {
-    k_sort_count<<<S.max_units + S.nruns, SORT_T, 0, st>>>(S);
-    k_sort_plan<<<dim3(S.g_max, S.nruns, 2), PLAN_T, 0, st>>>(S);
-    k_sort_scatter<<<S.max_units + 2 * S.nruns * S.g_max, SORT_T, 0, st>>>(S);
+void launch_sort(const SortParams& S, cudaStream_t st, int* launches, bool pdl) {
+    launch(pdl ? k_sort_count<true> : k_sort_count<false>, dim3(S.max_units + S.nruns), SORT_T, st, pdl, S);
+    launch(pdl ? k_sort_plan<true> : k_sort_plan<false>, dim3(S.g_max, S.nruns, 2), PLAN_T, st, pdl, S);
+    launch(pdl ? k_sort_scatter<true> : k_sort_scatter<false>, dim3(S.max_units + 2 * S.nruns * S.g_max), SORT_T, st, pdl, S);
     *launches += 3;
 }
 

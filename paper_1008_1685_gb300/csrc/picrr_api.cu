@@ -1159,6 +1159,7 @@ pic_status chunk_graph(Batch* b, int cur, cudaGraphExec_t* out) {
     drop_graph(b, cur);
     const int I = b->sort_interval;
     const bool fz = fuses(b);
+    const bool pdl = fz && !b->timing;  // (events lie between the launches otherwise)
     cudaStream_t cs = b->cap_stream;
     std::vector<EventPair>& ev = b->graph_ev[cur];
     // timing on: an event-record node before and after each timed launch
@@ -1171,18 +1172,19 @@ pic_status chunk_graph(Batch* b, int cur, cudaGraphExec_t* out) {
     for (int j = 0; j < I; ++j) {
         const bool fused = fz && j > 0;
         mark(0, true);
-        launch_push(push_params(b, j, cur), field_params(b, j - 1, fused ? j - 1 : 0), fused, b->max_units, b->slot_w, cs);
+        launch_push(push_params(b, j, cur), field_params(b, j - 1, fused ? j - 1 : 0), fused, b->max_units, b->slot_w, cs,
+                    pdl && j > 0);
         mark(0, false);
         if (fz && j + 1 < I) continue;
         mark(1, true);
-        launch_field(field_params(b, j, j), b->nblk, cs);
+        launch_field(field_params(b, j, j), b->nblk, cs, pdl);
         mark(1, false);
     }
     mark(2, true);
     SortParams S = sort_params(b, cur, false);
     S.k = I;
     int nl = 0;
-    launch_sort(S, cs, &nl);
+    launch_sort(S, cs, &nl, pdl);
     mark(2, false);
     cudaGraph_t g = nullptr;
     cudaError_t e = cudaStreamEndCapture(cs, &g);

@@ -87,7 +87,7 @@ struct DevSpecies {
 };
 
 struct UnitTable {
-    int32_t* run;      // [max_units] run of the unit
+    int32_t* run;      // [max_units] run of the unit, -1 behind the last one
     int32_t* species;  // species of the unit
     int32_t* start;    // first particle index (in the run's arrays)
     int32_t* end;      // one past the last
@@ -213,14 +213,47 @@ __device__ __forceinline__ void tma_load_1d(void* dst_smem, const void* src_gmem
         : "memory");
 }
 
+// Programmatic dependent launch (no effect in a kernel launched without it): a kernel
+// lets the next one of the stream start as soon as all its own blocks run, and waits for
+// the previous one before it touches what that one wrote.  What stays the same from one
+// sort to the next (run table, unit table) is read before the wait.  Only the kernels of
+// fused steps have it, where a step is a chain of latencies (small run 13.6 -> 11.8 us per
+// step); in the others the instructions alone cost more (Yee kernel of thin plasma 13 ->
+// 16 us) than the overlap gave back.  Some block of every such kernel waits, so that
+// a kernel's end is never before its predecessor's.
+template <bool ON>
+__device__ __forceinline__ void pdl_release() {
+    if constexpr (ON) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+template <bool ON>
+__device__ __forceinline__ void pdl_wait() {
+    if constexpr (ON) asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+
+// Launch on st, with the next launch allowed to overlap as above when `pdl`.
+template <class... P, class... A>
+inline void launch(void (*kernel)(P...), dim3 grid, int threads, cudaStream_t st, bool pdl, const A&... args) {
+    cudaLaunchConfig_t c{};
+    c.gridDim = grid;
+    c.blockDim = dim3(static_cast<unsigned>(threads));
+    c.stream = st;
+    cudaLaunchAttribute a{};
+    a.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    a.val.programmaticStreamSerializationAllowed = 1;
+    c.attrs = &a;
+    c.numAttrs = pdl ? 1 : 0;
+    cudaLaunchKernelEx(&c, kernel, P(args)...);
+}
+
 // ---------------------------------------------------------------------------
 // Host-side launch wrappers (each defined in its own translation unit).
 // ---------------------------------------------------------------------------
 // slot_w: 4 or 2 particles per thread and round.  fused (slot_w 2 only): also the Yee update of the step
 // before, whose parameters are Q: the push's blocks update the fields of their own windows, and Q.nblk more
 // blocks in front write the new fields.
-void launch_push(const PushParams& P, const FieldParams& Q, bool fused, int grid, int slot_w, cudaStream_t st);
-void launch_field(const FieldParams& P, int grid, cudaStream_t st);
+void launch_push(const PushParams& P, const FieldParams& Q, bool fused, int grid, int slot_w, cudaStream_t st,
+                 bool pdl = false);
+void launch_field(const FieldParams& P, int grid, cudaStream_t st, bool pdl = false);
 void launch_zero_current(const FieldParams& P, cudaStream_t st);
 
 struct SortParams {
@@ -245,7 +278,7 @@ struct SortParams {
 // Full re-sort of every active run (bounded displacement since the last sort)
 // and the new unit table; particles move from buffer cur to 1 - cur, radiated
 // partials into the tallies.
-void launch_sort(const SortParams& S, cudaStream_t st, int* launches);
+void launch_sort(const SortParams& S, cudaStream_t st, int* launches, bool pdl = false);
 // Unit table S.fresh of every active run from its current, already sorted particles.
 void launch_build_units(const SortParams& S, cudaStream_t st, int* launches);
 // Add each run's per-unit radiated energy into its tally[0]; zero them.

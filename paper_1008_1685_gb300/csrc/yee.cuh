@@ -62,7 +62,7 @@ struct FieldSmem {
     float ney[FIELD_NODES + 2], nez[FIELD_NODES + 2];
 };
 
-template <int T>
+template <int T, bool PDL>
 __device__ __forceinline__ void field_block(const FieldParams& P, unsigned phase, int blk, FieldSmem& S) {
     constexpr int N = FIELD_NODES, K = N / T;
     const int tid = threadIdx.x;
@@ -79,6 +79,7 @@ __device__ __forceinline__ void field_block(const FieldParams& P, unsigned phase
     unsigned long long* const* Jnext = R.J[next];
     const float* inc = P.inc + 6 * run;
     const float c = P.c, hc = P.hc, fdt = P.fdt, fpi = R.fp_inv, fph = R.fp_inv * 4294967296.0f;
+    pdl_wait<PDL>();
 
     // Every load of the block is issued here, before the first barrier: the old fields and the
     // transverse current of the stencil (J on node i0-1+q kept in the register of the thread that
