@@ -45,39 +45,31 @@ constexpr unsigned FULL = 0xffffffffu;
 constexpr int kThinPerCell = PICRR_THIN_PER_CELL;
 
 // The unit's current window in shared memory holds exact 64-bit integer sums
-// (in the 2^lscale units of the records) as two 32-bit words, lo (unsigned)
-// and hi (signed): value = hi * 2^32 + lo.  A signed 32-bit term t is added
-// with a 32-bit atomic on lo, which returns the old word: the addition
-// wrapped (carried) iff old + t carries out of 32 bits, and hi then gets
-// sign(t) + carry (-1, 0 or +1; nothing in most cases).  Every carry is seen by
+// (in the 2^lscale units of the records) as two signed 32-bit words:
+// value = hi * 2^32 + lo.  A term t is added with a 32-bit atomic on lo, which
+// returns the old word: the addition wrapped iff old and t have one sign and
+// old + t the other, and hi then gets that sign.  Every wrap is seen by
 // exactly one adder, so the pair always holds the exact sum, in any order.
+// Sums stay around zero, so wraps are rare (with lo unsigned, every change of
+// the sum's sign was a carry: five more atomics a particle in thin plasma).
 // (A 64-bit shared-memory atomic runs at a sixth of the 32-bit rate.)
 struct Window {
-    unsigned lo[3][WMAX];  // Jx (half nodes), Jy, Jz (nodes)
+    int lo[3][WMAX];  // Jx (half nodes), Jy, Jz (nodes)
     int hi[3][WMAX];
 };
 
 __device__ __forceinline__ uint32_t win_addr(const Window& w) { return smem_u32(&w.lo[0][0]); }
 
-// Adds t to the window word at shared address `addr` + OFF.  Predicated
-// throughout: a branch per nonzero test made every add two divergence points
-// (the dense run of hot particles 0.717 ms with this, 0.759 ms with branches;
-// thin plasma 106 and 111 us).  Two additions without return (t to lo, t >> 12
-// to a coarse word that resolves the wraps) took thin plasma to 104 us but the
-// dense run to 0.755 ms.
-template <int OFF>
-__device__ __forceinline__ void win_add(uint32_t addr, int t) {
-    asm volatile(
-        "{\n\t.reg .pred p, q;\n\t.reg .u32 o, s, h;\n\t"
-        "setp.ne.s32 p, %1, 0;\n\t"
-        "mov.u32 o, 0;\n\t"
-        "@p atom.shared.add.u32 o, [%0 + %2], %1;\n\t"
-        "add.cc.u32 s, o, %1;\n\t"
-        "shr.s32 h, %1, 31;\n\t"
-        "addc.u32 h, h, 0;\n\t"
-        "setp.ne.s32 q, h, 0;\n\t"
-        "@q red.shared.add.u32 [%0 + %3], h;\n\t}" ::"r"(addr), "r"(t), "n"(OFF), "n"(OFF + 3 * WMAX * 4)
-        : "memory");
+// Adds t to the window word at shared address `addr`; negative if the word wrapped.
+__device__ __forceinline__ int win_add(uint32_t addr, int t) {
+    int old;
+    asm volatile("atom.shared.add.s32 %0, [%1], %2;" : "=r"(old) : "r"(addr), "r"(t) : "memory");
+    const int now = old + t;
+    return (old ^ now) & (t ^ now);
+}
+// The wrap's entry in hi.
+__device__ __forceinline__ void win_carry(uint32_t addr, int t) {
+    asm volatile("red.shared.add.s32 [%0], %1;" ::"r"(addr + 3 * WMAX * 4), "r"(t < 0 ? -1 : 1) : "memory");
 }
 
 // Position of value q of a stencil record anchored at key: q 0..2 are Jy at
@@ -86,17 +78,36 @@ __device__ __forceinline__ int rec_comp(int q) { return q < 3 ? 1 : (q < 6 ? 2 :
 __device__ __forceinline__ int rec_at(int key, int q) { return key + (q < 3 ? q : (q < 6 ? q - 3 : q - 6)); }
 
 // One lane's record added by itself: each value rounded to 32-bit fixed point
-// (records are kept in the window's units, |value| < 2^26).
+// (records are kept in the window's units, |value| < 2^26).  The wraps of its
+// values are collected as bits and looked at once: five instructions a value.
+// Values that are zero unless a particle crossed a cell boundary (node key + 2,
+// half node key + 1) are skipped when all are.  (Carries predicated after every
+// add, with lo unsigned, came out as two divergence points a value; two
+// additions without return, t to lo and t >> 12 to a coarse word that resolves
+// the wraps, took the dense run of hot particles 5 % longer.)
 __device__ __forceinline__ void lane_add(int key, const float (&v)[8], uint32_t w) {
     const uint32_t a = w + 4u * key;
-    win_add<4 * (WMAX + 0)>(a, __float2int_rn(v[0]));
-    win_add<4 * (WMAX + 1)>(a, __float2int_rn(v[1]));
-    win_add<4 * (WMAX + 2)>(a, __float2int_rn(v[2]));
-    win_add<4 * (2 * WMAX + 0)>(a, __float2int_rn(v[3]));
-    win_add<4 * (2 * WMAX + 1)>(a, __float2int_rn(v[4]));
-    win_add<4 * (2 * WMAX + 2)>(a, __float2int_rn(v[5]));
-    win_add<0>(a, __float2int_rn(v[6]));
-    win_add<4>(a, __float2int_rn(v[7]));
+    constexpr int at[8] = {4 * WMAX, 4 * (WMAX + 1), 4 * (WMAX + 2), 8 * WMAX, 4 * (2 * WMAX + 1), 4 * (2 * WMAX + 2), 0, 4};
+    unsigned wraps = 0u;
+    auto add = [&](int q) { wraps = __funnelshift_l(static_cast<unsigned>(win_add(a + at[q], __float2int_rn(v[q]))), wraps, 1); };
+    add(0);
+    add(1);
+    add(3);
+    add(4);
+    add(6);
+    if (v[2] != 0.f || v[5] != 0.f || v[7] != 0.f) {
+        add(2);
+        add(5);
+        add(7);
+    } else {
+        wraps <<= 3;
+    }
+    if (wraps) {
+        constexpr int bit[8] = {7, 6, 2, 5, 4, 1, 3, 0};
+#pragma unroll
+        for (int q = 0; q < 8; ++q)
+            if (wraps >> bit[q] & 1u) win_carry(a + at[q], __float2int_rn(v[q]));
+    }
 }
 
 // One stencil record per lane (key < 0: none).  When every lane holds the
@@ -119,7 +130,10 @@ __device__ __forceinline__ void warp_add(int key, const float (&v)[8], uint32_t 
                 const int t = __reduce_add_sync(FULL, __float2int_rn(v[q]));
                 mine = lane == q ? t : mine;
             }
-            if (lane < 8) win_add<0>(w + 4u * (rec_comp(lane) * WMAX + rec_at(k0, lane)), mine);
+            if (lane < 8) {
+                const uint32_t a = w + 4u * (rec_comp(lane) * WMAX + rec_at(k0, lane));
+                if (win_add(a, mine) < 0) win_carry(a, mine);
+            }
         }
     } else {
         // (summing the records of neighbouring lanes with one anchor first saves
@@ -144,17 +158,16 @@ __device__ __forceinline__ float div_ge1(float a, float x) {
 }
 
 __device__ __forceinline__ int comp(const int4& a, int j) { return j == 0 ? a.x : j == 1 ? a.y : j == 2 ? a.z : a.w; }
-__device__ __forceinline__ float comp(const float4& a, int j) {
-    return j == 0 ? a.x : j == 1 ? a.y : j == 2 ? a.z : a.w;
-}
+__device__ __forceinline__ float& comp(float4& a, int j) { return j == 0 ? a.x : j == 1 ? a.y : j == 2 ? a.z : a.w; }
 __device__ __forceinline__ int comp(const int2& a, int j) { return j == 0 ? a.x : a.y; }
-__device__ __forceinline__ float comp(const float2& a, int j) { return j == 0 ? a.x : a.y; }
+__device__ __forceinline__ float& comp(float2& a, int j) { return j == 0 ? a.x : a.y; }
 
 // A thread takes W consecutive particles per round (one W x 4-byte slot of each
 // array).  W = 4: 128-bit loads and stores, fewest instructions per particle,
 // for dense foils.  W = 2: 64-bit, fewer registers and so more warps per SM,
 // which hides the latency of deposits that scatter over many cells (thinly
-// spread particles).
+// spread particles): 48 registers for 5 CTAs an SM (6 of them, with 40, spill 20
+// words: 8 M thinly spread particles 105 us a push against 93).
 template <int W>
 struct Slot;
 template <>
@@ -162,8 +175,6 @@ struct Slot<4> {
     using I = int4;
     using F = float4;
     static constexpr int MIN_BLOCKS = 4;
-    static __device__ __forceinline__ I empty_i() { return make_int4(-1, -1, -1, -1); }
-    static __device__ __forceinline__ F zero_f() { return make_float4(0.f, 0.f, 0.f, 0.f); }
     static __device__ __forceinline__ I pack(const int (&v)[4]) { return make_int4(v[0], v[1], v[2], v[3]); }
     static __device__ __forceinline__ F pack(const float (&v)[4]) { return make_float4(v[0], v[1], v[2], v[3]); }
 };
@@ -171,9 +182,7 @@ template <>
 struct Slot<2> {
     using I = int2;
     using F = float2;
-    static constexpr int MIN_BLOCKS = 6;
-    static __device__ __forceinline__ I empty_i() { return make_int2(-1, -1); }
-    static __device__ __forceinline__ F zero_f() { return make_float2(0.f, 0.f); }
+    static constexpr int MIN_BLOCKS = 5;
     static __device__ __forceinline__ I pack(const int (&v)[2]) { return make_int2(v[0], v[1]); }
     static __device__ __forceinline__ F pack(const float (&v)[2]) { return make_float2(v[0], v[1]); }
 };
@@ -305,7 +314,7 @@ __global__ void __launch_bounds__(PUSH_T, Slot<W>::MIN_BLOCKS) k_push_deposit(co
         for (int i = tid; i < L; i += PUSH_T)
 #pragma unroll
             for (int c = 0; c < 3; ++c) {
-                sJ.lo[c][i] = 0u;
+                sJ.lo[c][i] = 0;
                 sJ.hi[c][i] = 0;
             }
     };
@@ -347,18 +356,17 @@ __global__ void __launch_bounds__(PUSH_T, Slot<W>::MIN_BLOCKS) k_push_deposit(co
         }
     }
 
+    const int rounds = (nslots + PUSH_T - 1) / PUSH_T;
     const float qm = R.qm[s], qw = R.qw[s];
     const float cfl = P.cfl, dt = P.dt, eps = P.eps;
     const float lscale = R.lscale[s];
     const int shift = R.lshift[s];
     const bool rr = s == 0 && R.rr != 0;
-    const int Nx = R.Nx;
     const float hq = 0.5f * qm * dt;
     // the record's factors carry the window's power-of-two scale, so that records
     // are summed in its units (an exact scaling: the same bits as scaling each sum)
     const float jxf = qw / cfl * lscale;  // q w dx / dt
     const float hqw = 0.5f * qw * lscale;
-    const int rounds = (nslots + PUSH_T - 1) / PUSH_T;
 
     if constexpr (W == 2) {
         const bool got = mbar_wait_bounded(&bar, 0);
@@ -381,23 +389,27 @@ __global__ void __launch_bounds__(PUSH_T, Slot<W>::MIN_BLOCKS) k_push_deposit(co
     }
 
     const bool thin = end - start < kThinPerCell * (hi - lo + 1);  // block-uniform
+    // particles can leave the box in this step (block-uniform)
+    const bool walls = lo - k <= 0 || hi + k >= R.Nx - 1;
+    const unsigned in_unit = static_cast<unsigned>(end - start);
     float rad_h = 0.f, rad_l = 0.f;  // energy radiated by this thread's particles
-    int rk = -1;  // running stencil record of this thread (anchor rk)
-    float rv[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
 
+    // Bound by the instructions issued (240 to 390 a particle).  So the body has no branch on a
+    // lane's own state but for the adds: every lane computes its slot's particles (lanes behind
+    // the last slot that one's), and those that are not the unit's, frozen or outside the window
+    // count for nothing.  With the adds above, and before -> after, us a push: a dense foil of
+    // 64 M hot particles 623 -> 545, 8 M thinly spread ones 107 -> 93, a batch of 48 small
+    // foils (8 M together) 116 -> 109.
     for (int r = 0; r < rounds; ++r) {
         const int slot = r * PUSH_T + tid;
-        const int b4 = base + W * slot;
-        const bool slot_ok = slot < nslots;
-        I c4 = Slot<W>::empty_i();
-        F o4 = Slot<W>::zero_f(), x4 = o4, y4 = o4, z4 = o4;
-        if (slot_ok) {
-            c4 = __ldcs(reinterpret_cast<const I*>(sp.cell + b4));
-            o4 = __ldcs(reinterpret_cast<const F*>(sp.off + b4));
-            x4 = __ldcs(reinterpret_cast<const F*>(sp.px + b4));
-            y4 = __ldcs(reinterpret_cast<const F*>(sp.py + b4));
-            z4 = __ldcs(reinterpret_cast<const F*>(sp.pz + b4));
-        }
+        if ((slot & ~31) >= nslots) break;  // the warp has no slot left
+        const int b4 = base + W * min(slot, nslots - 1);
+        const int rel = base + W * slot - start;
+        const I c4 = __ldcs(reinterpret_cast<const I*>(sp.cell + b4));
+        F o4 = __ldcs(reinterpret_cast<const F*>(sp.off + b4));
+        F x4 = __ldcs(reinterpret_cast<const F*>(sp.px + b4));
+        F y4 = __ldcs(reinterpret_cast<const F*>(sp.py + b4));
+        F z4 = __ldcs(reinterpret_cast<const F*>(sp.pz + b4));
         // the next round's slots into L2 while this round computes, so that its loads
         // wait on L2 rather than HBM: one bulk (TMA) prefetch per array for the whole
         // CTA, with an evict-first policy (the large run's push 0.483 -> 0.463 ms)
@@ -417,22 +429,36 @@ __global__ void __launch_bounds__(PUSH_T, Slot<W>::MIN_BLOCKS) k_push_deposit(co
         }
         int cn[W];
         float fo[W], qx[W], qy[W], qz[W];
-        bool act[W];
+        bool act[W], all = true;
 #pragma unroll
         for (int j = 0; j < W; ++j) {
-            const int idx = b4 + j;
-            int c = comp(c4, j);
-            float f = comp(o4, j);
-            float px = comp(x4, j), py = comp(y4, j), pz = comp(z4, j);
-            const int lb = c + PADF - p0;  // local bin of the particle's cell
-            bool a = slot_ok && idx >= start && idx < end && c >= 0;
-            if (a && (lb < 1 || lb > L - 3)) {  // outside the window: leave it, report
-                atomicOr(P.status, ST_WINDOW);
-                a = false;
+            const int c = comp(c4, j), lb = c + PADF - p0;
+            act[j] = static_cast<unsigned>(rel + j) < in_unit && c >= 0 &&
+                     static_cast<unsigned>(lb - 1) <= static_cast<unsigned>(L - 4);
+            all = all && act[j];
+        }
+        if (!all) {
+#pragma unroll
+            for (int j = 0; j < W; ++j) {
+                if (act[j]) continue;
+                // outside the window: left as it is, reported
+                if (static_cast<unsigned>(rel + j) < in_unit && comp(c4, j) >= 0) atomicOr(P.status, ST_WINDOW);
+                // whatever the slot holds must not reach the sums as a NaN
+                comp(o4, j) = comp(x4, j) = comp(y4, j) = comp(z4, j) = 0.f;
             }
-            int ka = -1;  // anchor of this particle's stencil record
-            float ay = 0.f, az = 0.f, w0 = 0.f, w1 = 0.f, w2 = 0.f, dj0 = 0.f, dj1 = 0.f;
-            if (a) {
+        }
+        int rk = -1;  // anchor of this thread's running stencil record
+        float rv[8];
+#pragma unroll
+        for (int j = 0; j < W; ++j) {
+            const int c = comp(c4, j);
+            const float f = comp(o4, j);
+            float px = comp(x4, j), py = comp(y4, j), pz = comp(z4, j);
+            const bool a = act[j];
+            const int lb = a ? c + PADF - p0 : 1;  // local bin of the particle's cell
+            int ka;  // anchor of this particle's stencil record
+            float ay, az, w0, w1, w2, dj0, dj1;
+            {
                 // --- linear gather: nodes (Ey, Ez) and half nodes (Ex, By, Bz)
                 const float h = f - 0.5f;
                 const int jb = h < 0.f ? lb - 1 : lb;
@@ -497,7 +523,8 @@ __global__ void __launch_bounds__(PUSH_T, Slot<W>::MIN_BLOCKS) k_push_deposit(co
                     const float gL = qL * rsqrt_ge1(qL), gN = qN * ign;
                     // rad_h + rad_l -= de without the rounding (Knuth): the tally must not depend on the
                     // units' size.  (One addition in double per round: thin plasma +3 %, the scan +4 %.)
-                    const float de = div_ge1(kx * (lx + px) + ky * (ly + py) + kz * (lz + pz), gL + gN);
+                    const float dg = div_ge1(kx * (lx + px) + ky * (ly + py) + kz * (lz + pz), gL + gN);
+                    const float de = a ? dg : 0.f;
                     const float t = __fsub_rn(rad_h, de), z = __fsub_rn(t, rad_h);
                     rad_l = __fadd_rn(rad_l, __fsub_rn(__fsub_rn(rad_h, __fsub_rn(t, z)), __fadd_rn(de, z)));
                     rad_h = t;
@@ -515,16 +542,16 @@ __global__ void __launch_bounds__(PUSH_T, Slot<W>::MIN_BLOCKS) k_push_deposit(co
                 const bool edge = fn >= 1.f;  // rounded up to the boundary: same point as (c, 0)
                 d = edge ? 0 : d;
                 fn = edge ? 0.f : fn;
-                int cnew = c + d, store_c = cnew;
-                if (cnew < 0) {  // frozen at x = 0 (sorts under cell 0)
-                    cnew = 0;
-                    fn = 0.f;
-                    d = 0;
-                    store_c = -1;
-                } else if (cnew >= Nx) {  // frozen at x = L (sorts under its last cell Nx-1)
-                    cnew = Nx;
-                    fn = 0.f;
-                    store_c = -Nx;
+                int cnew = c + d;
+                if (walls) {
+                    if (cnew < 0) {  // frozen at x = 0 (sorts under cell 0)
+                        fn = 0.f;
+                        d = 0;
+                        cnew = -1;
+                    } else if (cnew >= R.Nx) {  // frozen at x = L (sorts under its last cell Nx-1)
+                        fn = 0.f;
+                        cnew = -R.Nx;
+                    }
                 }
                 // --- stencil record anchored at a = min(old bin, new bin): Jy, Jz on
                 // nodes a..a+2 and Jx on half nodes a, a+1 (Esirkepov for linear shapes).
@@ -542,48 +569,52 @@ __global__ void __launch_bounds__(PUSH_T, Slot<W>::MIN_BLOCKS) k_push_deposit(co
                     w0 = s0a + s0b;
                     w2 = s2a + s2b;
                     w1 = (2.f - w0) - w2;
-                    const float hqi = hqw * ign;  // (q w / 2) / gamma in the window's units: ay = that times p_y
+                    const float hqi = (a ? hqw : 0.f) * ign;  // (q w / 2) / gamma in the window's units: ay = that times p_y
                     ay = hqi * py;
                     az = hqi * pz;
                     dj0 = s0a - s0b;
                     dj1 = s2b - s2a;
                 }
-                c = store_c;
-                f = fn;
+                cn[j] = cnew;
+                fo[j] = fn;
             }
             // merge the particle's record into this thread's running record; when
             // its anchor changes, the lane adds the finished record by itself: a warp
             // vote and a warp-wide sum at every change cost more, with 4 particles
             // per thread too (hot particles on a dense foil, whose anchors change
             // mid-round: 0.717 -> 0.633 ms)
-            const bool merge = ka < 0 || rk < 0 || ka == rk;
-            if (!merge) {
-                lane_add(rk, rv, wJ);
+            const float jxa = a ? jxf : 0.f;
+            if (j == 0) {
+                rk = a ? ka : -1;
+                rv[0] = ay * w0;
+                rv[1] = ay * w1;
+                rv[2] = ay * w2;
+                rv[3] = az * w0;
+                rv[4] = az * w1;
+                rv[5] = az * w2;
+                rv[6] = jxa * dj0;
+                rv[7] = jxa * dj1;
+            } else {
+                if (a && rk >= 0 && ka != rk) {
+                    lane_add(rk, rv, wJ);
 #pragma unroll
-                for (int q = 0; q < 8; ++q) rv[q] = 0.f;
-            }
-            if (ka >= 0) {  // the record's eight values, added to the running record
-                rk = ka;
+                    for (int q = 0; q < 8; ++q) rv[q] = 0.f;
+                }
+                rk = a ? ka : rk;
                 rv[0] = fmaf(ay, w0, rv[0]);
                 rv[1] = fmaf(ay, w1, rv[1]);
                 rv[2] = fmaf(ay, w2, rv[2]);
                 rv[3] = fmaf(az, w0, rv[3]);
                 rv[4] = fmaf(az, w1, rv[4]);
                 rv[5] = fmaf(az, w2, rv[5]);
-                rv[6] = fmaf(jxf, dj0, rv[6]);
-                rv[7] = fmaf(jxf, dj1, rv[7]);
+                rv[6] = fmaf(jxa, dj0, rv[6]);
+                rv[7] = fmaf(jxa, dj1, rv[7]);
             }
-            act[j] = a;
-            cn[j] = c;
-            fo[j] = f;
             qx[j] = px;
             qy[j] = py;
             qz[j] = pz;
         }
         warp_add(rk, rv, wJ, !thin);
-        rk = -1;
-#pragma unroll
-        for (int q = 0; q < 8; ++q) rv[q] = 0.f;
         // with 4 per thread (dense foils), a warp whose particles all stayed in
         // their cells leaves its cell slots as they are: a tenth of the written
         // bytes for most warps of a dense foil (the large run's push 0.440 ->
@@ -593,26 +624,24 @@ __global__ void __launch_bounds__(PUSH_T, Slot<W>::MIN_BLOCKS) k_push_deposit(co
         if constexpr (W == 4) {
             bool moved = false;
 #pragma unroll
-            for (int j = 0; j < W; ++j) moved = moved || cn[j] != comp(c4, j);
+            for (int j = 0; j < W; ++j) moved = moved || (act[j] && cn[j] != comp(c4, j));
             warp_moved = __any_sync(FULL, moved);
         }
-        if (slot_ok) {
-            if (b4 >= start && b4 + W - 1 < end) {
-                if (warp_moved) __stcs(reinterpret_cast<I*>(sp.cell + b4), Slot<W>::pack(cn));
-                __stcs(reinterpret_cast<F*>(sp.off + b4), Slot<W>::pack(fo));
-                __stcs(reinterpret_cast<F*>(sp.px + b4), Slot<W>::pack(qx));
-                __stcs(reinterpret_cast<F*>(sp.py + b4), Slot<W>::pack(qy));
-                __stcs(reinterpret_cast<F*>(sp.pz + b4), Slot<W>::pack(qz));
-            } else {
+        if (all) {
+            if (warp_moved) __stcs(reinterpret_cast<I*>(sp.cell + b4), Slot<W>::pack(cn));
+            __stcs(reinterpret_cast<F*>(sp.off + b4), Slot<W>::pack(fo));
+            __stcs(reinterpret_cast<F*>(sp.px + b4), Slot<W>::pack(qx));
+            __stcs(reinterpret_cast<F*>(sp.py + b4), Slot<W>::pack(qy));
+            __stcs(reinterpret_cast<F*>(sp.pz + b4), Slot<W>::pack(qz));
+        } else {
 #pragma unroll
-                for (int j = 0; j < W; ++j) {
-                    if (!act[j]) continue;
-                    sp.cell[b4 + j] = cn[j];
-                    sp.off[b4 + j] = fo[j];
-                    sp.px[b4 + j] = qx[j];
-                    sp.py[b4 + j] = qy[j];
-                    sp.pz[b4 + j] = qz[j];
-                }
+            for (int j = 0; j < W; ++j) {
+                if (!act[j]) continue;
+                sp.cell[b4 + j] = cn[j];
+                sp.off[b4 + j] = fo[j];
+                sp.px[b4 + j] = qx[j];
+                sp.py[b4 + j] = qy[j];
+                sp.pz[b4 + j] = qz[j];
             }
         }
     }
@@ -636,7 +665,7 @@ __global__ void __launch_bounds__(PUSH_T, Slot<W>::MIN_BLOCKS) k_push_deposit(co
     for (int i = tid; i < L; i += PUSH_T) {
 #pragma unroll
         for (int c = 0; c < 3; ++c) {
-            const long long v = static_cast<long long>((static_cast<unsigned long long>(static_cast<unsigned>(sJ.hi[c][i])) << 32) | sJ.lo[c][i]);
+            const long long v = static_cast<long long>(sJ.hi[c][i]) * 4294967296ll + sJ.lo[c][i];
             if (v) atomicAdd(R.J[cset][c] + p0 + i, static_cast<unsigned long long>(v) << shift);
         }
     }

@@ -77,3 +77,29 @@ def test_more_units_in_a_group_than_are_staged(picrr):
         g.close()
     for a, b in zip(*res):
         assert np.max(np.abs(a - b)) <= 1e-4 * max(1.0, np.max(np.abs(b)))
+
+
+@pytest.mark.parametrize("sign", [1.0, -1.0])
+@pytest.mark.parametrize("n,cells,spread", [(4001, 1, 0.0), (40_003, 5, 0.0), (40_003, 5, 3.0), (9_001, 3, 30.0)])
+def test_window_words_wrap(picrr, n, cells, spread, sign):
+    """Thousands of particles a cell drifting one way, cold (all lanes in one cell) and hot (anchors change
+    from particle to particle): a particle's record is up to 2^22 of the window's units, so the 32-bit words
+    wrap many times.  Against the oracle: each value carries a few roundings of 2^-24 (weights, 1/gamma,
+    product) and 2^-23 of the record: below 2e-6 also if they all go one way."""
+    import oracle
+
+    kw = dict(length_lambda=2, cells_per_lambda=100, cfl=0.95, lambda_um=0.8, source_node=8)
+    g, o = picrr.Sim(seed=1, sort_interval=8, **kw), oracle.OracleSim(**kw)
+    r = np.random.default_rng(n)
+    cell = (100 + r.integers(0, cells, n)).astype(np.int32)
+    off = r.random(n)
+    p = [sign * d + spread * r.normal(size=n) for d in (1.1, -2.3, 1.7)]
+    for s in (g, o):
+        s.load_particles(0, cell, off, *p, 0.01, -1.0, 1.0)
+        s.load_particles(1, cell[:1], off[:1], *(v[:1] * 0 for v in p), 1e-6, 1.0, 1836.0)
+    g.step(1)
+    o.step(1)
+    for c in (5, 6, 7):
+        a, b = g.field(c), o.field(c)
+        assert np.linalg.norm(a - b) <= 2e-6 * np.linalg.norm(b), c
+    g.close()
