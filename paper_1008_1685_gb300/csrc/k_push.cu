@@ -22,8 +22,9 @@
 // particles that share an anchor, in a fixed order; the record is then
 // converted to 32-bit fixed point and added to the unit's window in shared
 // memory with integer atomics, which hold exact 64-bit sums as pairs of 32-bit
-// words (when all lanes of a warp hold the same anchor, as in dense plasma,
-// the lanes are first summed exactly by an integer warp reduction).  At the
+// words (when all lanes of a warp hold one anchor or, with 4 particles per
+// thread, two, as in dense plasma, the lanes are first summed exactly by an
+// integer warp reduction).  At the
 // end the window is shifted to the 64-bit scale of the accumulators and added
 // to global memory with integer atomics.  Integer addition is exact and
 // associative, so the result does not depend on the order in which lanes,
@@ -406,7 +407,7 @@ __global__ void __launch_bounds__(PUSH_T, Slot<W>::MIN_BLOCKS) k_push_deposit(co
     const unsigned in_unit = static_cast<unsigned>(end - start);
     float rad_h = 0.f, rad_l = 0.f;  // energy radiated by this thread's particles
 
-    // Bound by the instructions issued (240 to 390 a particle).  So the body has no branch on a
+    // Bound by the instructions issued (225 to 300 a particle).  So the body has no branch on a
     // lane's own state but for the adds: every lane computes its slot's particles (lanes behind
     // the last slot that one's), and those that are not the unit's, frozen or outside the window
     // count for nothing.  With the adds above, and before -> after, us a push: a dense foil of

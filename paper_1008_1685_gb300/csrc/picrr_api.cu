@@ -829,9 +829,9 @@ void finalize_run_params(Batch* b, RunHost& r) {
 }
 
 // Particles per part of a unit for `total` particles in the batch's active runs.
-int part_size(int64_t total, int unit_p) {
+int part_size(int64_t total, int unit_p, int slot_w) {
     int p = PART_MIN;
-    while (p < unit_p && total > static_cast<int64_t>(p) * PARTS) p *= 2;
+    while (p < unit_p && total > static_cast<int64_t>(p) * (slot_w == 2 && p >= PART_EVEN ? PARTS_EVEN : PARTS)) p *= 2;
     return p;
 }
 
@@ -983,12 +983,12 @@ void do_sort(Batch* b) {
 // entry; a group or half is not merged only if it holds more than unit_p particles, which makes at most
 // groups + 4 n / unit_p pieces, and never more than the tiles.
 template <class Counts>
-int64_t units_needed(const Batch* b, int unit_p, Counts counts, int* part) {
+int64_t units_needed(const Batch* b, int unit_p, int slot_w, Counts counts, int* part) {
     int64_t total = 0, need = 1;
     for (const auto& r : b->runs)
         for (int s = 0; counts(r) && s < 2; ++s)
             if (r.sp[s].loaded) total += r.sp[s].n;
-    *part = part_size(total, unit_p);
+    *part = part_size(total, unit_p, slot_w);
     for (const auto& r : b->runs) {
         if (!counts(r)) continue;
         const int64_t ntiles = (r.Nx + TILE - 1) / TILE, groups = (r.Nx + SPAN - 1) / SPAN;
@@ -1022,7 +1022,7 @@ pic_status activate_pending(Batch* b) {
         if (b->runs[i].used && !b->runs[i].started && !b->runs[i].finished) joining.push_back(i);
     auto counts = [](const RunHost& r) { return r.used && !r.finished && (!r.started || r.active); };
     int part = 0;
-    const int64_t need = units_needed(b, b->unit_p, counts, &part);
+    const int64_t need = units_needed(b, b->unit_p, b->slot_w, counts, &part);
     if (need > (1 << 30)) return fail(b, PIC_ERR_INVALID_ARG, "too many work units");
     st = ensure_units(b, static_cast<int>(need));
     if (st != PIC_OK) return st;  // the joining runs stay pending
@@ -1338,12 +1338,12 @@ pic_status set_shapes(Batch* b, int unit_p, int interval, int slot_w) {
     if (st != PIC_OK) return st;
     bool any = false;
     for (auto& r : b->runs) any = any || (r.used && r.active);
-    if (unit_p != b->unit_p) {
+    int part = 0;
+    const int64_t need = units_needed(b, unit_p, slot_w, [](const RunHost& r) { return r.used && r.active; }, &part);
+    if (unit_p != b->unit_p || (slot_w != b->slot_w && part != b->part_p)) {
         // sort with the current table first (it also flushes the radiated
         // partials), then rebuild the table from the sorted cells with the new size
         if (any && b->since_sort > 0) do_sort(b);
-        int part = 0;
-        const int64_t need = units_needed(b, unit_p, [](const RunHost& r) { return r.used && r.active; }, &part);
         if (need > (1 << 30)) return fail(b, PIC_ERR_INVALID_ARG, "too many work units");
         if ((st = ensure_units(b, static_cast<int>(need))) != PIC_OK) return st;
         b->unit_p = unit_p;

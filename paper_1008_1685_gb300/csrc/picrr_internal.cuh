@@ -54,10 +54,17 @@ constexpr int PUSH_T = 256;       // threads of the push kernel
 // table entry of its own: about PARTS of them for all particles, none below PART_MIN (one round of the push).
 // One CTA per unit took 27 us for the 12 units of a small run, eight rounds one after the other; with parts
 // 12 us.
-// 1216 (8 CTAs on each of 152 SMs) against 608, 912 and 2432: the paper-scale run 27.0 us per step with 1216,
-// 27.7, 27.6 and 28.4 otherwise; the small run 15.7 with each.
+// 1216 (8 for each of 152 SMs; parts are a power of two, so that whole units can be put together from them)
+// against 760 and 2280: the paper-scale run 23.0 us per step with 1216 (799 units), 27.5 (410) and 26.8 (1581)
+// otherwise; the small run 11.3 with each.
 constexpr int PARTS = 1216;
 constexpr int PART_MIN = 512;
+// With 2 particles per thread (760 CTAs at a time), units of more than 4096 are cut down to that also while
+// they fill the GPU a few times only, so that the last CTAs end together: up to 5472 parts (7.2 rounds of CTAs).
+// us per push, units of 8192: 48 small foils (9.6 M particles) 109.5 -> 104.0, 96 of them 217 -> 210; of 16384:
+// dense foils of 6, 10 and 20 M 90.4 -> 86.9, 137 -> 121, 238 -> 228, of 32 M (parts of 8192) 349 -> 348.  Parts
+// of 2048 took 103 instead of 93 in thin plasma.  With 4 per thread a dense foil of 10 M went from 99.6 to 103.
+constexpr int PART_EVEN = 4096, PARTS_EVEN = 5472;
 constexpr int FUSE_UNITS = 456;  // units up to which a push also updates its fields (picrr_api.cu, fuses)
 constexpr int WMAX = SPAN + 2 * KMAX + 16;  // window length bound in the push kernel (>= SPAN + 2 KMAX + 9)
 constexpr int SSTR = SPAN + 2 * KMAX + 4;   // per-unit key-window stride of the sort scratch (>= SPAN + 2 KMAX)

@@ -54,6 +54,30 @@ def test_few_and_many_units_give_the_same_bits(picrr, cells, foil, ppc, interval
     beside.close()
 
 
+def test_units_cut_to_even_parts_give_the_same_bits(picrr):
+    """5.2M particles beside, units of 16384, 2 particles per thread: parts of 4096 (and whole units again with 4)."""
+    cpl, run = 100.0, dict(length_lambda=6.0, foil_x0=0.3, foil_thickness=4.0, ne=20.0, a0=80.0, polarization=picrr.CP,
+                           duration=3.0, steps=10**9, ppc=300, seed=5)
+    alone = picrr.Batch(cpl, max_runs=1, sort_interval=8)
+    ra = alone.add_run(**run)
+    alone.set_shapes(16384, 8, 2)
+    beside = picrr.Batch(cpl, max_runs=2, sort_interval=8)
+    beside.add_run(length_lambda=20.0, foil_x0=1.0, foil_thickness=10.0, ne=1.0, a0=1.0, polarization=0, duration=3.0,
+                   steps=10**9, ppc=2600, seed=6)
+    rb = beside.add_run(**run)
+    units = []
+    for w in (4, 2):
+        beside.set_shapes(16384, 8, w)
+        units.append(beside.stats()["n_units"])
+    assert units[1] > 1.8 * units[0]
+    for n in (8, 11):
+        assert alone.step(n) == n and beside.step(n) == n
+        for x, y in zip(state(alone, ra)[0], state(beside, rb)[0]):
+            assert np.array_equal(x, y)
+    alone.close()
+    beside.close()
+
+
 def test_more_units_in_a_group_than_are_staged(picrr):
     """1400 units of 1024 particles in 600 cells: the planning kernel reads their bounds from
     the table.  Shapes change the order of single-precision sums only: fields of order 1 after
