@@ -115,36 +115,24 @@ __device__ __forceinline__ void lane_add(int key, const float (&v)[8], uint32_t 
 // same anchor (dense plasma), the records are summed exactly in 32-bit fixed
 // point (|value| < 2^26 per lane, so the warp sum fits) by one integer warp
 // reduction per value and lanes 0..7 add the eight sums (the large run's push
-// 0.463 -> 0.450 ms against eight adds by lane 0); with TWO, when every lane
-// holds the anchor of lane 0 or of lane 31, lanes 8..15 add a second sum (64 M
-// hot particles, 4 a thread: 547 -> 540 us; with 2 a thread the registers cost
-// more, 95 -> 97 us in thin plasma and 110.5 -> 111.5 us in a batch of small
-// foils); otherwise every lane adds its own record.
-template <bool TWO>
+// 0.463 -> 0.450 ms against eight adds by lane 0); otherwise every lane adds
+// its own record.  (A reduction over lanes grouped by anchor runs once per
+// distinct anchor, which costs more than the lanes' own atomics as soon as
+// the warp holds two.)
 __device__ __forceinline__ void warp_add(int key, const float (&v)[8], uint32_t w, bool vote) {
-    const int k0 = __shfl_sync(FULL, key, 0), k1 = TWO ? __shfl_sync(FULL, key, 31) : k0;
-    if (vote && __all_sync(FULL, key == k0 || key == k1)) {
-        if (TWO || k0 >= 0) {
-            // lane q (q < 8) adds the warp sum of value q, lane 8 + q that of the second
-            // anchor: distinct words but for the nodes that two neighbouring stencils share
-            const int lane = threadIdx.x & 31, mq = lane & 7;
-            const bool first = !TWO || key == k0;
+    const int k0 = __shfl_sync(FULL, key, 0);
+    if (vote && __all_sync(FULL, key == k0)) {
+        if (k0 >= 0) {
+            // lane q (q < 8) adds the warp sum of value q: eight distinct words
+            const int lane = threadIdx.x & 31;
             int mine = 0;
 #pragma unroll
             for (int q = 0; q < 8; ++q) {
-                const int t = __reduce_add_sync(FULL, first ? __float2int_rn(v[q]) : 0);
+                const int t = __reduce_add_sync(FULL, __float2int_rn(v[q]));
                 mine = lane == q ? t : mine;
             }
-            if (TWO && k0 != k1) {
-#pragma unroll
-                for (int q = 0; q < 8; ++q) {
-                    const int t = __reduce_add_sync(FULL, first ? 0 : __float2int_rn(v[q]));
-                    mine = lane == 8 + q ? t : mine;
-                }
-            }
-            const int k = lane < 8 ? k0 : k1;
-            if (k >= 0 && lane < (TWO && k0 != k1 ? 16 : 8)) {
-                const uint32_t a = w + 4u * (rec_comp(mq) * WMAX + rec_at(k, mq));
+            if (lane < 8) {
+                const uint32_t a = w + 4u * (rec_comp(lane) * WMAX + rec_at(k0, lane));
                 if (win_add(a, mine) < 0) win_carry(a, mine);
             }
         }
@@ -627,7 +615,7 @@ __global__ void __launch_bounds__(PUSH_T, Slot<W>::MIN_BLOCKS) k_push_deposit(co
             qy[j] = py;
             qz[j] = pz;
         }
-        warp_add<W == 4>(rk, rv, wJ, !thin);
+        warp_add(rk, rv, wJ, !thin);
         // with 4 per thread (dense foils), a warp whose particles all stayed in
         // their cells leaves its cell slots as they are: a tenth of the written
         // bytes for most warps of a dense foil (the large run's push 0.440 ->

@@ -103,12 +103,11 @@ def test_more_units_in_a_group_than_are_staged(picrr):
         assert np.max(np.abs(a - b)) <= 1e-4 * max(1.0, np.max(np.abs(b)))
 
 
-@pytest.mark.parametrize("slots", [2, 4])
 @pytest.mark.parametrize("sign", [1.0, -1.0])
 @pytest.mark.parametrize("n,cells,spread", [(4001, 1, 0.0), (40_003, 5, 0.0), (40_003, 5, 3.0), (9_001, 3, 30.0)])
-def test_window_words_wrap(picrr, n, cells, spread, sign, slots):
-    """Thousands of particles a cell drifting one way, cold (a warp's lanes in one cell or two) and hot
-    (anchors change from particle to particle): a particle's record is up to 2^22 of the window's units, so the 32-bit words
+def test_window_words_wrap(picrr, n, cells, spread, sign):
+    """Thousands of particles a cell drifting one way, cold (all lanes in one cell) and hot (anchors change
+    from particle to particle): a particle's record is up to 2^22 of the window's units, so the 32-bit words
     wrap many times.  Against the oracle: each value carries a few roundings of 2^-24 (weights, 1/gamma,
     product) and 2^-23 of the record: below 2e-6 also if they all go one way."""
     import oracle
@@ -122,7 +121,6 @@ def test_window_words_wrap(picrr, n, cells, spread, sign, slots):
     for s in (g, o):
         s.load_particles(0, cell, off, *p, 0.01, -1.0, 1.0)
         s.load_particles(1, cell[:1], off[:1], *(v[:1] * 0 for v in p), 1e-6, 1.0, 1836.0)
-    g.set_shapes(4096, 8, slots)
     g.step(1)
     o.step(1)
     for c in (5, 6, 7):
