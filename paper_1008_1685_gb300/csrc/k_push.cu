@@ -22,9 +22,8 @@
 // particles that share an anchor, in a fixed order; the record is then
 // converted to 32-bit fixed point and added to the unit's window in shared
 // memory with integer atomics, which hold exact 64-bit sums as pairs of 32-bit
-// words (when all lanes of a warp hold one anchor or, with 4 particles per
-// thread, two, as in dense plasma, the lanes are first summed exactly by an
-// integer warp reduction).  At the
+// words (when all lanes of a warp hold the same anchor, as in dense plasma,
+// the lanes are first summed exactly by an integer warp reduction).  At the
 // end the window is shifted to the 64-bit scale of the accumulators and added
 // to global memory with integer atomics.  Integer addition is exact and
 // associative, so the result does not depend on the order in which lanes,
@@ -82,7 +81,12 @@ __device__ __forceinline__ int rec_at(int key, int q) { return key + (q < 3 ? q 
 // (records are kept in the window's units, |value| < 2^26).  The wraps of its
 // values are collected as bits and looked at once: five instructions a value.
 // Values that are zero unless a particle crossed a cell boundary (node key + 2,
-// half node key + 1) are skipped when all are.  (Carries predicated after every
+// half node key + 1) are skipped when all are, and Jz when it is zero (linear
+// polarization: 217 -> 203 us in the late phase of 96 small foils, half of them
+// so; adds of zeros to the few words that a warp's lanes share are not free).
+// A second integer reduction for a warp whose lanes hold two anchors was no
+// gain (a cold dense foil 411 -> 422, hot 540 -> 541, small foils 101 -> 109 us
+// a push).  (Carries predicated after every
 // add, with lo unsigned, came out as two divergence points a value; two
 // additions without return, t to lo and t >> 12 to a coarse word that resolves
 // the wraps, took the dense run of hot particles 5 % longer.)
@@ -93,9 +97,13 @@ __device__ __forceinline__ void lane_add(int key, const float (&v)[8], uint32_t 
     auto add = [&](int q) { wraps = __funnelshift_l(static_cast<unsigned>(win_add(a + at[q], __float2int_rn(v[q]))), wraps, 1); };
     add(0);
     add(1);
-    add(3);
-    add(4);
     add(6);
+    if (v[3] != 0.f || v[4] != 0.f) {
+        add(3);
+        add(4);
+    } else {
+        wraps <<= 2;
+    }
     if (v[2] != 0.f || v[5] != 0.f || v[7] != 0.f) {
         add(2);
         add(5);
@@ -104,7 +112,7 @@ __device__ __forceinline__ void lane_add(int key, const float (&v)[8], uint32_t 
         wraps <<= 3;
     }
     if (wraps) {
-        constexpr int bit[8] = {7, 6, 2, 5, 4, 1, 3, 0};
+        constexpr int bit[8] = {7, 6, 2, 4, 3, 1, 5, 0};
 #pragma unroll
         for (int q = 0; q < 8; ++q)
             if (wraps >> bit[q] & 1u) win_carry(a + at[q], __float2int_rn(v[q]));
@@ -399,8 +407,9 @@ __global__ void __launch_bounds__(PUSH_T, Slot<W>::MIN_BLOCKS) k_push_deposit(co
     // lane's own state but for the adds: every lane computes its slot's particles (lanes behind
     // the last slot that one's), and those that are not the unit's, frozen or outside the window
     // count for nothing.  With the adds above, and before -> after, us a push: a dense foil of
-    // 64 M hot particles 623 -> 545, 8 M thinly spread ones 107 -> 93, a batch of 48 small
-    // foils (8 M together) 116 -> 109.
+    // 64 M hot particles 623 -> 540, of cold ones 437 -> 411, 8 M thinly spread ones 107 -> 94,
+    // a batch of 48 small foils 116 -> 101 (with parts of 4096, PART_EVEN, which gave 5 of that),
+    // of 96 late in their runs 215 -> 203.
     for (int r = 0; r < rounds; ++r) {
         const int slot = r * PUSH_T + tid;
         if ((slot & ~31) >= nslots) break;  // the warp has no slot left

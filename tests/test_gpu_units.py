@@ -103,9 +103,10 @@ def test_more_units_in_a_group_than_are_staged(picrr):
         assert np.max(np.abs(a - b)) <= 1e-4 * max(1.0, np.max(np.abs(b)))
 
 
-@pytest.mark.parametrize("sign", [1.0, -1.0])
+@pytest.mark.parametrize("slots", [2, 4])
+@pytest.mark.parametrize("sign,planar", [(1.0, False), (-1.0, False), (1.0, True)])
 @pytest.mark.parametrize("n,cells,spread", [(4001, 1, 0.0), (40_003, 5, 0.0), (40_003, 5, 3.0), (9_001, 3, 30.0)])
-def test_window_words_wrap(picrr, n, cells, spread, sign):
+def test_window_words_wrap(picrr, n, cells, spread, sign, planar, slots):
     """Thousands of particles a cell drifting one way, cold (all lanes in one cell) and hot (anchors change
     from particle to particle): a particle's record is up to 2^22 of the window's units, so the 32-bit words
     wrap many times.  Against the oracle: each value carries a few roundings of 2^-24 (weights, 1/gamma,
@@ -118,9 +119,12 @@ def test_window_words_wrap(picrr, n, cells, spread, sign):
     cell = (100 + r.integers(0, cells, n)).astype(np.int32)
     off = r.random(n)
     p = [sign * d + spread * r.normal(size=n) for d in (1.1, -2.3, 1.7)]
+    if planar:  # no Jz, as with linear polarization
+        p[2] = 0 * p[2]
     for s in (g, o):
         s.load_particles(0, cell, off, *p, 0.01, -1.0, 1.0)
         s.load_particles(1, cell[:1], off[:1], *(v[:1] * 0 for v in p), 1e-6, 1.0, 1836.0)
+    g.set_shapes(4096, 8, slots)
     g.step(1)
     o.step(1)
     for c in (5, 6, 7):
