@@ -160,6 +160,7 @@ struct Batch {
 
     UnitTable units[2] = {};  // alternate with the particle buffers
     int max_units = 0;
+    int table_units = 0;  // unit table entries in use at most (<= max_units): what the launches cover
     double* rad_part = nullptr;
     uint16_t* cnt = nullptr;
     int32_t *offs = nullptr, *rs_units[2] = {};
@@ -886,7 +887,7 @@ SortParams sort_params(Batch* b, int cur, bool build) {
     S.status = b->d_status;
     S.k = b->since_sort;
     S.cur = cur;
-    S.max_units = b->max_units;
+    S.max_units = b->table_units;
     int mx = 1;
     for (auto& r : b->runs)
         if (r.used) mx = std::max(mx, r.Nx);
@@ -1028,6 +1029,10 @@ pic_status activate_pending(Batch* b) {
     if (st != PIC_OK) return st;  // the joining runs stay pending
     if (part != b->part_p) b->epoch++;
     b->part_p = part;
+    if (need > b->table_units) {  // with room to grow, as the graphs hold it
+        b->table_units = b->max_units;
+        b->epoch++;
+    }
     for (int i : joining) {
         RunHost& r = b->runs[i];
         finalize_run_params(b, r);
@@ -1172,7 +1177,7 @@ pic_status chunk_graph(Batch* b, int cur, cudaGraphExec_t* out) {
     for (int j = 0; j < I; ++j) {
         const bool fused = fz && j > 0;
         mark(0, true);
-        launch_push(push_params(b, j, cur), field_params(b, j - 1, fused ? j - 1 : 0), fused, b->max_units, b->slot_w, cs,
+        launch_push(push_params(b, j, cur), field_params(b, j - 1, fused ? j - 1 : 0), fused, b->table_units, b->slot_w, cs,
                     pdl && j > 0);
         mark(0, false);
         if (fz && j + 1 < I) continue;
@@ -1277,7 +1282,7 @@ pic_status batch_step(Batch* b, int64_t n, int64_t* done) {
         {
             Timed t(b, 0);
             launch_push(push_params(b, b->since_sort, b->cur), field_params(b, b->since_sort - 1, field_due ? inc_pos - 1 : 0),
-                        field_due, b->max_units, b->slot_w, b->stream);
+                        field_due, b->table_units, b->slot_w, b->stream);
         }
         b->launches++;
         inc_pos++;
@@ -1348,6 +1353,9 @@ pic_status set_shapes(Batch* b, int unit_p, int interval, int slot_w) {
         if ((st = ensure_units(b, static_cast<int>(need))) != PIC_OK) return st;
         b->unit_p = unit_p;
         b->part_p = part;
+        // no blocks for the entries that only smaller units needed (a table grown for units of 2048, as when
+        // tuning, cost the large run's push 424 -> 411 us: blocks without a unit run after the others)
+        b->table_units = static_cast<int>(need);
         if (any) {
             SortParams S = sort_params(b, b->cur, true);
             int nl = 0;

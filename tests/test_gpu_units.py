@@ -78,6 +78,29 @@ def test_units_cut_to_even_parts_give_the_same_bits(picrr):
     beside.close()
 
 
+@pytest.mark.parametrize("first", [1024, 16384])
+def test_table_in_use_shrinks_and_grows(picrr, first):
+    """Units of 1024, then of 16384 (fewer entries in use), then a run that joins: as that run alone."""
+    cpl, run = 100.0, dict(length_lambda=6.0, foil_x0=0.3, foil_thickness=4.0, ne=20.0, a0=80.0, polarization=picrr.CP,
+                           duration=3.0, steps=10**9, ppc=300, seed=5)
+    alone = picrr.Batch(cpl, max_runs=1, sort_interval=8)
+    ra = alone.add_run(**run)
+    alone.set_shapes(16384, 8, 4)
+    beside = picrr.Batch(cpl, max_runs=2, sort_interval=8)
+    beside.add_run(length_lambda=20.0, foil_x0=1.0, foil_thickness=10.0, ne=1.0, a0=1.0, polarization=0, duration=3.0,
+                   steps=10**9, ppc=2600, seed=6)
+    for unit in (first, 16384):
+        beside.set_shapes(unit, 8, 4)
+        assert beside.step(8) == 8
+    rb = beside.add_run(**run)
+    for n in (8, 19):
+        assert alone.step(n) == n and beside.step(n) == n
+        for x, y in zip(state(alone, ra)[0], state(beside, rb)[0]):
+            assert np.array_equal(x, y)
+    alone.close()
+    beside.close()
+
+
 def test_more_units_in_a_group_than_are_staged(picrr):
     """1400 units of 1024 particles in 600 cells: the planning kernel reads their bounds from
     the table.  Shapes change the order of single-precision sums only: fields of order 1 after
