@@ -203,7 +203,7 @@ struct Slot<2> {
 // and (Bz, dBz), so that a particle's gather is three loads and five FMAs
 // (the large run's push 0.451 -> 0.441 ms).  With 2 per thread (thin plasma,
 // few particles per cell) the components are copied as they are by bulk TMA,
-// and the smaller footprint keeps six CTAs per SM.
+// and the smaller footprint keeps five CTAs per SM.
 template <int W>
 struct PushSmem;
 template <>
