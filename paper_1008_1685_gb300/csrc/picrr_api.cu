@@ -1212,7 +1212,9 @@ pic_status batch_step(Batch* b, int64_t n, int64_t* done) {
     if ((st = upload_table(b)) != PIC_OK) return st;
     if ((st = upload_blocks(b)) != PIC_OK) return st;
     const int I = b->sort_interval;
-    bool fz = n > 0 && begin_steps(b);
+    // whether the coming steps are fused; asked again when a run has ended, but only once another step follows
+    // (begin_steps may clear the last step's currents, which stay readable until then)
+    bool fz = false, ask = true;
     int64_t it = 0;
     // laser source values of the single steps below, uploaded for up to KMAX
     // steps at a time (one copy instead of one per step); a graph launch
@@ -1236,6 +1238,8 @@ pic_status batch_step(Batch* b, int64_t n, int64_t* done) {
             if (r.steps_target > 0 && r.steps_target - r.steps_done < I) whole_chunk = false;
         }
         if (nact == 0) break;
+        if (ask) fz = begin_steps(b);
+        ask = false;
         if (whole_chunk) {
             // a whole sort interval as one graph launch; no run ends before its last step
             cudaGraphExec_t ex = nullptr;
@@ -1266,7 +1270,7 @@ pic_status batch_step(Batch* b, int64_t n, int64_t* done) {
                 }
                 if ((st = upload_table(b)) != PIC_OK) return st;
                 if ((st = upload_blocks(b)) != PIC_OK) return st;
-                fz = begin_steps(b);
+                ask = true;
             }
             cudaError_t e = cudaGetLastError();
             if (e != cudaSuccess) return cuda_fail(b, e, "chunk launch");
@@ -1308,7 +1312,7 @@ pic_status batch_step(Batch* b, int64_t n, int64_t* done) {
             }
             if ((st = upload_table(b)) != PIC_OK) return st;
             if ((st = upload_blocks(b)) != PIC_OK) return st;
-            fz = begin_steps(b);
+            ask = true;
         }
         if ((it & 255) == 255) {
             cudaError_t e = cudaGetLastError();
