@@ -306,7 +306,11 @@ NODE_COMPONENTS = (EY, EZ, JY, JZ)
 def _field(call, check, nx, comp):
     out = np.empty(nx + 1 if comp in NODE_COMPONENTS else nx)
     n = C.c_int64(0)
-    check(call(comp, len(out), _ptr(out), C.byref(n)))
+    rc = call(comp, len(out), _ptr(out), C.byref(n))
+    if rc != 0 and n.value > len(out):  # a box of an odd number of half cells: the library rounds up, round() to even
+        out = np.empty(n.value)
+        rc = call(comp, len(out), _ptr(out), C.byref(n))
+    check(rc)
     return out if n.value == len(out) else out[: n.value].copy()
 
 
