@@ -1,4 +1,4 @@
-"""The Python side of calls: sizes of field arrays."""
+"""The Python side of calls: sizes of field arrays and conversion of electron cases."""
 import ctypes as C
 
 import numpy as np
@@ -28,6 +28,29 @@ def test_field_takes_the_library_s_size(cells, comp):
     if cells == 20:  # a refusal for another reason stays one
         with pytest.raises(B.PicError):
             B._field(lambda *a: -1, check, 20, comp)
+
+
+def case(**kw):
+    return dict(dict(wave=0, a0=1.0, tau=2.0, x0=3.0, p0=(4.0, 5.0, 6.0)), **kw)
+
+
+@pytest.mark.parametrize("bad", [dict(a0=None), dict(tau=None), dict(x0=None), dict(p0=(1.0, None, 2.0)), dict(wave=None),
+                                 dict(a0=np.timedelta64(5, "s")), dict(p0={1.0, 2.0, 3.0}), dict(p0=(1.0, 2.0)),
+                                 dict(a0=1j)])
+def test_electron_cases_refuse_what_is_no_number(bad):
+    with pytest.raises((TypeError, IndexError)):
+        B._electron_cases([case(), case(**bad), case()])
+
+
+def test_electron_cases_keep_their_values():
+    odd = [case(p0=[1, 2.5, np.float32(3)]), case(p0=np.arange(3)), case(p0={0: 7.0, 1: 8.0, 2: 9.0}), case(p0=(1, 2, 3, 4)),
+           case(a0="1.5", wave="2"), {"wave": 1.9, "a0": True, "p0": (0, 0, 0)}, case(wave=2**32 + 1)]
+    for cases in ([], odd, [case(a0=k / 7, wave=k % 3) for k in range(50)], *[[c] for c in odd]):
+        got = B._electron_cases(cases)
+        assert len(got) == max(1, len(cases))
+        for a, c in zip(got, cases):
+            assert (a["wave"], a["a0"], a["tau"], a["x0"]) == (int(c["wave"]) % 2**32, float(c["a0"]), c.get("tau", 0.0), c.get("x0", 0.0))
+            assert list(a["p0"]) == [float(c["p0"][j]) for j in range(3)]
 
 
 @pytest.mark.gpu
