@@ -132,8 +132,10 @@ __device__ __forceinline__ void wave_at(const Wave& w, double phi, double& ey, d
         dey = -ez;
         dez = ey;
     } else {
+        // outside the pulse the field is zero at any phase, infinities and NaN too
         const bool in = phi >= 0.0 && phi <= w.tau;
-        sines<LANES, SHORT, DERIV, true, DERIV>(phi, in ? w.k * phi : 0.0, s, c, se, ce);
+        const double at = in ? phi : 0.0;
+        sines<LANES, SHORT, DERIV, true, DERIV>(at, w.k * at, s, c, se, ce);
         const double h = in ? w.a0 * se : 0.0;
         ey = h * se * c;
         if constexpr (DERIV) dey = h * (2.0 * w.k * ce * c - se * s);
@@ -253,7 +255,7 @@ __device__ __forceinline__ void leapfrog_step(const Wave& w, double t, double dt
 template <int KIND, bool RK4, bool RR, bool DERIV, int LANES>
 __device__ void integrate(const pic_electron_case& C, double dt, int64_t nsteps, int every, double eps, double* out,
                           int64_t nsamples) {
-    const Wave w{C.a0, C.tau, kPiD / C.tau};
+    const Wave w{C.a0, C.tau, fmin(kPiD / C.tau, 1e300)};  // (finite, so that 0 times it is 0)
     double x = C.x0, p[3] = {C.p0[0], C.p0[1], C.p0[2]};
     int64_t k = 0;
     int left = every;  // steps to the next row

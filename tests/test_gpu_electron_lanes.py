@@ -62,3 +62,15 @@ def test_large_phases(picrr, x0):
         for i, c in enumerate(few):
             b = reference(c, integrator, True, deriv, 0.01, 200, 50)
             assert off(a[i][:, 2:], b[:, 2:]) <= 1e-5, (x0, integrator, i)
+
+
+@pytest.mark.parametrize("pad", [0, 4900])  # four lanes an electron, one lane
+@pytest.mark.parametrize("integrator,rr,deriv", [(0, True, False), (0, False, False), (1, True, True), (1, False, False)])
+def test_no_field_outside_the_pulse_at_any_phase(picrr, integrator, rr, deriv, pad):
+    """An electron that no pulse reaches keeps its momentum bit for bit: at infinite or undefined phases,
+    and in a pulse so short that pi / tau is not finite."""
+    far = [dict(wave=2, a0=100.0, tau=40.0, x0=x0, p0=(0.5, -0.25, 2.0)) for x0 in (np.inf, -np.inf, np.nan, 5.0)]
+    short = dict(wave=2, a0=100.0, tau=1e-310, x0=0.0, p0=(0.0, 0.0, 0.0))
+    out = picrr.electron_scan(far + [short] + cases(pad), integrator=integrator, rr=rr, deriv=deriv, dt=0.01, nsteps=9, every=3)
+    assert np.all(out[:4, :, 2:] == (0.5, -0.25, 2.0)) and np.all(out[4, :, 1:] == 0.0)
+    assert np.all(out[0, :, 1] == np.inf) and np.all(out[1, :, 1] == -np.inf) and np.all(np.isnan(out[2, :, 1]))
