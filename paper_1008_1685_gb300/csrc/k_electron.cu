@@ -209,22 +209,23 @@ template <int KIND, bool RR>
 __device__ __forceinline__ void leapfrog_kick(double p[3], double ey, double ez, double dt, double eps) {
     constexpr bool Z = KIND == 1;  // the wave has an Ez
     const double h = -0.5 * dt;  // q/m (dt/2) for an electron
-    double e2 = ey * ey;
-    if constexpr (Z) e2 += ez * ez;
-    // Boris: half E kick, rotation about B (t = b (0, -ez, ey)), half E kick
+    // Boris: half E kick, rotation about B, half E kick.  t = (0, -tz, ty) is formed before it is squared or
+    // multiplied by a momentum, so that amplitudes above 1e154 do not overflow
     const double mx = p[0], my = p[1] + h * ey, mz = Z ? p[2] + h * ez : p[2];
     const double b = h * rsqrt_f64(1.0 + mx * mx + my * my + mz * mz);
-    const double s = 2.0 * b * rcp_f64(1.0 + b * b * e2);
+    const double ty = b * ey, tz = Z ? b * ez : 0.0;
+    double t2 = 1.0 + ty * ty;
+    if constexpr (Z) t2 += tz * tz;
+    const double s = 2.0 * rcp_f64(t2);
     // m' = m + m x t ; m+ = m + m' x (s t)
-    const double bx = b * mx;
-    const double uy = my - bx * ey, uz = Z ? mz - bx * ez : mz;
-    double me = my * ey, ue = uy * ey;
+    const double uy = my - mx * ty, uz = Z ? mz - mx * tz : mz;
+    double ux = mx + my * ty, ut = uy * ty;
     if constexpr (Z) {
-        me += mz * ez;
-        ue += uz * ez;
+        ux += mz * tz;
+        ut += uz * tz;
     }
-    const double sx = s * (mx + b * me);
-    const double pLx = mx + s * ue, pLy = (my - sx * ey) + h * ey, pLz = Z ? (mz - sx * ez) + h * ez : mz;
+    const double sx = s * ux;
+    const double pLx = mx + s * ut, pLy = (my - sx * ty) + h * ey, pLz = Z ? (mz - sx * tz) + h * ez : mz;
     if constexpr (!RR) {
         p[0] = pLx;
         p[1] = pLy;
@@ -237,6 +238,8 @@ __device__ __forceinline__ void leapfrog_kick(double p[3], double ey, double ez,
     const double vx = qx * iq, vy = qy * iq, vz = qz * iq;
     // Eq. (f_r): f_R = -eps { f_L x B - (v.E) E + gamma^2 [f_L^2 - (v.E)^2] v } with
     // f_L = -(E + v x B); the terms collapse as in ll_force
+    double e2 = ey * ey;
+    if constexpr (Z) e2 += ez * ez;
     const double u = 1.0 - vx, r = dt * eps * (u * e2), sq = g2 * u * r;
     // Eq. (pertfull): p^{n+1/2} = p_L^{n+1/2} + dt f_R
     p[0] = pLx + (r - sq * vx);

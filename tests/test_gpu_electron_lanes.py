@@ -74,3 +74,16 @@ def test_no_field_outside_the_pulse_at_any_phase(picrr, integrator, rr, deriv, p
     out = picrr.electron_scan(far + [short] + cases(pad), integrator=integrator, rr=rr, deriv=deriv, dt=0.01, nsteps=9, every=3)
     assert np.all(out[:4, :, 2:] == (0.5, -0.25, 2.0)) and np.all(out[4, :, 1:] == 0.0)
     assert np.all(out[0, :, 1] == np.inf) and np.all(out[1, :, 1] == -np.inf) and np.all(np.isnan(out[2, :, 1]))
+
+
+@pytest.mark.parametrize("pad", [0, 4900])
+@pytest.mark.parametrize("a0", [1e3, 1e153, 1e155, 1e200])
+def test_leapfrog_amplitudes_whose_square_overflows(picrr, a0, pad):
+    """Without radiation reaction no product in the step needs the square of the field: 20 steps agree with the
+    oracle's to a few roundings of 2^-53 a step, relative to the momenta's size."""
+    few = [dict(wave=w, a0=a0, tau=0.19, x0=0.0, p0=(0.0, 0.0, 0.0)) for w in (0, 1, 2)]
+    out = picrr.electron_scan(few + cases(pad), integrator=0, rr=False, dt=0.01, nsteps=20, every=1)
+    for i, c in enumerate(few):
+        b = reference(c, 0, False, False, 0.01, 20, 1)
+        assert np.all(np.isfinite(b)) and np.max(np.abs(b[:, 2:])) > 1e-3 * a0
+        assert off(out[i], b[:20]) <= 1e-13, (i, a0)
