@@ -27,6 +27,7 @@
 //     pulse needs four).
 // 4096 electrons x 2000 RK4 steps: 47.1 -> 18.5 ms; 20,000 x 1000 leapfrog steps:
 // 15.6 -> 4.7 ms.
+#include <new>
 #include <string>
 #include <vector>
 
@@ -353,6 +354,18 @@ extern "C" pic_status pic_electron_scan(const pic_electron_case* cases, int64_t 
         if (cases[c].wave < 0 || cases[c].wave > 2 || (cases[c].wave == 2 && !(cases[c].tau > 0.0)))
             return set_null_handle_error("bad wave (0, 1, or 2 with tau > 0)"), PIC_ERR_INVALID_ARG;
     if (n == 0) return PIC_OK;
+    // electrons grouped by the kind of their wave, each group padded to whole warps
+    std::vector<int32_t> order;
+    try {
+        order.reserve(static_cast<size_t>(n) + 3 * picrr::ELEC_T);
+    } catch (const std::bad_alloc&) {
+        return set_null_handle_error("out of host memory"), PIC_ERR_OOM;
+    }
+    for (int kind = 0; kind < 3; ++kind) {
+        for (int64_t c = 0; c < n; ++c)
+            if (cases[c].wave == kind) order.push_back(static_cast<int32_t>(c));
+        while (order.size() % picrr::ELEC_T) order.push_back(-1);
+    }
     int prev = -1;
     cudaGetDevice(&prev);
     if (cudaSetDevice(device) != cudaSuccess) {
@@ -364,14 +377,6 @@ extern "C" pic_status pic_electron_scan(const pic_electron_case* cases, int64_t 
     pic_electron_case* dc = nullptr;
     int32_t* dorder = nullptr;
     double* dout = nullptr;
-    // electrons grouped by the kind of their wave, each group padded to whole warps
-    std::vector<int32_t> order;
-    order.reserve(static_cast<size_t>(n) + 3 * picrr::ELEC_T);
-    for (int kind = 0; kind < 3; ++kind) {
-        for (int64_t c = 0; c < n; ++c)
-            if (cases[c].wave == kind) order.push_back(static_cast<int32_t>(c));
-        while (order.size() % picrr::ELEC_T) order.push_back(-1);
-    }
     const size_t out_bytes = static_cast<size_t>(n) * static_cast<size_t>(nsamples) * 5 * sizeof(double);
     cudaError_t e = cudaStreamCreateWithFlags(&st, cudaStreamNonBlocking);
     if (e == cudaSuccess) e = cudaMallocAsync(&dc, sizeof(pic_electron_case) * n, st);

@@ -1,5 +1,8 @@
 """The Python side of calls: sizes of field arrays and conversion of electron cases."""
 import ctypes as C
+import os
+import subprocess
+import sys
 
 import numpy as np
 import pytest
@@ -51,6 +54,26 @@ def test_electron_cases_keep_their_values():
         for a, c in zip(got, cases):
             assert (a["wave"], a["a0"], a["tau"], a["x0"]) == (int(c["wave"]) % 2**32, float(c["a0"]), c.get("tau", 0.0), c.get("x0", 0.0))
             assert list(a["p0"]) == [float(c["p0"][j]) for j in range(3)]
+
+
+def test_electron_scan_reports_a_lack_of_host_memory():
+    """An allocation that fails in the library comes back as an error of the call."""
+    from paper_1008_1685_gb300 import build
+
+    build.build()
+    code = """
+import resource
+import numpy as np
+from paper_1008_1685_gb300 import binding as B
+L, n = B.library(), 1 << 22
+cases, out = np.zeros(n, np.dtype(B.ElectronCase)), np.zeros(5)
+used = int(open("/proc/self/statm").read().split()[0]) * resource.getpagesize()
+resource.setrlimit(resource.RLIMIT_AS, (used + (4 << 20), resource.RLIM_INFINITY))
+print(L.pic_electron_scan(cases.ctypes.data, n, 1, 0, 0.01, 0, 1, 0.8, 0, out.ctypes.data, 0))
+"""
+    root = os.path.dirname(os.path.dirname(os.path.abspath(B.__file__)))
+    r = subprocess.run([sys.executable, "-c", code], cwd=root, capture_output=True, text=True)
+    assert (r.returncode, r.stdout.strip()) == (0, "-3"), r.stderr  # PIC_ERR_OOM
 
 
 @pytest.mark.gpu
