@@ -51,11 +51,11 @@ __device__ __forceinline__ int key_of(int c) { return c < 0 ? -1 - c : c; }
 __device__ __forceinline__ int groups_of(int Nx) { return (Nx + SPAN - 1) / SPAN; }
 
 // radiated energy of run r: sum of its electron units, fixed order (SORT_T threads)
-__device__ __forceinline__ void rad_flush_block(const RunDev* runs, int r, int nruns, const int32_t* rs_units, double* part,
-                                                double* sred) {
+__device__ __forceinline__ void rad_flush_block(const RunDev* runs, int r, int tab, double* part, double* sred) {
     const RunDev& R = runs[r];
     if (!R.active) return;
-    const int b = rs_units[2 * nruns + 2 * r], n = rs_units[2 * r];  // electron units
+    const int32_t* gf = R.group_first[0][tab];
+    const int b = gf[0], n = gf[groups_of(R.Nx)] - b;  // electron units
     const int t = threadIdx.x;
     double a[4] = {0.0, 0.0, 0.0, 0.0};
     for (int i = t; i < n; i += 4 * SORT_T) {
@@ -78,9 +78,17 @@ __device__ __forceinline__ void rad_flush_block(const RunDev* runs, int r, int n
     }
 }
 
-__global__ void __launch_bounds__(SORT_T) k_rad_flush(const RunDev* runs, int nruns, const int32_t* rs_units, double* part) {
+__global__ void __launch_bounds__(SORT_T) k_rad_flush(const RunDev* runs, int tab, double* part) {
     __shared__ double sred[SORT_T / 32];
-    rad_flush_block(runs, blockIdx.x, nruns, rs_units, part, sred);
+    rad_flush_block(runs, blockIdx.x, tab, part, sred);
+}
+
+// Sums of grp_n, counted up by count_entries: over each 256 groups, then over each 65536.
+__device__ __forceinline__ int sums1(const SortParams& S) { return (S.ngroups + 255) >> 8; }
+__device__ __forceinline__ int sums2(const SortParams& S) { return (S.ngroups + 65535) >> 16; }
+// cleared by block b of nb (SORT_T threads)
+__device__ __forceinline__ void clear_sums(const SortParams& S, int b, int nb) {
+    for (int i = b * SORT_T + threadIdx.x; i < sums1(S) + sums2(S); i += nb * SORT_T) S.grp_sum[i] = 0;
 }
 
 // ---- 1. per-unit window counts -------------------------------------------------
@@ -93,9 +101,8 @@ __global__ void __launch_bounds__(SORT_T) k_sort_count(const SortParams S) {
     const int u = static_cast<int>(blockIdx.x) - S.nruns;
     if (u < 0) {  // block-uniform
         pdl_wait<PDL>();
-        const int r = blockIdx.x;
-        if (threadIdx.x < 2) S.rs_new[2 * r + threadIdx.x] = 0;  // entries of the new table, counted by the next launch
-        rad_flush_block(S.runs, r, S.nruns, S.rs_units, S.rad_part, sred);
+        clear_sums(S, blockIdx.x, S.nruns);
+        rad_flush_block(S.runs, blockIdx.x, S.tab, S.rad_part, sred);
         return;
     }
     const int run = S.units.run[u];
@@ -177,8 +184,8 @@ __device__ __forceinline__ void tile_range(const int* ks, int cells, int t, int 
     }
 }
 
-// the group's entries, by the first GROUP threads (ks complete)
-__device__ __forceinline__ void count_entries(const SortParams& S, int run, int s, int g, const int* ks, int cells) {
+// the entries of group j, by the first GROUP threads (ks complete)
+__device__ __forceinline__ void count_entries(const SortParams& S, int j, const int* ks, int cells) {
     const int t = threadIdx.x;
     if (t >= 32) return;
     int n = 0;
@@ -190,12 +197,15 @@ __device__ __forceinline__ void count_entries(const SortParams& S, int run, int 
 #pragma unroll
     for (int o = 4; o > 0; o >>= 1) n += __shfl_xor_sync(FULL, n, o);
     if (t == 0) {
-        S.runs[run].group_n[s][g] = n;
-        if (n) atomicAdd(&S.rs_new[2 * run + s], n);
+        S.grp_n[j] = n;
+        if (n) {
+            atomicAdd(&S.grp_sum[j >> 8], n);
+            atomicAdd(&S.grp_sum[sums1(S) + (j >> 16)], n);
+        }
     }
 }
 
-// grid (groups of the largest run, runs, species)
+// a block per group
 template <bool PDL>
 __global__ void __launch_bounds__(PLAN_T, 4) k_sort_plan(const SortParams S) {
     __shared__ int sh[PLAN_T / 32];
@@ -203,11 +213,9 @@ __global__ void __launch_bounds__(PLAN_T, 4) k_sort_plan(const SortParams S) {
     __shared__ int slo[PLAN_UNITS], shi[PLAN_UNITS];
     __shared__ int sbase[2];
     pdl_release<PDL>();
-    const int run = blockIdx.y, s = blockIdx.z, g = blockIdx.x, tid = threadIdx.x;
-    const RunDev& R = S.runs[run];
-    const int C0 = g * SPAN;
-    if (!R.active || C0 >= R.Nx) return;  // block-uniform
-    const int cells = min(SPAN, R.Nx - C0), k = S.k;
+    const int j = blockIdx.x, pair = S.grp_pair[j], s = pair & 1, g = S.grp_at[j], tid = threadIdx.x;
+    const RunDev& R = S.runs[pair >> 1];
+    const int C0 = g * SPAN, cells = min(SPAN, R.Nx - C0), k = S.k;
     // units of the old table that can reach into the group (k < SPAN)
     const int32_t* gf = R.group_first[s][S.tab];
     const int ua = gf[max(g - 1, 0)], ub = gf[g + 2], nu = ub - ua;
@@ -265,58 +273,61 @@ __global__ void __launch_bounds__(PLAN_T, 4) k_sort_plan(const SortParams S) {
         at += S.cnt[q];
     }
     __syncthreads();
-    count_entries(S, run, s, g, ks, cells);
+    count_entries(S, j, ks, cells);
 }
 
-// ---- 4. the new unit table --------------------------------------------------------
+// ---- 3a. the new unit table -------------------------------------------------------
 // One block (SORT_T threads) per group: the table index of its first entry is the number of
-// entries of the pairs (run, species) and groups before it.
+// entries of the groups before it.  Of these it adds up the sums over 65536 and over 256 of them and
+// the rest one by one, so that a block reads at most 512 numbers and those few over 65536, whatever the
+// number of groups and of run slots (blocks for every slot, each reading the entries of all of them, made a step
+// of one run of 15,000 cells in a batch of 8192 slots 322 us long; it takes 13, and 11 with one slot).
 struct FillSmem {
     int ks[SPAN + 1];
     int first[GROUP + 1];
-    int red[3];
+    int red[2];
 };
-__device__ __forceinline__ void fill_block(const SortParams& S, int run, int s, int g, FillSmem& F) {
-    const RunDev& R = S.runs[run];
-    const int C0 = g * SPAN, tid = threadIdx.x, np = 2 * S.nruns, p = 2 * run + s;
-    const bool in = R.active && C0 < R.Nx;  // block-uniform
-    if (tid < 3) F.red[tid] = 0;
+// The table's blocks of a launch: one per group, and one if there is none (the phase advances in any case).
+__host__ __device__ __forceinline__ int fill_blocks(const SortParams& S) { return S.ngroups > 0 ? S.ngroups : 1; }
+
+__device__ __forceinline__ void fill_block(const SortParams& S, int j, FillSmem& F) {
+    const int tid = threadIdx.x;
+    if (tid < 2) F.red[tid] = 0;
     __syncthreads();
-    // entries before this pair, and in all; entries of this pair before this group
-    int before = 0, all = 0, prev = 0;
-    for (int i = tid; i < np; i += SORT_T) {
-        const int n = S.rs_new[i];
+    // entries before this group, and in all
+    const int n2 = sums2(S);
+    const int32_t *sum1 = S.grp_sum, *sum2 = sum1 + sums1(S);
+    int before = 0, all = 0;
+    for (int i = tid; i < n2; i += SORT_T) {
+        const int n = sum2[i];
         all += n;
-        before += i < p ? n : 0;
+        before += i < (j >> 16) ? n : 0;
     }
-    if (in)
-        for (int i = tid; i < g; i += SORT_T) prev += R.group_n[s][i];
+    for (int i = (j >> 16 << 8) + tid; i < (j >> 8); i += SORT_T) before += sum1[i];
+    for (int i = (j >> 8 << 8) + tid; i < j; i += SORT_T) before += S.grp_n[i];
     before = __reduce_add_sync(FULL, before);
-    prev = __reduce_add_sync(FULL, prev);
     all = __reduce_add_sync(FULL, all);
     if ((tid & 31) == 0) {
         atomicAdd(&F.red[0], before);
-        atomicAdd(&F.red[1], prev);
-        atomicAdd(&F.red[2], all);
+        atomicAdd(&F.red[1], all);
     }
     __syncthreads();
-    all = min(F.red[2], S.max_units);
-    if (p == 0 && g == 0 && tid == 0) {
+    all = min(F.red[1], S.max_units);
+    if (j == 0 && tid == 0) {
         S.fresh.count[0] = all;
         *S.phase = (*S.phase + S.k) % 6u;
     }
     // behind the last entry (each block of the launch a stretch)
-    for (int64_t i = all + static_cast<int64_t>(p * S.g_max + g) * SORT_T + tid; i < S.max_units;
-         i += static_cast<int64_t>(np) * S.g_max * SORT_T)
+    for (int64_t i = all + static_cast<int64_t>(j) * SORT_T + tid; i < S.max_units;
+         i += static_cast<int64_t>(fill_blocks(S)) * SORT_T)
         S.fresh.run[i] = -1;
-    if (!in) {
-        if (g == 0 && tid == 0) S.rs_new[np + p] = 0;  // (no entries)
-        return;
-    }
-    const int cells = min(SPAN, R.Nx - C0);
+    if (j >= S.ngroups) return;
+    const int run = S.grp_pair[j] >> 1, s = S.grp_pair[j] & 1, g = S.grp_at[j];
+    const RunDev& R = S.runs[run];
+    const int C0 = g * SPAN, cells = min(SPAN, R.Nx - C0);
     for (int i = tid; i <= cells; i += SORT_T) F.ks[i] = R.keystart[s][C0 + i];
     __syncthreads();
-    const int pair = F.red[0], base = pair + F.red[1];
+    const int base = F.red[0];
     if (tid < 32) {
         int a = 0, b = 0;
         if (tid < GROUP) tile_range(F.ks, cells, tid, S.unit_p, a, b);
@@ -332,10 +343,7 @@ __device__ __forceinline__ void fill_block(const SortParams& S, int run, int s, 
     __syncthreads();
     const int n = F.first[GROUP], G = groups_of(R.Nx);
     int32_t* gf = R.group_first[s][S.tab_new];
-    if (tid == 0) {
-        gf[g] = base;
-        if (g == 0) S.rs_new[np + p] = pair;
-    }
+    if (tid == 0) gf[g] = base;
     if (g == G - 1 && tid < 3) gf[G + tid] = base + n;
     for (int v = tid; v < n; v += SORT_T) {
         int t = 0;
@@ -370,7 +378,7 @@ __device__ __forceinline__ void fill_block(const SortParams& S, int run, int s, 
     }
 }
 
-// ---- 3. stable scatter ----------------------------------------------------------
+// ---- 3b. stable scatter ----------------------------------------------------------
 // Each warp owns one contiguous slice of the unit's particles.  Pass 1 counts
 // the slice's particles per cell (warp match; only the warp writes its row);
 // the rows are then turned into per-warp destination starts (unit offset plus
@@ -389,18 +397,17 @@ __device__ __forceinline__ int window_key(const int32_t* cell, int i, int we, in
     return (l >= 0 && l < SSTR) ? l : -1;  // out of window cannot happen (counted as an error)
 }
 
-// A block per (species, run, group) for the new table, then a block per unit (the table
+// A block per group for the new table, then a block per unit (the table
 // holds up to max_units, usually far fewer: behind their empty blocks the others came last,
 // 19 us later on thin plasma).
 template <bool PDL>
 __global__ void __launch_bounds__(SORT_T) k_sort_scatter(const SortParams S) {
     __shared__ int row[SC_W][SSTR];
     pdl_release<PDL>();
-    const int u = static_cast<int>(blockIdx.x) - 2 * S.nruns * S.g_max;
+    const int u = static_cast<int>(blockIdx.x) - fill_blocks(S);
     if (u < 0) {  // block-uniform
         pdl_wait<PDL>();
-        const int v = blockIdx.x, q = v / S.g_max;
-        fill_block(S, q >> 1, q & 1, v - q * S.g_max, reinterpret_cast<FillSmem&>(row));
+        fill_block(S, blockIdx.x, reinterpret_cast<FillSmem&>(row));
         return;
     }
     const int of_run = S.units.run[u];
@@ -613,7 +620,7 @@ __global__ void __launch_bounds__(KEY_T) k_keystart(const SortParams S) {
 __global__ void k_zero_keycount(const SortParams S) {
     const RunDev& R = S.runs[blockIdx.y];
     const int s = blockIdx.z;
-    if (blockIdx.x == 0 && threadIdx.x == 0) S.rs_new[2 * blockIdx.y + s] = 0;
+    if (blockIdx.y == 0 && s == 0) clear_sums(S, blockIdx.x, gridDim.x);
     if (!R.active) return;
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < R.Nx + 2; i += gridDim.x * blockDim.x)
         R.keycount[s][i] = 0;
@@ -622,27 +629,25 @@ __global__ void k_zero_keycount(const SortParams S) {
 // entries of every group, from the cell starts
 __global__ void __launch_bounds__(SORT_T) k_group_entries(const SortParams S) {
     __shared__ int ks[SPAN + 1];
-    const RunDev& R = S.runs[blockIdx.y];
-    const int s = blockIdx.z, C0 = blockIdx.x * SPAN;
-    if (!R.active || C0 >= R.Nx) return;  // block-uniform
+    const int j = blockIdx.x, s = S.grp_pair[j] & 1, C0 = S.grp_at[j] * SPAN;
+    const RunDev& R = S.runs[S.grp_pair[j] >> 1];
     const int cells = min(SPAN, R.Nx - C0);
     for (int i = threadIdx.x; i <= cells; i += SORT_T) ks[i] = R.keystart[s][C0 + i];
     __syncthreads();
-    count_entries(S, blockIdx.y, s, blockIdx.x, ks, cells);
+    count_entries(S, j, ks, cells);
 }
 
 __global__ void __launch_bounds__(SORT_T) k_fill(const SortParams S) {
     __shared__ FillSmem F;
-    const int q = blockIdx.x / S.g_max;
-    fill_block(S, q >> 1, q & 1, blockIdx.x - q * S.g_max, F);
+    fill_block(S, blockIdx.x, F);
 }
 
 }  // namespace
 
 void launch_sort(const SortParams& S, cudaStream_t st, int* launches, bool pdl) {
     launch(pdl ? k_sort_count<true> : k_sort_count<false>, dim3(S.max_units + S.nruns), SORT_T, st, pdl, S);
-    launch(pdl ? k_sort_plan<true> : k_sort_plan<false>, dim3(S.g_max, S.nruns, 2), PLAN_T, st, pdl, S);
-    launch(pdl ? k_sort_scatter<true> : k_sort_scatter<false>, dim3(S.max_units + 2 * S.nruns * S.g_max), SORT_T, st, pdl, S);
+    if (S.ngroups > 0) launch(pdl ? k_sort_plan<true> : k_sort_plan<false>, dim3(S.ngroups), PLAN_T, st, pdl, S);
+    launch(pdl ? k_sort_scatter<true> : k_sort_scatter<false>, dim3(S.max_units + fill_blocks(S)), SORT_T, st, pdl, S);
     *launches += 3;
 }
 
@@ -653,13 +658,13 @@ void launch_build_units(const SortParams& S, cudaStream_t st, int* launches) {  
     k_block_sums<<<kg, KEY_T, 0, st>>>(S);
     k_scan_blocks<<<dim3(S.nruns, 2), SCAN_T, 0, st>>>(S);
     k_keystart<<<kg, KEY_T, 0, st>>>(S);
-    k_group_entries<<<dim3(S.g_max, S.nruns, 2), SORT_T, 0, st>>>(S);
-    k_fill<<<2 * S.nruns * S.g_max, SORT_T, 0, st>>>(S);
+    if (S.ngroups > 0) k_group_entries<<<S.ngroups, SORT_T, 0, st>>>(S);
+    k_fill<<<fill_blocks(S), SORT_T, 0, st>>>(S);
     *launches += 7;
 }
 
-void launch_rad_flush(const RunDev* runs, int nruns, const int32_t* rs_units, double* rad_part, cudaStream_t st) {
-    k_rad_flush<<<nruns, SORT_T, 0, st>>>(runs, nruns, rs_units, rad_part);
+void launch_rad_flush(const RunDev* runs, int nruns, int tab, double* rad_part, cudaStream_t st) {
+    k_rad_flush<<<nruns, SORT_T, 0, st>>>(runs, tab, rad_part);
 }
 
 // ---- foil loader -------------------------------------------------------------

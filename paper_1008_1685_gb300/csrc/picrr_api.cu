@@ -131,9 +131,14 @@ struct Batch {
     char* pinned = nullptr;    // one pinned allocation for h_runs, h_inc and stage
     RunDev* h_runs = nullptr;  // pinned staging of the run table
     char* stage = nullptr;     // pinned, kStage bytes: small read-outs (kernels and copies write it directly)
-    int32_t* d_blk_run = nullptr;
-    int32_t* d_blk_i0 = nullptr;
-    int nblk = 0, blk_cap = 0;
+    // the layout of the active runs (upload_blocks), one allocation: the blocks of the Yee kernel, then the
+    // groups of the sort and its scratch for them (SortParams)
+    int32_t* layout = nullptr;
+    size_t layout_cap = 0;
+    int32_t *d_blk_run = nullptr, *d_blk_i0 = nullptr;
+    int nblk = 0;
+    int32_t *d_grp_pair = nullptr, *d_grp_at = nullptr, *grp_n = nullptr, *grp_sum = nullptr;
+    int ngroups = 0;
     float* d_inc = nullptr;  // [KMAX][max_runs * 6]
     float* h_inc = nullptr;  // pinned ring [kIncRing][KMAX][max_runs * 6]
     cudaEvent_t inc_ev[kIncRing] = {};
@@ -163,7 +168,7 @@ struct Batch {
     int table_units = 0;  // unit table entries in use at most (<= max_units): what the launches cover
     double* rad_part = nullptr;
     uint16_t* cnt = nullptr;
-    int32_t *offs = nullptr, *rs_units[2] = {};
+    int32_t* offs = nullptr;
     int* d_status = nullptr;
     unsigned* d_phase = nullptr;  // batch step of the last sort mod 6, advanced by the sort
     double* diag_partials = nullptr;
@@ -422,7 +427,6 @@ pic_status batch_create(const pic_config* cfg, int max_runs, Batch** out) {
     slab.add(&b->d_phase, 1);
     slab.add(&b->diag_partials, 3 * kMaxDiagBlocks);
     slab.add(&b->snap_out, 4);
-    for (int32_t*& t : b->rs_units) slab.add(&t, static_cast<size_t>(4) * max_runs);
     if ((st = dalloc_slab(b, b->mem, slab)) != PIC_OK) {
         g_null_error = b->err;
         batch_destroy(b);
@@ -521,7 +525,6 @@ pic_status run_open(Batch* b, double length_lambda, int source_node, int rr_on, 
         slab.add(&d.keystart[s], nk);
         slab.add(&d.blocksum[s], nkb);
         slab.add(&d.blockstart[s], nkb);
-        slab.add(&d.group_n[s], ngr);
         for (int32_t*& g : d.group_first[s]) slab.add(&g, ngr);
     }
     const pic_status st = dalloc_slab(b, r.mem, slab);
@@ -545,7 +548,7 @@ size_t run_footprint_cpl(double cells_per_lambda, double length_lambda, int64_t 
     size_t t = 10 * rounded(glen * 4) + 9 * rounded(glen * 8) + rounded(32);
     const size_t nk = static_cast<size_t>(Nx) + 2, nkb = static_cast<size_t>(Nx) / KEY_T + 2,
                  ngr = static_cast<size_t>(Nx) / SPAN + 4;
-    t += 2 * (2 * rounded(nk * 4) + 2 * rounded(nkb * 4) + 3 * rounded(ngr * 4));
+    t += 2 * (2 * rounded(nk * 4) + 2 * rounded(nkb * 4) + 2 * rounded(ngr * 4));
     const size_t cap = static_cast<size_t>((n + 3) / 4 * 4 + 8);
     t += 2 * 2 * 6 * rounded(cap * 4);
     const int64_t ntiles = (Nx + TILE - 1) / TILE;
@@ -554,7 +557,7 @@ size_t run_footprint_cpl(double cells_per_lambda, double length_lambda, int64_t 
                                             std::min<int64_t>(2 * ((n + PART_MIN - 1) / PART_MIN), PARTS));
     const size_t units = static_cast<size_t>(parts + 2 * (ntiles + 1));
     t += units * (2 * 6 * 4 + 8 + SSTR * 6) * 3 / 2;
-    t += static_cast<size_t>(Nx / FIELD_NODES + 1) * 8 * 3 / 2;
+    t += (static_cast<size_t>(Nx / FIELD_NODES + 1) * 8 + 2 * ngr * 14) * 3 / 2;  // layout
     return t;
 }
 
@@ -881,8 +884,11 @@ SortParams sort_params(Batch* b, int cur, bool build) {
     S.fresh = b->units[S.tab_new];
     S.cnt = b->cnt;
     S.offs = b->offs;
-    S.rs_units = b->rs_units[S.tab];
-    S.rs_new = b->rs_units[S.tab_new];
+    S.grp_pair = b->d_grp_pair;
+    S.grp_at = b->d_grp_at;
+    S.grp_n = b->grp_n;
+    S.grp_sum = b->grp_sum;
+    S.ngroups = b->ngroups;
     S.rad_part = b->rad_part;
     S.status = b->d_status;
     S.k = b->since_sort;
@@ -892,7 +898,6 @@ SortParams sort_params(Batch* b, int cur, bool build) {
     for (auto& r : b->runs)
         if (r.used) mx = std::max(mx, r.Nx);
     S.kb_max = (mx + KEY_T - 1) / KEY_T;
-    S.g_max = (mx + SPAN - 1) / SPAN;
     S.unit_p = b->unit_p;
     S.phase = b->d_phase;
     S.part_p = b->part_p;
@@ -919,49 +924,62 @@ pic_status upload_table(Batch* b) {
     return PIC_OK;
 }
 
-// Block table of the Yee kernel: FIELD_NODES nodes of one active run per block.
+// Blocks of the Yee kernel (FIELD_NODES nodes of one active run each), and the groups of the sort (SPAN cells of
+// one active run and species each).  The cells' own arrays fill the memory long before the counts leave 32 bits.
 pic_status upload_blocks(Batch* b) {
     if (!b->layout_dirty) return PIC_OK;
-    std::vector<int32_t> br, bi;
+    size_t nb = 0, ng = 0;
+    for (const RunHost& r : b->runs) {
+        if (!r.used || !r.active) continue;
+        nb += static_cast<size_t>(r.Nx / FIELD_NODES + 1);
+        ng += static_cast<size_t>(2) * ((r.Nx + SPAN - 1) / SPAN);
+    }
+    const size_t sent = 2 * (nb + ng), all = sent + ng + (ng / 256 + 1) + (ng / 65536 + 1);
+    std::vector<int32_t> h(sent);
+    int32_t *run = h.data(), *i0 = run + nb, *pair = i0 + nb, *at = pair + ng;
     for (int i = 0; i < b->max_runs; ++i) {
         const RunHost& r = b->runs[i];
         if (!r.used || !r.active) continue;
-        for (int i0 = 0; i0 <= r.Nx; i0 += FIELD_NODES) {
-            br.push_back(i);
-            bi.push_back(i0);
+        for (int q = 0; q <= r.Nx / FIELD_NODES; ++q) {
+            *run++ = i;
+            *i0++ = q * FIELD_NODES;
         }
+        for (int s = 0; s < 2; ++s)
+            for (int g = 0; g < (r.Nx + SPAN - 1) / SPAN; ++g) {
+                *pair++ = 2 * i + s;
+                *at++ = g;
+            }
     }
-    const int n = static_cast<int>(br.size());
-    if (n > b->blk_cap) {
+    if (all > b->layout_cap) {
         std::vector<std::pair<void*, size_t>> fresh;
-        int32_t *a = nullptr, *c = nullptr;
-        pic_status st = dalloc_t(b, fresh, &a, static_cast<size_t>(n));
-        if (st == PIC_OK) st = dalloc_t(b, fresh, &c, static_cast<size_t>(n));
-        if (st != PIC_OK) {
-            free_all(b, fresh);
-            return st;
-        }
-        free_one(b, b->d_blk_run);
-        free_one(b, b->d_blk_i0);
-        for (auto& f : fresh) b->mem.push_back(f);
-        b->d_blk_run = a;
-        b->d_blk_i0 = c;
-        b->blk_cap = n;
+        int32_t* a = nullptr;
+        const pic_status st = dalloc_t(b, fresh, &a, all);
+        if (st != PIC_OK) return st;
+        free_one(b, b->layout);
+        b->mem.push_back(fresh[0]);
+        b->layout = a;
+        b->layout_cap = all;
     }
-    if (n > 0) {
-        PIC_CK(b, cudaMemcpyAsync(b->d_blk_run, br.data(), sizeof(int32_t) * n, cudaMemcpyHostToDevice, b->stream));
-        PIC_CK(b, cudaMemcpyAsync(b->d_blk_i0, bi.data(), sizeof(int32_t) * n, cudaMemcpyHostToDevice, b->stream));
+    if (sent > 0) {
+        PIC_CK(b, cudaMemcpyAsync(b->layout, h.data(), sizeof(int32_t) * sent, cudaMemcpyHostToDevice, b->stream));
         PIC_CK(b, cudaStreamSynchronize(b->stream));
     }
-    b->nblk = n;
+    b->d_blk_run = b->layout;
+    b->d_blk_i0 = b->d_blk_run + nb;
+    b->d_grp_pair = b->d_blk_i0 + nb;
+    b->d_grp_at = b->d_grp_pair + ng;
+    b->grp_n = b->d_grp_at + ng;
+    b->grp_sum = b->grp_n + ng;
+    b->nblk = static_cast<int>(nb);
+    b->ngroups = static_cast<int>(ng);
     b->layout_dirty = false;
-    b->epoch++;  // the Yee grid, and possibly the sort's, changed shape
+    b->epoch++;  // the grids of the Yee kernel and the sort changed
     return PIC_OK;
 }
 
 void rad_flush(Batch* b, cudaStream_t st) {
     if (b->max_units == 0) return;
-    launch_rad_flush(b->d_runs, b->max_runs, b->rs_units[b->cur], b->rad_part, st);
+    launch_rad_flush(b->d_runs, b->max_runs, b->cur, b->rad_part, st);
     b->launches++;
 }
 void rad_flush(Batch* b) { rad_flush(b, b->stream); }

@@ -124,8 +124,7 @@ struct RunDev {
     int32_t* keystart[2];  // [Nx + 2]; keystart[Nx] = particles
     int32_t* blocksum[2];  // [Nx / 256 + 2]
     int32_t* blockstart[2];
-    int32_t* group_n[2];         // [groups of SPAN cells]: entries of the new unit table
-    int32_t* group_first[2][2];  // per table, [groups + 3]: first entry of the group or a later one; the last three: the end
+    int32_t* group_first[2][2];  // per table, [groups of SPAN cells + 3]: first entry of the group or a later one; the last three: the end
 };
 
 // Buffers of a run at a batch step of phase g: the step, or anything equal to it mod 6 (and >= 0).
@@ -271,13 +270,16 @@ struct SortParams {
     int tab, tab_new;      // which of a run's group_first belongs to each
     uint16_t* cnt;         // [max_units * SSTR] key counts per unit window
     int32_t* offs;         // [max_units * SSTR] destinations per unit window
-    const int32_t* rs_units;  // [4 * nruns]: entries per (run, species) pair, then the first of each pair
-    int32_t* rs_new;       // the same of the new table
+    // the groups of SPAN cells of the active runs, in the order of the table: by run, species and cell
+    const int32_t* grp_pair;  // [ngroups] 2 * run + species
+    const int32_t* grp_at;    // [ngroups] the group's place in its run
+    int32_t* grp_n;           // [ngroups] entries of the new table
+    int32_t* grp_sum;         // their sums over every 256 groups, then over every 65536
+    int ngroups;
     double* rad_part;
     int* status;
     int k, cur, max_units;
     int kb_max;            // key blocks of the largest run: ceil(max Nx / 256)
-    int g_max;             // groups of the largest run: ceil(max Nx / SPAN)
     int unit_p;            // particles per unit at most (UNIT_P_MIN..UNIT_P_MAX)
     int part_p;            // particles per part of a unit (a power of two, PART_MIN..unit_p)
     unsigned* phase;       // += k, mod 6
@@ -289,8 +291,8 @@ void launch_sort(const SortParams& S, cudaStream_t st, int* launches, bool pdl =
 // Unit table S.fresh of every active run from its current, already sorted particles.
 void launch_build_units(const SortParams& S, cudaStream_t st, int* launches);
 // Add each run's per-unit radiated energy into its tally[0]; zero them.
-// rs_units as in SortParams.
-void launch_rad_flush(const RunDev* runs, int nruns, const int32_t* rs_units, double* rad_part, cudaStream_t st);
+// tab: the table in use, as in SortParams.
+void launch_rad_flush(const RunDev* runs, int nruns, int tab, double* rad_part, cudaStream_t st);
 
 void launch_foil(DevSpecies e, DevSpecies ion, int c0, int ncell, int ppc, uint64_t seed, cudaStream_t st);
 void launch_iota(int32_t* id, int64_t n, cudaStream_t st);

@@ -177,3 +177,54 @@ def test_currents_stay_readable_when_a_large_run_ends(picrr, steps):
             assert c not in (5, 6, 7) or np.any(f)
     alone.close()
     beside.close()
+
+
+def test_few_runs_in_a_batch_of_many_slots(picrr):
+    """Three of 4000 slots, with released ones before and between them, of different lengths."""
+    cpl = 100.0
+    runs = [dict(length_lambda=l, foil_x0=0.3, foil_thickness=0.7 * l, ne=20.0, a0=80.0, polarization=picrr.CP, duration=3.0,
+                 steps=10**9, ppc=20, seed=7 + k) for k, l in enumerate((6.0, 23.0, 2.5))]
+    b = picrr.Batch(cpl, max_runs=4000, sort_interval=8)
+    ids = []
+    for k in range(9):
+        r = b.add_run(**runs[k // 3])
+        if k % 3 == 2:
+            ids.append(r)
+        else:
+            b.step(0)  # starts it
+            b.stop_run(r)
+            b.release_run(r)
+            b.add_run(**runs[k // 3])  # the slot's next run stays
+    b.step(45)
+    for r, kw in zip(ids, runs):
+        a = picrr.Batch(cpl, max_runs=1, sort_interval=8)
+        ra = a.add_run(**kw)
+        a.step(45)
+        (x, ex), (y, ey) = state(a, ra), state(b, r)
+        assert all(np.array_equal(p, q) for p, q in zip(x, y))
+        assert ey[3] == pytest.approx(ex[3], rel=1e-12, abs=1e-300)
+        a.close()
+    b.close()
+
+
+@pytest.mark.parametrize("cells", [200_003, 17_000_001])  # 782 and 66,408 groups of 512 cells, both species
+def test_long_boxes(picrr, cells):
+    """Hardly any charge: every particle flies straight on, each step exactly once, through sorts and new
+    tables over the whole box.  A step rounds the offset (2^-24) and the velocity (4 x 2^-24, times 0.95): 40
+    steps stay below 1.2e-5 cells."""
+    n, steps, dx = 60_000, 40, 2 * np.pi / 500.0
+    r = np.random.default_rng(cells)
+    g = picrr.Sim(cells / 500.0, 500.0, cfl=0.95, sort_interval=8, source_node=8)
+    want = []
+    for sp, (q, m) in enumerate(((-1.0, 1.0), (1.0, 1836.15267343))):
+        cell = np.sort(r.integers(100, cells - 100, n)).astype(np.int32)
+        off = r.random(n, dtype=np.float32)
+        p = [(3.0 * r.normal(size=n)).astype(np.float32) for _ in range(3)]
+        g.load_particles_f32(sp, cell, off, *p, 1e-25, q, m)
+        p = [v.astype(float) for v in p]
+        want.append(cell + off.astype(float) + steps * 0.95 * p[0] / np.sqrt(1 + p[0] ** 2 + p[1] ** 2 + p[2] ** 2))
+    assert g.step(steps) == steps
+    assert 2 * n // 512 < g.stats()["n_units"] <= 2 * (n // 512 + (cells + 511) // 512 + 1)
+    for sp in (0, 1):
+        assert np.max(np.abs(g.particles(sp)["x"] / dx - want[sp])) < 1.2e-5
+    g.close()
