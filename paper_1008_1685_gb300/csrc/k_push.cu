@@ -60,12 +60,16 @@ struct Window {
 
 __device__ __forceinline__ uint32_t win_addr(const Window& w) { return smem_u32(&w.lo[0][0]); }
 
+// Negative if old + t leaves the signed 32-bit range.  (Added as unsigned words, where that is defined.)
+__device__ __forceinline__ int win_wrapped(int old, int t) {
+    const unsigned o = static_cast<unsigned>(old), a = static_cast<unsigned>(t), now = o + a;
+    return static_cast<int>((o ^ now) & (a ^ now));
+}
 // Adds t to the window word at shared address `addr`; negative if the word wrapped.
 __device__ __forceinline__ int win_add(uint32_t addr, int t) {
     int old;
     asm volatile("atom.shared.add.s32 %0, [%1], %2;" : "=r"(old) : "r"(addr), "r"(t) : "memory");
-    const int now = old + t;
-    return (old ^ now) & (t ^ now);
+    return win_wrapped(old, t);
 }
 // The wrap's entry in hi.
 __device__ __forceinline__ void win_carry(uint32_t addr, int t) {
