@@ -50,13 +50,15 @@ __device__ __forceinline__ int key_of(int c) { return c < 0 ? -1 - c : c; }
 
 __device__ __forceinline__ int groups_of(int Nx) { return (Nx + SPAN - 1) / SPAN; }
 
-// radiated energy of run r: sum of its electron units, fixed order (SORT_T threads)
-__device__ __forceinline__ void rad_flush_block(const RunDev* runs, int r, int tab, double* part, double* sred) {
-    const RunDev& R = runs[r];
-    if (!R.active) return;
+// an active run's electron units in the table in use: the first one and their number
+__device__ __forceinline__ int2 electron_units(const RunDev& R, int tab) {
     const int32_t* gf = R.group_first[0][tab];
-    const int b = gf[0], n = gf[groups_of(R.Nx)] - b;  // electron units
-    const int t = threadIdx.x;
+    const int b = gf[0];
+    return make_int2(b, gf[groups_of(R.Nx)] - b);
+}
+// its radiated energy: sum over these units, fixed order (SORT_T threads)
+__device__ __forceinline__ void rad_flush_block(const RunDev& R, int2 units, double* part, double* sred) {
+    const int b = units.x, n = units.y, t = threadIdx.x;
     double a[4] = {0.0, 0.0, 0.0, 0.0};
     for (int i = t; i < n; i += 4 * SORT_T) {
 #pragma unroll
@@ -80,7 +82,8 @@ __device__ __forceinline__ void rad_flush_block(const RunDev* runs, int r, int t
 
 __global__ void __launch_bounds__(SORT_T) k_rad_flush(const RunDev* runs, int tab, double* part) {
     __shared__ double sred[SORT_T / 32];
-    rad_flush_block(runs, blockIdx.x, tab, part, sred);
+    const RunDev& R = runs[blockIdx.x];
+    if (R.active) rad_flush_block(R, electron_units(R, tab), part, sred);
 }
 
 // Sums of grp_n, counted up by count_entries: over each 256 groups, then over each 65536.
@@ -100,9 +103,12 @@ __global__ void __launch_bounds__(SORT_T) k_sort_count(const SortParams S) {
     pdl_release<PDL>();
     const int u = static_cast<int>(blockIdx.x) - S.nruns;
     if (u < 0) {  // block-uniform
+        const RunDev& R = S.runs[blockIdx.x];
+        const bool active = R.active;
+        const int2 units = active ? electron_units(R, S.tab) : make_int2(0, 0);
         pdl_wait<PDL>();
         clear_sums(S, blockIdx.x, S.nruns);
-        rad_flush_block(S.runs, blockIdx.x, S.tab, S.rad_part, sred);
+        if (active) rad_flush_block(R, units, S.rad_part, sred);
         return;
     }
     const int run = S.units.run[u];
@@ -290,9 +296,31 @@ struct FillSmem {
 // The table's blocks of a launch: one per group, and one if there is none (the phase advances in any case).
 __host__ __device__ __forceinline__ int fill_blocks(const SortParams& S) { return S.ngroups > 0 ? S.ngroups : 1; }
 
-__device__ __forceinline__ void fill_block(const SortParams& S, int j, FillSmem& F) {
-    const int tid = threadIdx.x;
+// A group as fill_block needs it: what the launches before do not write, so that it is read before they end.
+struct FillGroup {
+    int run, s, g, Nx;
+    const int32_t* ks;  // starts of its cells
+    int32_t* gf;        // the run's group_first of the new table
+};
+__device__ __forceinline__ FillGroup fill_group(const SortParams& S, int j) {
+    FillGroup G{};
+    if (j >= S.ngroups) return G;
+    const int p = S.grp_pair[j];
+    G.g = S.grp_at[j];
+    G.run = p >> 1;
+    G.s = p & 1;
+    const RunDev& R = S.runs[G.run];
+    G.Nx = R.Nx;
+    G.ks = R.keystart[G.s] + G.g * SPAN;
+    G.gf = R.group_first[G.s][S.tab_new];
+    return G;
+}
+
+__device__ __forceinline__ void fill_block(const SortParams& S, int j, const FillGroup& H, FillSmem& F) {
+    const int tid = threadIdx.x, run = H.run, s = H.s, g = H.g, C0 = g * SPAN, cells = min(SPAN, H.Nx - C0);
     if (tid < 2) F.red[tid] = 0;
+    if (j < S.ngroups)
+        for (int i = tid; i <= cells; i += SORT_T) F.ks[i] = H.ks[i];
     __syncthreads();
     // entries before this group, and in all
     const int n2 = sums2(S);
@@ -322,11 +350,6 @@ __device__ __forceinline__ void fill_block(const SortParams& S, int j, FillSmem&
          i += static_cast<int64_t>(fill_blocks(S)) * SORT_T)
         S.fresh.run[i] = -1;
     if (j >= S.ngroups) return;
-    const int run = S.grp_pair[j] >> 1, s = S.grp_pair[j] & 1, g = S.grp_at[j];
-    const RunDev& R = S.runs[run];
-    const int C0 = g * SPAN, cells = min(SPAN, R.Nx - C0);
-    for (int i = tid; i <= cells; i += SORT_T) F.ks[i] = R.keystart[s][C0 + i];
-    __syncthreads();
     const int base = F.red[0];
     if (tid < 32) {
         int a = 0, b = 0;
@@ -341,8 +364,8 @@ __device__ __forceinline__ void fill_block(const SortParams& S, int j, FillSmem&
         if (tid == GROUP - 1) F.first[GROUP] = x;
     }
     __syncthreads();
-    const int n = F.first[GROUP], G = groups_of(R.Nx);
-    int32_t* gf = R.group_first[s][S.tab_new];
+    const int n = F.first[GROUP], G = groups_of(H.Nx);
+    int32_t* gf = H.gf;
     if (tid == 0) gf[g] = base;
     if (g == G - 1 && tid < 3) gf[G + tid] = base + n;
     for (int v = tid; v < n; v += SORT_T) {
@@ -406,8 +429,9 @@ __global__ void __launch_bounds__(SORT_T) k_sort_scatter(const SortParams S) {
     pdl_release<PDL>();
     const int u = static_cast<int>(blockIdx.x) - fill_blocks(S);
     if (u < 0) {  // block-uniform
+        const FillGroup G = fill_group(S, blockIdx.x);
         pdl_wait<PDL>();
-        fill_block(S, blockIdx.x, reinterpret_cast<FillSmem&>(row));
+        fill_block(S, blockIdx.x, G, reinterpret_cast<FillSmem&>(row));
         return;
     }
     const int of_run = S.units.run[u];
@@ -639,7 +663,7 @@ __global__ void __launch_bounds__(SORT_T) k_group_entries(const SortParams S) {
 
 __global__ void __launch_bounds__(SORT_T) k_fill(const SortParams S) {
     __shared__ FillSmem F;
-    fill_block(S, blockIdx.x, F);
+    fill_block(S, blockIdx.x, fill_group(S, blockIdx.x), F);
 }
 
 }  // namespace
