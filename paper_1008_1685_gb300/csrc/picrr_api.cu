@@ -1143,14 +1143,20 @@ FieldParams field_params(const Batch* b, int k, int j) {
 }
 
 // With 2 particles per thread a push that follows another one also does the Yee update of the step before
-// (launch_push); the last push's update is a launch of its own.  That pays while the units leave the GPU
-// half empty, where a step is a chain of latencies (small run 35 -> 30 us per step); with more units each
-// block's update of its own window costs more than the launch it saves (thin plasma, 2700 units, 142 -> 158
-// us; a 48-run scan, 1600 units, 125 -> 134 us).  The 4-per-thread kernel (dense foils, for which the Yee
-// update is a hundredth of a step) leaves every update to the Yee kernel.
+// (launch_push); the last push's update is a launch of its own.  That pays while a step is a chain of latencies
+// (one run of 15,000 cells 13.7 -> 9.9 us per step), which asks for two things:
+// - few whole units: with many, each block's update of its own window costs more than the launch it saves
+//   (thin plasma, 2700 units, 142 -> 158 us; a 48-run scan, 1600 units, 125 -> 134 us);
+// - Yee blocks that find a place on the GPU all at once, 5 on each of 152 SMs: they come before the push's and take
+//   a whole place each, where the Yee kernel runs many on an SM.  us per step without and with: a foil of 20,000
+//   particles in a box of 60,000 cells (235 blocks) 13.8 and 10.6, of 180,000 (704) 14.6 and 11.7, of 200,000 (782)
+//   14.6 and 15.1, of 10^6 (3907) 29.2 and 37.4; plasma all over a box of 450,000 cells (1758) 48.2 and 54.3.
+// The 4-per-thread kernel (dense foils, for which the Yee update is a hundredth of a step) leaves every update to
+// the Yee kernel.  (The layout, and with it nblk, is uploaded.)
+constexpr int FUSE_BLOCKS = 5 * 152;
 bool fuses(const Batch* b) {
-    if (b->slot_w != 2) return false;
-    int64_t units = 0;  // about: full units, and tile groups
+    if (b->slot_w != 2 || b->nblk > FUSE_BLOCKS) return false;
+    int64_t units = 0;  // whole ones
     for (const auto& r : b->runs) {
         if (!r.used || !r.active) continue;
         for (int s = 0; s < 2; ++s)

@@ -228,3 +228,22 @@ def test_long_boxes(picrr, cells):
     for sp in (0, 1):
         assert np.max(np.abs(g.particles(sp)["x"] / dx - want[sp])) < 1.2e-5
     g.close()
+
+
+def test_steps_of_long_boxes_are_not_fused(picrr):
+    """Fused, an interval of 8 steps is 8 pushes, one Yee launch and 3 for the sort, else 8 Yee launches; the
+    bits are the same in boxes that differ by a cell at the far end."""
+    res = []
+    for cells, launches in ((194_559, 12), (194_560, 19)):  # 760 and 761 Yee blocks
+        g = picrr.Sim(cells / 500.0, 500.0, cfl=0.95, sort_interval=8, source_node=8, seed=3)
+        g.load_foil(0.2, 1.0, 20.0, 1, 1.0, 20)
+        g.inject_laser(80.0, picrr.CP, picrr.ENV_SIN2, 3.0)
+        g.step(8)
+        n = g.stats()["kernel_launches"]
+        g.step(160)
+        assert g.stats()["kernel_launches"] - n == 20 * launches
+        q = g.particles(0)
+        res.append([g.field(c)[:150_000] for c in range(8)] + [q[k] for k in ("x", "px", "py", "pz")])
+        g.close()
+    for a, b in zip(*res):
+        assert np.any(a) and np.array_equal(a, b)
