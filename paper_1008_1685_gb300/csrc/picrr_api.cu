@@ -1714,8 +1714,9 @@ pic_status run_read_fields(Batch* b, int id, int comp, int64_t cap, double* out,
     launch_widen(f, fix, scale, n, reinterpret_cast<double*>(tmp), b->stream);
     b->launches++;
     touch_pages(out, static_cast<size_t>(n) * 8);
-    PIC_CK(b, cudaMemcpyAsync(out, tmp, static_cast<size_t>(n) * 8, cudaMemcpyDeviceToHost, b->stream));
-    PIC_CK(b, cudaMemsetAsync(tmp, 0, static_cast<size_t>(n) * 8, b->stream));
+    const cudaError_t copied = cudaMemcpyAsync(out, tmp, static_cast<size_t>(n) * 8, cudaMemcpyDeviceToHost, b->stream);
+    PIC_CK(b, cudaMemsetAsync(tmp, 0, static_cast<size_t>(n) * 8, b->stream));  // also when the copy could not be queued
+    PIC_CK(b, copied);
     PIC_CK(b, cudaStreamSynchronize(b->stream));
     PIC_CK(b, cudaGetLastError());
     return PIC_OK;
