@@ -1,5 +1,5 @@
-// The Yee update of one step as a kernel of its own (yee.cuh): after a push that
-// nothing follows, and after every push with 4 particles per thread.  (A version
+// The Yee update of one step as a kernel of its own (yee.cuh): after every push that is
+// not followed by one fused with it.  (A version
 // without shared memory and barriers, each thread recomputing the half-step B and
 // new E it shares with its neighbours from global loads, ran at half the speed.)
 #include "yee.cuh"

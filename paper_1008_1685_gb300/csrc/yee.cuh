@@ -51,7 +51,7 @@ __device__ __forceinline__ float yee_mur(float old_in, float new_in, float old_w
 }
 
 // The update of FIELD_NODES nodes of one run (block `blk` of the block table) by T
-// threads, FIELD_NODES / T nodes each: old and new fields live in separate buffers and
+// threads, FIELD_NODES / T nodes each (one, by some of them, where that is below one): old and new fields live in separate buffers and
 // the guard values are recomputed from the neighbours' old data, so that one launch does
 // the whole step.  It also zeroes the current accumulators of the next step (two sets), or of the one after it (three) and
 // adds the exact discrete Poynting flux through the two accounting planes.
@@ -64,7 +64,8 @@ struct FieldSmem {
 
 template <int T, bool PDL>
 __device__ __forceinline__ void field_block(const FieldParams& P, unsigned phase, int blk, FieldSmem& S) {
-    constexpr int N = FIELD_NODES, K = N / T;
+    constexpr int N = FIELD_NODES, K = (N + T - 1) / T;
+    constexpr bool EVEN = N % T == 0;  // else not every thread has a node in each of the K rounds
     const int tid = threadIdx.x;
     const int run = P.blk_run[blk];
     const RunDev& R = P.runs[run];
@@ -89,7 +90,7 @@ __device__ __forceinline__ void field_block(const FieldParams& P, unsigned phase
 #pragma unroll
     for (int k = 0; k <= K; ++k) {
         const int q = tid + k * T;
-        if (k == K && q >= N + 4) break;  // the 4 guard entries past the tile
+        if ((k == K || !EVEN) && q >= N + 4) break;  // the 4 guard entries past the tile
         const int i = i0 - 2 + q + PADF;  // padded index, >= PADF - 2 >= 0
         const bool in = i < glen;         // the last block reaches past the array end
         S.ey[q] = in ? Fo[1][i] : 0.f;
@@ -105,8 +106,8 @@ __device__ __forceinline__ void field_block(const FieldParams& P, unsigned phase
     }
 #pragma unroll
     for (int k = 0; k < K; ++k) {
-        const int pi = i0 + tid + k * T + PADF;
-        const bool own = i0 + tid + k * T < Nx;
+        const int q = tid + k * T, pi = i0 + q + PADF;
+        const bool own = (EVEN || q < N) && i0 + q < Nx;
         jx[k] = own ? Jacc[0][pi] : 0ull;
         ex[k] = own ? Fo[0][pi] : 0.f;
     }
@@ -116,7 +117,7 @@ __device__ __forceinline__ void field_block(const FieldParams& P, unsigned phase
 #pragma unroll
     for (int k = 0; k <= K; ++k) {
         const int q = tid + k * T;
-        if (k == K && q >= N + 3) break;
+        if ((k == K || !EVEN) && q >= N + 3) break;
         float by = S.by[q], bz = S.bz[q];
         yee_b(by, bz, S.ey[q], S.ey[q + 1], S.ez[q], S.ez[q + 1], hc, i0 - 2 + q == is - 1, inc[0], inc[1]);
         S.by[q] = by;
@@ -128,7 +129,7 @@ __device__ __forceinline__ void field_block(const FieldParams& P, unsigned phase
 #pragma unroll
     for (int k = 0; k <= K; ++k) {
         const int q = tid + k * T;
-        if (k == K && q >= N + 2) break;
+        if ((k == K || !EVEN) && q >= N + 2) break;
         const int i = i0 - 1 + q;
         // node i: old E at sE[q+1], half nodes i-1, i at sB[q], sB[q+1]
         float ey = S.ey[q + 1], ez = S.ez[q + 1];
@@ -161,6 +162,7 @@ __device__ __forceinline__ void field_block(const FieldParams& P, unsigned phase
 #pragma unroll
     for (int k = 0; k < K; ++k) {
         const int q = tid + k * T;  // node i: nE[q+1], sE[q+2]; half node i: sB[q+2]
+        if (!EVEN && q >= N) break;
         const int i = i0 + q;
         const int pi = i + PADF;
         if (i <= Nx) {

@@ -247,3 +247,40 @@ def test_steps_of_long_boxes_are_not_fused(picrr):
         g.close()
     for a, b in zip(*res):
         assert np.any(a) and np.array_equal(a, b)
+
+
+@pytest.mark.parametrize("npt", [1, 4])  # nodes per thread of the Yee kernel; 2 in the library
+def test_other_yee_blocks_give_the_same_bits(picrr, tmp_path, npt):
+    """The build option changes which block updates a node, in the kernel of its own and inside the push."""
+    code = """
+import sys
+import numpy as np
+from paper_1008_1685_gb300 import binding, build
+npt, out = sys.argv[1:]
+if npt != "2":
+    build.LIB, build.BUILD = out + ".so", out + "_build"
+    binding._LIB_PATH = build.build(force=True, extra=["-DPICRR_FIELD_NPT=" + npt])
+res = []
+for cells, slots in ((500, 2), (1153, 2), (1153, 4)):
+    g = binding.Sim(cells / 100.0, 100.0, sort_interval=8, seed=4)
+    g.load_foil(0.3, 3.0, 20.0, 1, 1.0, 20)
+    g.inject_laser(80.0, binding.CP, binding.ENV_SIN2, 3.0)
+    g.set_shapes(4096, 8, slots)
+    g.step(150)
+    res += [g.field(c) for c in range(8)] + [g.energy()[[0, 1, 2, 4, 5]]]
+    g.close()
+np.savez(out, *res)
+"""
+    import os
+    import subprocess
+    import sys
+
+    root = os.path.dirname(os.path.dirname(os.path.abspath(picrr.__file__)))
+    got = []
+    for v in ("2", str(npt)):
+        out = str(tmp_path / ("npt" + v))
+        subprocess.run([sys.executable, "-c", code, v, out], cwd=root, check=True)
+        with np.load(out + ".npz") as z:
+            got.append([z[k] for k in z.files])
+    for a, b in zip(*got):
+        assert np.any(a) and np.array_equal(a, b)
