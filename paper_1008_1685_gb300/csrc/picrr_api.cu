@@ -1146,7 +1146,9 @@ FieldParams field_params(const Batch* b, int k, int j) {
 // (launch_push); the last push's update is a launch of its own.  That pays while a step is a chain of latencies
 // (one run of 15,000 cells 13.7 -> 9.9 us per step), which asks for two things:
 // - few whole units: with many, each block's update of its own window costs more than the launch it saves
-//   (thin plasma, 2700 units, 142 -> 158 us; a 48-run scan, 1600 units, 125 -> 134 us);
+//   (thin plasma, 2700 units, 142 -> 158 us; a 48-run scan, 1600 units, 125 -> 134 us).  Smaller units than 4096
+//   count as such: few enough to be fused, they are about as many entries of the table as parts would be
+//   (480,000 to 1.8 M particles in units of 1024 or 2048: 21.6 to 41.7 us fused, 24.6 to 44.9 not);
 // - Yee blocks that find a place on the GPU all at once, 5 on each of 152 SMs: they come before the push's and take
 //   a whole place each, where the Yee kernel runs many on an SM.  us per step without and with: a foil of 20,000
 //   particles in a box of 60,000 cells (235 blocks) 13.8 and 10.6, of 180,000 (704) 14.6 and 11.7, of 200,000 (782)
@@ -1160,7 +1162,7 @@ bool fuses(const Batch* b) {
     for (const auto& r : b->runs) {
         if (!r.used || !r.active) continue;
         for (int s = 0; s < 2; ++s)
-            if (r.sp[s].loaded) units += r.sp[s].n / b->unit_p;
+            if (r.sp[s].loaded) units += r.sp[s].n / std::max(b->unit_p, UNIT_P);
     }
     return units <= FUSE_UNITS;
 }

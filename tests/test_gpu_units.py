@@ -158,16 +158,15 @@ def test_window_words_wrap(picrr, n, cells, spread, sign, planar, slots):
 
 @pytest.mark.parametrize("steps", [48, 45])  # (the pulse is in the foil) the last step ends a sort interval, or lies inside one
 def test_currents_stay_readable_when_a_large_run_ends(picrr, steps):
-    """A run of 585 units of 1024 ends on the last step of a call, the small run beside it goes on: from
+    """A run of 488 units ends on the last step of a call, the small run beside it goes on: from
     then on its steps take another form, but its last current is still that of the run alone."""
     cpl, small = 100.0, dict(length_lambda=6.0, foil_x0=0.3, foil_thickness=4.0, ne=20.0, a0=80.0, polarization=picrr.CP,
                              duration=3.0, steps=10**9, ppc=30, seed=5)
     alone, beside = (picrr.Batch(cpl, max_runs=m, sort_interval=8) for m in (1, 2))
     beside.add_run(length_lambda=20.0, foil_x0=1.0, foil_thickness=10.0, ne=1.0, a0=1.0, polarization=0, duration=3.0,
-                   steps=steps, ppc=300, seed=6)
+                   steps=steps, ppc=1000, seed=6)
     ra, rb = alone.add_run(**small), beside.add_run(**small)
     for b in (alone, beside):
-        b.set_shapes(1024, 8, 2)
         assert b.step(steps) == steps
     for n in (0, 1, 9):
         assert alone.step(n) == n and beside.step(n) == n
@@ -284,3 +283,15 @@ np.savez(out, *res)
             got.append([z[k] for k in z.files])
     for a, b in zip(*got):
         assert np.any(a) and np.array_equal(a, b)
+
+
+@pytest.mark.parametrize("unit", [1024, 4096])
+def test_small_units_are_fused_like_the_default_s(picrr, unit):
+    g = picrr.Sim(20.0, 500.0, cfl=0.95, sort_interval=8, source_node=8, seed=3)
+    g.load_foil(0.2, 1.0, 20.0, 1, 1.0, 600)  # 600,000 particles
+    g.set_shapes(unit, 8, 2)
+    g.step(8)
+    n = g.stats()["kernel_launches"]
+    g.step(80)
+    assert g.stats()["kernel_launches"] - n == 10 * 12
+    g.close()
