@@ -26,7 +26,7 @@
 //     hold its state, and each evaluates one of the sines and cosines of a stage (the
 //     pulse needs four).
 // 4096 electrons x 2000 RK4 steps: 47.1 -> 18.5 ms; 20,000 x 1000 leapfrog steps:
-// 15.6 -> 4.7 ms.
+// 15.6 -> 4.5 ms.
 #include <new>
 #include <string>
 #include <vector>

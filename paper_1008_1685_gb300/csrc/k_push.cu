@@ -86,14 +86,9 @@ __device__ __forceinline__ int rec_at(int key, int q) { return key + (q < 3 ? q 
 // values are collected as bits and looked at once: five instructions a value.
 // Values that are zero unless a particle crossed a cell boundary (node key + 2,
 // half node key + 1) are skipped when all are, and Jz when it is zero (linear
-// polarization: 217 -> 203 us in the late phase of 96 small foils, half of them
-// so; adds of zeros to the few words that a warp's lanes share are not free).
-// A second integer reduction for a warp whose lanes hold two anchors was no
-// gain (a cold dense foil 411 -> 422, hot 540 -> 541, small foils 101 -> 109 us
-// a push).  (Carries predicated after every
-// add, with lo unsigned, came out as two divergence points a value; two
-// additions without return, t to lo and t >> 12 to a coarse word that resolves
-// the wraps, took the dense run of hot particles 5 % longer.)
+// polarization): adds of zeros to the few words that a warp's lanes share are
+// not free (late in the runs of 96 small foils, half of them linear, 217 us a
+// push with them, 203 without).
 __device__ __forceinline__ void lane_add(int key, const float (&v)[8], uint32_t w) {
     const uint32_t a = w + 4u * key;
     constexpr int at[8] = {4 * WMAX, 4 * (WMAX + 1), 4 * (WMAX + 2), 8 * WMAX, 4 * (2 * WMAX + 1), 4 * (2 * WMAX + 2), 0, 4};
@@ -126,8 +121,8 @@ __device__ __forceinline__ void lane_add(int key, const float (&v)[8], uint32_t 
 // One stencil record per lane (key < 0: none).  When every lane holds the
 // same anchor (dense plasma), the records are summed exactly in 32-bit fixed
 // point (|value| < 2^26 per lane, so the warp sum fits) by one integer warp
-// reduction per value and lanes 0..7 add the eight sums (the large run's push
-// 0.463 -> 0.450 ms against eight adds by lane 0); otherwise every lane adds
+// reduction per value and lanes 0..7 add the eight sums (3 % of the large run's
+// push against eight adds by lane 0); otherwise every lane adds
 // its own record.  (A reduction over lanes grouped by anchor runs once per
 // distinct anchor, which costs more than the lanes' own atomics as soon as
 // the warp holds two.)
@@ -150,7 +145,7 @@ __device__ __forceinline__ void warp_add(int key, const float (&v)[8], uint32_t 
         }
     } else {
         // (summing the records of neighbouring lanes with one anchor first saves
-        // atomics but not time: scan 116 us either way)
+        // atomics but not time)
         if (key >= 0) lane_add(key, v, w);
     }
 }
@@ -205,7 +200,7 @@ struct Slot<2> {
 // fields are read with plain loads into a layout made for the gather: per node
 // i (Ey, Ey[i+1] - Ey, Ez, Ez[i+1] - Ez) and per half node (Ex, dEx, By, dBy)
 // and (Bz, dBz), so that a particle's gather is three loads and five FMAs
-// (the large run's push 0.451 -> 0.441 ms).  With 2 per thread (thin plasma,
+// (2 % of the large run's push).  With 2 per thread (thin plasma,
 // few particles per cell) the components are copied as they are by bulk TMA,
 // and the smaller footprint keeps five CTAs per SM.
 template <int W>
@@ -410,10 +405,8 @@ __global__ void __launch_bounds__(PUSH_T, Slot<W>::MIN_BLOCKS) k_push_deposit(co
     // Bound by the instructions issued (225 to 300 a particle).  So the body has no branch on a
     // lane's own state but for the adds: every lane computes its slot's particles (lanes behind
     // the last slot that one's), and those that are not the unit's, frozen or outside the window
-    // count for nothing.  With the adds above, and before -> after, us a push: a dense foil of
-    // 64 M hot particles 623 -> 540, of cold ones 437 -> 411, 8 M thinly spread ones 107 -> 94,
-    // a batch of 48 small foils 116 -> 101 (with parts of 4096, PART_EVEN, which gave 5 of that),
-    // of 96 late in their runs 215 -> 203.
+    // count for nothing.  us a push with branches -> without: a dense foil of 64 M hot particles
+    // 623 -> 540, of cold ones 437 -> 411, 8 M thinly spread ones 107 -> 94.
     for (int r = 0; r < rounds; ++r) {
         const int slot = r * PUSH_T + tid;
         if ((slot & ~31) >= nslots) break;  // the warp has no slot left
@@ -426,7 +419,7 @@ __global__ void __launch_bounds__(PUSH_T, Slot<W>::MIN_BLOCKS) k_push_deposit(co
         F z4 = __ldcs(reinterpret_cast<const F*>(sp.pz + b4));
         // the next round's slots into L2 while this round computes, so that its loads
         // wait on L2 rather than HBM: one bulk (TMA) prefetch per array for the whole
-        // CTA, with an evict-first policy (the large run's push 0.483 -> 0.463 ms)
+        // CTA, with an evict-first policy (4 % of the large run's push)
         if (tid == 0 && (r + 1) * PUSH_T < nslots) {
             const int n0 = base + W * (r + 1) * PUSH_T;                      // first particle of the next round
             const int n1 = base + W * min((r + 2) * PUSH_T, nslots);         // one past its last
@@ -535,8 +528,9 @@ __global__ void __launch_bounds__(PUSH_T, Slot<W>::MIN_BLOCKS) k_push_deposit(co
                     const float qN = 1.f + px * px + py * py + pz * pz;
                     ign = rsqrt_ge1(qN);
                     const float gL = qL * rsqrt_ge1(qL), gN = qN * ign;
-                    // rad_h + rad_l -= de without the rounding (Knuth): the tally must not depend on the
-                    // units' size.  (One addition in double per round: thin plasma +3 %, the scan +4 %.)
+                    // rad_h + rad_l -= de, compensated (Knuth): only rad_l, about 2^-24 of the sum, is rounded at
+                    // each particle, so that the units' size changes the tally by 1e-12 at most.  (One addition
+                    // in double per round: thin plasma +3 %, a batch of small foils +4 %.)
                     const float dg = div_ge1(kx * (lx + px) + ky * (ly + py) + kz * (lz + pz), gL + gN);
                     const float de = a ? dg : 0.f;
                     const float t = __fsub_rn(rad_h, de), z = __fsub_rn(t, rad_h);
@@ -595,8 +589,8 @@ __global__ void __launch_bounds__(PUSH_T, Slot<W>::MIN_BLOCKS) k_push_deposit(co
             // merge the particle's record into this thread's running record; when
             // its anchor changes, the lane adds the finished record by itself: a warp
             // vote and a warp-wide sum at every change cost more, with 4 particles
-            // per thread too (hot particles on a dense foil, whose anchors change
-            // mid-round: 0.717 -> 0.633 ms)
+            // per thread too (13 % on a dense foil of hot particles, whose anchors
+            // change mid-round)
             const float jxa = a ? jxf : 0.f;
             if (j == 0) {
                 rk = a ? ka : -1;
@@ -631,9 +625,9 @@ __global__ void __launch_bounds__(PUSH_T, Slot<W>::MIN_BLOCKS) k_push_deposit(co
         warp_add(rk, rv, wJ, !thin);
         // with 4 per thread (dense foils), a warp whose particles all stayed in
         // their cells leaves its cell slots as they are: a tenth of the written
-        // bytes for most warps of a dense foil (the large run's push 0.440 ->
-        // 0.425 ms); with 2 per thread (thin, hot plasma, where particles cross
-        // cells every step) the vote cost more than it saved
+        // bytes for most warps of a dense foil (3 % of the large run's push); with
+        // 2 per thread (thin, hot plasma, where particles cross cells every step)
+        // the vote cost more than it saved
         bool warp_moved = true;
         if constexpr (W == 4) {
             bool moved = false;

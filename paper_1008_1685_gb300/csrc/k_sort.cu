@@ -438,7 +438,7 @@ __device__ __forceinline__ void fill_block(const SortParams& S, int j, const Fil
 // its rank among the lanes with the same cell.  Equal cells therefore keep
 // index order, with two block barriers per unit.  (Ranking in pass 1 with the result kept
 // in registers, so that nothing in pass 2 waits, and more or fewer blocks an SM and rows in
-// flight, came to 170 to 217 us per sort of thin plasma against 172.)
+// flight, were no faster.)
 constexpr int SC_W = SORT_T / 32;
 constexpr int SC_U = 4;  // slice rows of 32 particles in flight per pass step
 

@@ -29,16 +29,20 @@
 
 #include <cuda_runtime.h>
 
-#include "picrr.h"
 #include <stdint.h>
+#include <string>
+
+#include <unistd.h>
+
+#include "picrr.h"
 
 namespace picrr {
 
 constexpr int PADF = 40;          // guard elements left of index 0 of every grid array
 constexpr int TILE = 64;          // cells per tile: a dense tile is split into units of at most unit_p particles
 // Consecutive tiles that form one unit when they hold <= unit_p particles (else each aligned half
-// group that does; else single tiles).  Groups of 8 instead of 4 took thinly spread plasma's push
-// from 0.651 to 0.595 ms (fewer, longer units) and the 256-run scan's late phase from 0.569 to 0.551.
+// group that does; else single tiles).  Groups of 8 instead of 4 took 9 % off the push of thinly
+// spread plasma (fewer, longer units) and 3 % off the 256-run scan's late phase.
 constexpr int GROUP = 8;
 constexpr int SPAN = GROUP * TILE;  // cell span bound of a unit
 constexpr int UNIT_P = 4096;      // default particles per unit at most (unit_p, a run-time shape of a batch)
@@ -53,17 +57,15 @@ constexpr int PUSH_T = 256;       // threads of the push kernel
 // When the units (of at most unit_p particles) would not fill the GPU, they are cut into parts, each a unit
 // table entry of its own: about PARTS of them for all particles, none below PART_MIN (one round of the push).
 // One CTA per unit took 27 us for the 12 units of a small run, eight rounds one after the other; with parts
-// 12 us.
-// 1216 (8 for each of 152 SMs; parts are a power of two, so that whole units can be put together from them)
-// against 760 and 2280: the paper-scale run 23.0 us per step with 1216 (799 units), 27.5 (410) and 26.8 (1581)
-// otherwise; the small run 11.3 with each.
+// 12 us.  Parts are a power of two, so that whole units can be put together from them.  1216 (8 for each of 152
+// SMs) against 760 and 2280: the paper-scale run 23.0 us per step (799 parts), 27.5 (410) and 26.8 (1581).
 constexpr int PARTS = 1216;
 constexpr int PART_MIN = 512;
 // With 2 particles per thread (760 CTAs at a time), units of more than 4096 are cut down to that also while
 // they fill the GPU a few times only, so that the last CTAs end together: up to 5472 parts (7.2 rounds of CTAs).
-// us per push, units of 8192: 48 small foils (9.6 M particles) 109.5 -> 104.0, 96 of them 217 -> 210; of 16384:
-// dense foils of 6, 10 and 20 M 90.4 -> 86.9, 137 -> 121, 238 -> 228, of 32 M (parts of 8192) 349 -> 348.  Parts
-// of 2048 took 103 instead of 93 in thin plasma.  With 4 per thread a dense foil of 10 M went from 99.6 to 103.
+// us per push without and with: 48 small foils (9.6 M particles) in units of 8192 109.5 and 104.0; dense foils of
+// 10 and 20 M in units of 16384 137 and 121, 238 and 228, of 32 M (too many for it) 349 and 348.  With 4 per
+// thread a dense foil of 10 M took 103 instead of 99.6, and parts of 2048 thin plasma 103 instead of 93.
 constexpr int PART_EVEN = 4096, PARTS_EVEN = 5472;
 constexpr int FUSE_UNITS = 456;  // units up to which a push also updates its fields (picrr_api.cu, fuses)
 constexpr int WMAX = SPAN + 2 * KMAX + 16;  // window length bound in the push kernel (>= SPAN + 2 KMAX + 9)
@@ -296,11 +298,7 @@ void launch_rad_flush(const RunDev* runs, int nruns, int tab, double* rad_part, 
 
 void launch_foil(DevSpecies e, DevSpecies ion, int c0, int ncell, int ppc, uint64_t seed, cudaStream_t st);
 void launch_iota(int32_t* id, int64_t n, cudaStream_t st);
-}  // namespace picrr
-#include <string>
 
-#include <unistd.h>
-namespace picrr {
 // Writes to every page of a caller's array that a copy is about to fill: the copy engine reaches pages that the
 // host has not touched yet through its page faults (five fresh arrays of 3.2 MB: 12.5 ms; touched first, 1.0 ms,
 // most of it the kernel's zeroing; already resident 0.2 ms).
